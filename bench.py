@@ -101,7 +101,7 @@ def peaks():
 # sources that compile into the step kernel (host code, the adjoint and the
 # allocation-free wall force are left out)
 STEP_SOURCES = ("lbm_device.cuh", "lbm_kernels.cuh", "lbm_staged.cuh", "lbm_internal.h",
-                "inst_f64.cu", "inst_f32.cu", "inst_f16.cu", "inst_bf16.cu")
+                *(f"inst_{s}_{q}.cu" for s in ("f64", "f32", "f16", "bf16") for q in ("d2q9", "d3q19")))
 
 
 def source_hash():

@@ -64,7 +64,7 @@ def build(force: bool = False, verbose: bool = False, extra=()) -> str:
     if force:
         for f in os.listdir(OBJ):
             os.remove(os.path.join(OBJ, f))
-    with cf.ThreadPoolExecutor(max_workers=min(8, len(srcs))) as ex:
+    with cf.ThreadPoolExecutor(max_workers=min(os.cpu_count() or 8, len(srcs))) as ex:
         objs = list(ex.map(lambda s: _compile(nvcc, s, list(extra)), srcs))
     if force or _stale(LIB, objs):
         tmp = LIB + f".{os.getpid()}.tmp"

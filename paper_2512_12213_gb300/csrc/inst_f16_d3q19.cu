@@ -1,0 +1,10 @@
+// inst_f16_d3q19.cu -- kernels and launchers of D3Q19 with the StoreF16 population format
+#include "lbm_kernels.cuh"
+
+namespace lbm {
+const Dispatch& dispatch_f16_d3q19()
+{
+    static const Dispatch d = make_dispatch<19, StoreF16>();
+    return d;
+}
+}  // namespace lbm

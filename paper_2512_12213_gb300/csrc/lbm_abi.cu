@@ -646,11 +646,12 @@ lbm_status lbm_create(const lbm_config* cfg, const uint8_t* host_wall_id, void* 
     for (int k = 0; k < 6; ++k) x.geo.face_wall[k] = cfg->face_wall[k];
     x.elem = elem_of(cfg->storage);
     x.relem = cfg->storage == LBM_STORE_F64 ? 8 : 4;
+    const bool d2 = cfg->lattice == LBM_D2Q9;
     switch (cfg->storage) {
-    case LBM_STORE_F64: x.ops = &dispatch_f64(); break;
-    case LBM_STORE_F32: x.ops = &dispatch_f32(); break;
-    case LBM_STORE_F16S: x.ops = &dispatch_f16(); break;
-    default: x.ops = &dispatch_bf16(); break;
+    case LBM_STORE_F64: x.ops = d2 ? &dispatch_f64_d2q9() : &dispatch_f64_d3q19(); break;
+    case LBM_STORE_F32: x.ops = d2 ? &dispatch_f32_d2q9() : &dispatch_f32_d3q19(); break;
+    case LBM_STORE_F16S: x.ops = d2 ? &dispatch_f16_d2q9() : &dispatch_f16_d3q19(); break;
+    default: x.ops = d2 ? &dispatch_bf16_d2q9() : &dispatch_bf16_d3q19(); break;
     }
     fill_params(x);
 

@@ -1052,6 +1052,117 @@ __device__ __forceinline__ void gather_node(const typename S::T* __restrict__ P,
 }
 
 
+// The pull sources of a node: source x - E_b of direction b in the padded
+// layout (periodic wrap), whether it lies outside a closed face, and that
+// face's wall (the first closed axis crossed, x, y, z).
+template <int Q> struct Around {
+    int xs[3];                 // x - e, index e + 1
+    unsigned rows[3][3];       // rows (y - ey, z - ez)
+    bool ox[3], oy[3], oz[3];  // beyond a closed face
+    int x;
+    __device__ __forceinline__ Around(const Geo& g, int x_, int y, int z) : x(x_)
+    {
+        xs[0] = x == g.nx - 1 ? 0 : x + 1;
+        xs[1] = x;
+        xs[2] = x == 0 ? g.nx - 1 : x - 1;
+        const int ys[3] = {y == g.ny - 1 ? 0 : y + 1, y, y == 0 ? g.ny - 1 : y - 1};
+        const int zs[3] = {z == g.nz - 1 ? 0 : z + 1, z, z == 0 ? g.nz - 1 : z - 1};
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+#pragma unroll
+            for (int j = 0; j < 3; ++j)
+                rows[i][j] = ((unsigned)(Q == 19 ? zs[j] : 0) * (unsigned)g.ny + (unsigned)ys[i]) * (unsigned)g.nxp;
+        ox[0] = !g.periodic[0] && x == g.nx - 1;
+        ox[2] = !g.periodic[0] && x == 0;
+        oy[0] = !g.periodic[1] && y == g.ny - 1;
+        oy[2] = !g.periodic[1] && y == 0;
+        oz[0] = Q == 19 && !g.periodic[2] && z == g.nz - 1;
+        oz[2] = Q == 19 && !g.periodic[2] && z == 0;
+        ox[1] = oy[1] = oz[1] = false;
+    }
+    __device__ __forceinline__ unsigned own() const { return rows[1][1] + (unsigned)x; }
+    __device__ __forceinline__ unsigned at(int b) const
+    {
+        return rows[EY<Q>(b) + 1][EZ<Q>(b) + 1] + (unsigned)xs[EX<Q>(b) + 1];
+    }
+    __device__ __forceinline__ bool out(int b) const { return ox[EX<Q>(b) + 1] || oy[EY<Q>(b) + 1] || oz[EZ<Q>(b) + 1]; }
+    __device__ __forceinline__ int face(const Geo& g, int b) const
+    {
+        if (ox[EX<Q>(b) + 1]) return EX<Q>(b) > 0 ? g.face_wall[0] : g.face_wall[1];
+        if (oy[EY<Q>(b) + 1]) return EY<Q>(b) > 0 ? g.face_wall[2] : g.face_wall[3];
+        return EZ<Q>(b) > 0 ? g.face_wall[4] : g.face_wall[5];
+    }
+};
+__device__ __forceinline__ bool any_closed(const Geo& g, int Q)
+{
+    return !(g.periodic[0] && g.periodic[1] && (Q == 9 || g.periodic[2]));
+}
+
+// gather_node for kernels that visit every node, given the node's class byte:
+// the class decides once how the 19 loads are formed, so that they are issued
+// together instead of each behind its own class lookup and branch (the
+// canonical export of a 256^3 FP32 box: 2,254 -> 526 us, 0.72 of the copy
+// bandwidth).  Bulk nodes add nine row offsets and three x positions; in a
+// box with closed faces, bulk and face nodes alike pick the source or the
+// node's own opposite population by the node's position (no class bytes; one
+// path, so warps at the row ends do not diverge); nodes beside a solid load
+// their 18 sources' class bytes together, then the 18 values.  CURVED: nodes
+// beside a solid take gather_node (interpolated bounce-back).  Same values as
+// gather_node, bit for bit.
+template <int Q, class S, bool RAW, bool CURVED>
+__device__ __forceinline__ void pull_node(const typename S::T* __restrict__ P, const uint8_t* __restrict__ cls,
+                                          const Geo& g, const KP<typename S::R>& p, uint8_t c, int x, int y, int z,
+                                          typename S::R (&d)[Q])
+{
+    using T = typename S::T;
+    using R = typename S::R;
+    auto cv = [](T v) { return RAW ? S::to_raw(v) : S::to_r(v); };
+    if constexpr (CURVED) {
+        if (c == NC_BOUND) {
+            gather_node<Q, S, RAW, true>(P, cls, g, p, x, y, z, d);
+            return;
+        }
+    }
+    const Around<Q> ar(g, x, y, z);
+    if (!any_closed(g, Q) && c == NC_BULK) {
+        T v[Q];
+#pragma unroll
+        for (int b = 0; b < Q; ++b) v[b] = P[(long long)b * g.sq + ar.at(b)];
+#pragma unroll
+        for (int b = 0; b < Q; ++b) d[b] = cv(v[b]);
+        return;
+    }
+    const unsigned own = ar.own();
+    if (c != NC_BOUND) {
+        T v[Q];
+#pragma unroll
+        for (int b = 0; b < Q; ++b)
+            v[b] = P[ar.out(b) ? (long long)OPP<Q>(b) * g.sq + own : (long long)b * g.sq + ar.at(b)];
+#pragma unroll
+        for (int b = 0; b < Q; ++b) d[b] = cv(v[b]);
+        if (c == NC_FACE && p.face_ladd) {
+#pragma unroll
+            for (int b = 1; b < Q; ++b)
+                if (ar.out(b)) d[b] += ladd_of<Q, R>(p, b, ar.face(g, b));
+        }
+        return;
+    }
+    uint8_t cs[Q];
+    T v[Q];
+#pragma unroll
+    for (int b = 1; b < Q; ++b) cs[b] = ar.out(b) ? nc_make_solid(ar.face(g, b)) : cls[ar.at(b)];
+    v[0] = P[own];
+#pragma unroll
+    for (int b = 1; b < Q; ++b)
+        v[b] = P[nc_solid(cs[b]) ? (long long)OPP<Q>(b) * g.sq + own : (long long)b * g.sq + ar.at(b)];
+    d[0] = cv(v[0]);
+#pragma unroll
+    for (int b = 1; b < Q; ++b) {
+        d[b] = cv(v[b]);
+        if (nc_solid(cs[b])) d[b] += ladd_of<Q, R>(p, b, nc_wall(cs[b]));
+    }
+}
+
 // ----------------------------------------------------- induced field
 // Field distributions on the axis velocities of the fluid lattice: the
 // first QM fluid directions (rest, +-x, +-y [, +-z]) with weights W0, W1.

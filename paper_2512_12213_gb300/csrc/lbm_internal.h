@@ -98,10 +98,14 @@ struct Dispatch {
                            const double* dir, double seedw, double* partials, cudaStream_t);
 };
 
-const Dispatch& dispatch_f64();
-const Dispatch& dispatch_f32();
-const Dispatch& dispatch_f16();
-const Dispatch& dispatch_bf16();
+const Dispatch& dispatch_f64_d2q9();
+const Dispatch& dispatch_f64_d3q19();
+const Dispatch& dispatch_f32_d2q9();
+const Dispatch& dispatch_f32_d3q19();
+const Dispatch& dispatch_f16_d2q9();
+const Dispatch& dispatch_f16_d3q19();
+const Dispatch& dispatch_bf16_d2q9();
+const Dispatch& dispatch_bf16_d3q19();
 
 cudaError_t launch_reduce_rows(const double* partials, int nb, int W, double* out, double weight, int accumulate,
                                cudaStream_t st);

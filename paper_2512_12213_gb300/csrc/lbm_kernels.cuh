@@ -5,6 +5,7 @@
 #pragma once
 
 #include <algorithm>
+#include <type_traits>
 
 #include "lbm_device.cuh"
 #include "lbm_internal.h"
@@ -547,6 +548,34 @@ k_step(const typename S::T* __restrict__ src, typename S::T* __restrict__ dst,
     put_v();
 }
 
+// ------------------------------------------------- deviations and populations
+// w rho0 of the speed classes (rest, axis, diagonal) in FP64 and as an
+// unevaluated FP32 sum hi + lo (48 bits)
+struct WRho {
+    double c[3];
+    float hi[3], lo[3];
+};
+template <int Q> inline WRho wrho_of(double rho0)
+{
+    WRho w;
+    constexpr int a[3] = {0, 1, Q == 9 ? 5 : 7};
+    for (int k = 0; k < 3; ++k) {
+        w.c[k] = WD<Q>(a[k]) * rho0;
+        w.hi[k] = (float)w.c[k];
+        w.lo[k] = (float)(w.c[k] - (double)w.hi[k]);
+    }
+    return w;
+}
+// d + (hi + lo) rounded once to FP32: the error of d + hi recovered exactly
+// (Knuth's two-sum) and added with lo.  An FP64 addition holds an SM's FP64
+// pipe ~20 cycles a warp, 19 of them a node 0.17 ms of a 256 x 128 x 128 box.
+__device__ __forceinline__ float add_split(float d, float hi, float lo)
+{
+    const float s = __fadd_rn(d, hi), b = __fsub_rn(s, d);
+    const float e = __fadd_rn(__fsub_rn(d, __fsub_rn(s, b)), __fsub_rn(hi, b));
+    return __fadd_rn(s, __fadd_rn(e, lo));
+}
+
 // ------------------------------------------ inverse propagation (import/init)
 // Stored state P with gather(P) = the given canonical f: P_a(y) = f_a(y + E_a)
 // if y + E_a is fluid, else f_opp(a)(y) - (Ladd term of opp(a)).
@@ -671,27 +700,49 @@ k_inverse_stream(typename S::T* __restrict__ P, const uint8_t* __restrict__ cls,
 }
 
 // ---------------------------------------------------------------- export
-template <int Q, class S, typename OutT>
+// position of canonical node n (32-bit: the padded node count is below 2^31)
+struct NodeXYZ {
+    int x, y, z;
+    unsigned own;       // padded index
+};
+__device__ __forceinline__ NodeXYZ node_at(const Geo& g, unsigned n)
+{
+    const unsigned r = n / (unsigned)g.nx;
+    NodeXYZ q;
+    q.x = (int)(n - r * (unsigned)g.nx);
+    q.z = (int)(r / (unsigned)g.ny);
+    q.y = (int)(r - (unsigned)q.z * (unsigned)g.ny);
+    q.own = r * (unsigned)g.nxp + (unsigned)q.x;
+    return q;
+}
+
+// f = d + w rho0, one node per thread: bound by its loads and stores (bulk
+// nodes: 19 independent loads, no class lookups; see pull_node)
+template <int Q, class S, typename OutT, bool CURVED>
 __global__ void __launch_bounds__(NODE_THREADS)
 k_export(const typename S::T* __restrict__ P, const uint8_t* __restrict__ cls, const Geo g,
-         const KP<typename S::R> p, OutT* __restrict__ out)
+         const KP<typename S::R> p, const WRho wr, OutT* __restrict__ out)
 {
     using R = typename S::R;
-    const long long N = (long long)g.nx * g.ny * g.nz;
-    for (long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x; n < N; n += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(n % g.nx);
-        const long long r = n / g.nx;
-        const int y = (int)(r % g.ny), z = (int)(r / g.ny);
-        const uint8_t c = cls[r * g.nxp + x];
+    const unsigned N = (unsigned)g.nx * (unsigned)g.ny * (unsigned)g.nz;
+    for (unsigned n = blockIdx.x * blockDim.x + threadIdx.x; n < N; n += gridDim.x * blockDim.x) {
+        const NodeXYZ q = node_at(g, n);
+        const uint8_t c = cls[q.own];
         if (nc_solid(c)) {
 #pragma unroll
             for (int a = 0; a < Q; ++a) out[(long long)a * N + n] = OutT(0);
             continue;
         }
         R d[Q];
-        gather_node<Q, S>(P, cls, g, p, x, y, z, d);
+        pull_node<Q, S, false, CURVED>(P, cls, g, p, c, q.x, q.y, q.z, d);
 #pragma unroll
-        for (int a = 0; a < Q; ++a) out[(long long)a * N + n] = OutT((double)d[a] + WD<Q>(a) * (double)p.rho0);
+        for (int a = 0; a < Q; ++a) {
+            const int k = SPEED2<Q>(a);
+            if constexpr (sizeof(R) == 4 && sizeof(OutT) == 4)
+                out[(long long)a * N + n] = add_split(d[a], wr.hi[k], wr.lo[k]);
+            else
+                out[(long long)a * N + n] = OutT((double)d[a] + wr.c[k]);
+        }
     }
 }
 
@@ -760,42 +811,147 @@ k_links(const typename S::T* __restrict__ P, const uint8_t* __restrict__ cls, co
         for (int k = 0; k < 3; ++k) partials[(long long)blockIdx.x * 3 + k] = acc[k];
 }
 
+// ------------------------------------------------- exact moments of a node
+// Sums of a node's populations and momentum for the FP64 reductions.  The
+// FP64 pipe adds 1.6 lanes per cycle and SM: the plain FP64 sums (95
+// operations and conversions a node) held k_balance at 1.03 ms and k_residual
+// at 1.36 ms on the 256 x 128 x 128 box, 15 times their memory time.  FP32
+// deviations below 1/2 are therefore split without error into three 32-bit
+// integers on the grids 2^-23, 2^-43 and 2^-59 (adding 1.5 times a power of
+// two leaves the rounded multiple in the mantissa), summed in integer
+// arithmetic and joined in one 64-bit integer of units 2^-59: exact for every
+// deviation above 3e-11, and off by 2^-60 below, where an FP64 sum of values
+// near 0.01 rounds by 2^-60 at every addition.  A node with a larger or a
+// non-finite value takes FP64 sums.
+constexpr double FIX_UNIT = 1.0 / 576460752303423488.0;      // 2^-59
+
+// V = sum d, sum E d in units of 2^-59; false (V not set) if some |d| >= 1/2
+template <int Q>
+__device__ __forceinline__ bool fixed_moments(const float (&d)[Q], long long (&V)[4])
+{
+    constexpr int NP = LatDim<Q>::NP;
+    constexpr float M1 = 1.5f, M2 = 1.5f / 1048576.0f, M3 = 1.5f / 68719476736.0f;   // 1.5, 1.5 2^-20, 1.5 2^-36
+    unsigned sum[3][4] = {{0, 0, 0, 0}, {0, 0, 0, 0}, {0, 0, 0, 0}};
+    unsigned range = 0;
+    auto split = [&](F2 v, unsigned (&lo)[3], unsigned (&hi)[3]) {
+        constexpr float M[3] = {M1, M2, M3};
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const F2 t = f2add(v, f2s(M[k]));
+            lo[k] = __float_as_uint(t.v.x);
+            hi[k] = __float_as_uint(t.v.y);
+            if (k < 2) v = f2sub(v, f2add(t, f2s(-M[k])));
+        }
+        range |= (lo[0] ^ 0x3F800000u) | (hi[0] ^ 0x3F800000u);
+    };
+    constexpr unsigned K[3] = {0x3FC00000u, 0x35C00000u, 0x2DC00000u};      // the bits of M1, M2, M3
+#pragma unroll
+    for (int k = 0; k < NP; ++k) {
+        const int a = PAIR<Q>(k), b = OPP<Q>(a);
+        unsigned ua[3], ub[3];
+        split(F2{make_float2(d[a], d[b])}, ua, ub);
+        const int e[3] = {EX<Q>(a), EY<Q>(a), EZ<Q>(a)};
+#pragma unroll
+        for (int l = 0; l < 3; ++l) {
+            sum[l][0] += ua[l] + ub[l];
+            const unsigned df = ua[l] - ub[l];
+#pragma unroll
+            for (int c = 0; c < 3; ++c)
+                if (e[c]) sum[l][1 + c] += (e[c] > 0) ? df : 0u - df;
+        }
+    }
+    {
+        unsigned u0[3], u1[3];
+        split(F2{make_float2(d[0], 0.0f)}, u0, u1);
+#pragma unroll
+        for (int l = 0; l < 3; ++l) sum[l][0] += u0[l] - (unsigned)Q * K[l];
+    }
+    if (range >> 23) return false;
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+        V[c] = ((long long)(int)sum[0][c] << 36) + ((long long)(int)sum[1][c] << 16) + (long long)(int)sum[2][c];
+    return true;
+}
+// the same in FP64, from the even and odd parts of the opposite pairs
+template <int Q, typename R>
+__device__ __forceinline__ void double_moments(const R (&d)[Q], double (&s)[4])
+{
+    s[0] = (double)d[0];
+    s[1] = s[2] = s[3] = 0.0;
+#pragma unroll
+    for (int k = 0; k < LatDim<Q>::NP; ++k) {
+        const int a = PAIR<Q>(k), b = OPP<Q>(a);
+        const double da = (double)d[a], db = (double)d[b], df = da - db;
+        s[0] += da + db;
+        const int e[3] = {EX<Q>(a), EY<Q>(a), EZ<Q>(a)};
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+            if (e[c]) s[1 + c] = (e[c] > 0) ? s[1 + c] + df : s[1 + c] - df;
+    }
+}
+
 // ---------------------------------------------------------------- balance
-template <int Q, class S, bool EXT>
+// A thread's nodes are summed first (FP32 compute: exactly, the 64-bit node
+// sums in two 32-bit halves), then the block in FP64; the uniform body force
+// multiplies the summed density, a velocity-dependent one each node's.
+template <int Q, class S, bool EXT, bool CURVED>
 __global__ void __launch_bounds__(RED_THREADS)
 k_balance(const typename S::T* __restrict__ P, const uint8_t* __restrict__ cls, const Geo g,
           const KP<typename S::R> p, double vol, double* __restrict__ partials)
 {
     using R = typename S::R;
     __shared__ double sm[7 * 32];
-    double acc[7] = {0, 0, 0, 0, 0, 0, 0};
-    const long long N = (long long)g.nx * g.ny * g.nz;
-    const double c = (double)p.c;
-    for (long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x; n < N; n += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(n % g.nx);
-        const long long r = n / g.nx;
-        const int y = (int)(r % g.ny), z = (int)(r / g.ny);
-        if (nc_solid(cls[r * g.nxp + x])) continue;
+    double tot[4] = {0, 0, 0, 0}, fa[3] = {0, 0, 0};     // sums of d and E d; of rho A with EXT
+    long long hi[4] = {0, 0, 0, 0}, lo[4] = {0, 0, 0, 0};
+    int count = 0;
+    const unsigned N = (unsigned)g.nx * (unsigned)g.ny * (unsigned)g.nz;
+    for (unsigned n = blockIdx.x * blockDim.x + threadIdx.x; n < N; n += gridDim.x * blockDim.x) {
+        const NodeXYZ q = node_at(g, n);
+        const uint8_t c = cls[q.own];
+        if (nc_solid(c)) continue;
         R d[Q];
-        gather_node<Q, S>(P, cls, g, p, x, y, z, d);
-        double dr = 0, jx = 0, jy = 0, jz = 0;
+        pull_node<Q, S, false, CURVED>(P, cls, g, p, c, q.x, q.y, q.z, d);
+        ++count;
+        double s[4];
+        bool fixed = false;
+        if constexpr (sizeof(R) == 4) {
+            long long V[4];
+            fixed = fixed_moments<Q>(d, V);
+            if (fixed) {
 #pragma unroll
-        for (int a = 0; a < Q; ++a) {
-            const double da = (double)d[a];
-            dr += da;
-            jx += EX<Q>(a) * da;
-            jy += EY<Q>(a) * da;
-            jz += EZ<Q>(a) * da;
+                for (int k = 0; k < 4; ++k) {
+                    hi[k] += V[k] >> 32;
+                    lo[k] += V[k] & 0xFFFFFFFFll;
+                }
+                if (EXT) s[0] = (double)V[0] * FIX_UNIT;
+            }
         }
-        NodeM<R> m;
-        node_macro<R, Q, EXT>(d, p, m);
-        const double rho = (double)p.rho0 + dr;
-        acc[0] += vol * rho;
-        acc[1] += vol * c * jx;
-        acc[2] += vol * c * jy;
-        acc[3] += vol * c * jz;
+        if (!fixed) {
+            double_moments<Q, R>(d, s);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) tot[k] += s[k];
+        }
+        if constexpr (EXT) {
+            NodeM<R> m;
+            node_macro<R, Q, EXT>(d, p, m);
+            const double rho = (double)p.rho0 + s[0];
+#pragma unroll
+            for (int k = 0; k < 3; ++k) fa[k] += rho * (double)m.A[k];
+        }
+    }
+    if constexpr (sizeof(R) == 4) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) tot[k] += ((double)hi[k] * 4294967296.0 + (double)lo[k]) * FIX_UNIT;
+    }
+    const double rho = (double)p.rho0 * count + tot[0], c = (double)p.c;
+    double acc[7];
+    acc[0] = vol * rho;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        acc[1 + k] = vol * c * tot[1 + k];
         // rho a = rho (c/dt) A
-        for (int k = 0; k < 3; ++k) acc[4 + k] += vol * rho * (c / (double)p.dt) * (double)m.A[k];
+        if constexpr (!EXT) fa[k] = rho * ((k < LatDim<Q>::D) ? (double)p.AG[k] : 0.0);
+        acc[4 + k] = vol * (c / (double)p.dt) * fa[k];
     }
     block_sum<7>(acc, sm);
     if (threadIdx.x == 0)
@@ -805,11 +961,12 @@ k_balance(const typename S::T* __restrict__ P, const uint8_t* __restrict__ cls, 
 // ------------------------------------------------------- steady residual
 // Sec. 6: the balance of Eq. (32) between wall force and body force holds
 // once the flow stops changing.  Per fluid node of f(T): the flow velocity
-// v = c (j/rho + A/2) (text after Eq. 1; the moments summed in FP64 from the
-// stored values), |v - v_ref| and |v| (Euclidean norms), block sums in FP64
-// for the fixed-order pass; with `update` the node's v replaces v_ref (each
-// thread reads its own entries before it writes them; solid nodes get 0).
-template <int Q, class S, bool EXT>
+// v = c (j/rho + A/2) (text after Eq. 1; the moments summed in FP64 or
+// exactly from the stored values, see above), |v - v_ref| and |v| (Euclidean
+// norms), block sums in FP64 for the fixed-order pass; with `update` the
+// node's v replaces v_ref (each thread reads its own entries before it writes
+// them; solid nodes get 0).
+template <int Q, class S, bool EXT, bool CURVED>
 __global__ void __launch_bounds__(RED_THREADS)
 k_residual(const typename S::T* __restrict__ P, const uint8_t* __restrict__ cls, const Geo g,
            const KP<typename S::R> p, double* __restrict__ vref, int update, double* __restrict__ partials)
@@ -817,37 +974,50 @@ k_residual(const typename S::T* __restrict__ P, const uint8_t* __restrict__ cls,
     using R = typename S::R;
     __shared__ double sm[2 * 32];
     double acc[2] = {0.0, 0.0};
-    const long long N = (long long)g.nx * g.ny * g.nz;
+    const unsigned N = (unsigned)g.nx * (unsigned)g.ny * (unsigned)g.nz;
     const double c = (double)p.c;
-    for (long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x; n < N; n += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(n % g.nx);
-        const long long r = n / g.nx;
-        const int y = (int)(r % g.ny), z = (int)(r / g.ny);
-        if (nc_solid(cls[r * g.nxp + x])) {
+    for (unsigned n = blockIdx.x * blockDim.x + threadIdx.x; n < N; n += gridDim.x * blockDim.x) {
+        const NodeXYZ q = node_at(g, n);
+        const uint8_t cl = cls[q.own];
+        if (nc_solid(cl)) {
             if (update)
 #pragma unroll
                 for (int k = 0; k < 3; ++k) vref[(long long)k * N + n] = 0.0;
             continue;
         }
-        R d[Q];
-        gather_node<Q, S>(P, cls, g, p, x, y, z, d);
-        NodeM<R> m;
-        node_macro<R, Q, EXT>(d, p, m);
-        double dr = 0.0, j[3] = {0.0, 0.0, 0.0};
+        double vr[3];
 #pragma unroll
-        for (int a = 0; a < Q; ++a) {
-            const double da = (double)d[a];
-            dr += da;
-            j[0] += EX<Q>(a) * da;
-            j[1] += EY<Q>(a) * da;
-            j[2] += EZ<Q>(a) * da;
+        for (int k = 0; k < 3; ++k) vr[k] = vref[(long long)k * N + n];
+        R d[Q];
+        pull_node<Q, S, false, CURVED>(P, cls, g, p, cl, q.x, q.y, q.z, d);
+        double s[4], unit = 1.0;         // the moments in units of `unit`
+        bool fixed = false;
+        if constexpr (sizeof(R) == 4) {
+            long long V[4];
+            fixed = fixed_moments<Q>(d, V);
+            if (fixed) {
+                unit = FIX_UNIT;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) s[k] = (double)V[k];
+            }
         }
-        const double rho = (double)p.rho0 + dr;
+        if (!fixed) double_moments<Q, R>(d, s);
+        double A[3];
+        if constexpr (EXT) {
+            NodeM<R> m;
+            node_macro<R, Q, EXT>(d, p, m);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) A[k] = (double)m.A[k];
+        } else {
+#pragma unroll
+            for (int k = 0; k < 3; ++k) A[k] = (k < LatDim<Q>::D) ? (double)p.AG[k] : 0.0;
+        }
+        const double ir = c * unit / fma(s[0], unit, (double)p.rho0);
         double dd = 0.0, vv = 0.0;
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            const double vk = c * (j[k] / rho + 0.5 * (double)m.A[k]);
-            const double dk = vk - vref[(long long)k * N + n];
+            const double vk = fma(s[1 + k], ir, 0.5 * c * A[k]);
+            const double dk = vk - vr[k];
             dd += dk * dk;
             vv += vk * vk;
             if (update) vref[(long long)k * N + n] = vk;
@@ -863,7 +1033,7 @@ k_residual(const typename S::T* __restrict__ P, const uint8_t* __restrict__ cls,
 // ----------------------------------------------------------------- stress
 // Variants 1, 2 at f(T) = gather(cur); 3, 4 at the half step between T-1 and
 // T: fbar = (cur + gather(cur))/2 with the node's state at T-1 = gather(prev).
-template <int Q, class S, bool EXT>
+template <int Q, class S, bool EXT, bool CURVED>
 __global__ void __launch_bounds__(NODE_THREADS)
 k_stress(const typename S::T* __restrict__ cur, const typename S::T* __restrict__ prev,
          const uint8_t* __restrict__ cls, const Geo g, const KP<typename S::R> p, int variant,
@@ -873,15 +1043,15 @@ k_stress(const typename S::T* __restrict__ cur, const typename S::T* __restrict_
     using R = typename S::R;
     constexpr int D = LatDim<Q>::D;
     constexpr int NC = (D == 3) ? 6 : 3;
-    const long long N = (long long)g.nx * g.ny * g.nz;
+    const unsigned N = (unsigned)g.nx * (unsigned)g.ny * (unsigned)g.nz;
     const R c = p.c, c2 = p.c * p.c;
-    for (long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x; n < N; n += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(n % g.nx);
-        const long long r = n / g.nx;
-        const int y = (int)(r % g.ny), z = (int)(r / g.ny);
-        const long long own = r * g.nxp + x;
+    for (unsigned n = blockIdx.x * blockDim.x + threadIdx.x; n < N; n += gridDim.x * blockDim.x) {
+        const NodeXYZ q = node_at(g, n);
+        const int x = q.x, y = q.y, z = q.z;
+        const unsigned own = q.own;
+        const uint8_t cl = cls[own];
         R out[6] = {0, 0, 0, 0, 0, 0}, Sv[6] = {0, 0, 0, 0, 0, 0}, rr = 0, vv[3] = {0, 0, 0};
-        if (!nc_solid(cls[own])) {
+        if (!nc_solid(cl)) {
             R d[Q];
             NodeM<R> m;
             // component index -> (i, j)
@@ -903,7 +1073,7 @@ k_stress(const typename S::T* __restrict__ cur, const typename S::T* __restrict_
                 Lh[5] = -kl * B[1] * B[2];
             }
             if (variant <= 2) {
-                gather_node<Q, S>(cur, cls, g, p, x, y, z, d);
+                pull_node<Q, S, false, CURVED>(cur, cls, g, p, cl, x, y, z, d);
                 node_macro<R, Q, EXT>(d, p, m);
                 const R fac = -(R(1) - R(0.5) * m.om) * c2;
                 const bool model_a = (p.model == MODEL_A);
@@ -934,7 +1104,7 @@ k_stress(const typename S::T* __restrict__ cur, const typename S::T* __restrict_
                 for (int k = 0; k < 3; ++k) vv[k] = c * m.v[k];
             } else {
                 R dn[Q];
-                gather_node<Q, S>(cur, cls, g, p, x, y, z, dn);
+                pull_node<Q, S, false, CURVED>(cur, cls, g, p, cl, x, y, z, dn);
                 R db[Q];
                 R drb = 0, jb[3] = {0, 0, 0};
 #pragma unroll
@@ -947,7 +1117,7 @@ k_stress(const typename S::T* __restrict__ cur, const typename S::T* __restrict_
                 }
                 const R rb = p.rho0 + drb;
                 const R ub[3] = {jb[0] / rb, jb[1] / rb, jb[2] / rb};
-                gather_node<Q, S>(prev, cls, g, p, x, y, z, d);
+                pull_node<Q, S, false, CURVED>(prev, cls, g, p, cl, x, y, z, d);
                 node_macro<R, Q, EXT>(d, p, m);
 #pragma unroll
                 for (int cc = 0; cc < NC; ++cc) {
@@ -1240,6 +1410,22 @@ cudaError_t launch_step(const Ctx& c, const void* src, void* dst, uint32_t seed,
                  : launch_step_q<Q, S, false, false>(c, src, dst, seed, st);
 }
 
+// calls f with the kernel's compile-time flags: CURVED (interpolated walls)
+template <class F> inline cudaError_t with_curved(const Ctx& c, F&& f)
+{
+    if (c.cfg.curved) f(std::true_type{});
+    else f(std::false_type{});
+    return cudaGetLastError();
+}
+// and EXT, CURVED
+template <class F> inline cudaError_t with_ext_curved(const Ctx& c, F&& f)
+{
+    return with_curved(c, [&](auto cu) {
+        if (c.ext) f(std::true_type{}, cu);
+        else f(std::false_type{}, cu);
+    });
+}
+
 template <int Q, class S>
 cudaError_t launch_import(const Ctx& c, const void* srcf, int dtype, void* dst, cudaStream_t st)
 {
@@ -1275,11 +1461,28 @@ cudaError_t launch_export(const Ctx& c, const void* P, void* out, int dtype, cud
     using T = typename S::T;
     const long long N = (long long)c.geo.nx * c.geo.ny * c.geo.nz;
     const int blocks = grid_for(N, NODE_THREADS, 65535ll * 16);
-    if (dtype == 0)
-        k_export<Q, S, double><<<blocks, NODE_THREADS, 0, st>>>((const T*)P, c.cls, c.geo, kp_of<S>(c), (double*)out);
-    else
-        k_export<Q, S, float><<<blocks, NODE_THREADS, 0, st>>>((const T*)P, c.cls, c.geo, kp_of<S>(c), (float*)out);
-    return cudaGetLastError();
+    const WRho wr = wrho_of<Q>((double)kp_of<S>(c).rho0);
+    return with_curved(c, [&](auto cu) {
+        if (dtype == 0)
+            k_export<Q, S, double, cu.value><<<blocks, NODE_THREADS, 0, st>>>((const T*)P, c.cls, c.geo, kp_of<S>(c),
+                                                                               wr, (double*)out);
+        else
+            k_export<Q, S, float, cu.value><<<blocks, NODE_THREADS, 0, st>>>((const T*)P, c.cls, c.geo, kp_of<S>(c),
+                                                                              wr, (float*)out);
+    });
+}
+
+// grid of a reduction over nodes: at most the two blocks per SM that its
+// registers allow at once, so that there is no second wave and each block's
+// FP64 tail (~1.3 us of an SM's FP64 pipe) is paid twice an SM; fewer threads
+// per block, a warp at least, where a box is too small for a block of 256
+// nodes on every SM
+inline int red_grid(const Ctx& c, long long N, int& threads)
+{
+    threads = RED_THREADS;
+    while (threads > 32 && N < (long long)threads * c.sm_count) threads /= 2;
+    const long long most = N / (8ll * threads) > c.sm_count ? 2ll * c.sm_count : c.sm_count;
+    return grid_for(N, threads, std::min<long long>(MAX_PARTIAL_ROWS, most));
 }
 
 template <int Q, class S>
@@ -1299,14 +1502,14 @@ cudaError_t launch_balance(const Ctx& c, const void* P, double* partials, int* n
 {
     using T = typename S::T;
     const long long N = (long long)c.geo.nx * c.geo.ny * c.geo.nz;
-    const int blocks = grid_for(N, RED_THREADS, MAX_PARTIAL_ROWS);
+    int threads;
+    const int blocks = red_grid(c, N, threads);
     *nblocks = blocks;
     const double vol = (Q == 9) ? c.cfg.dx * c.cfg.dx : c.cfg.dx * c.cfg.dx * c.cfg.dx;
-    if (c.ext)
-        k_balance<Q, S, true><<<blocks, RED_THREADS, 0, st>>>((const T*)P, c.cls, c.geo, kp_of<S>(c), vol, partials);
-    else
-        k_balance<Q, S, false><<<blocks, RED_THREADS, 0, st>>>((const T*)P, c.cls, c.geo, kp_of<S>(c), vol, partials);
-    return cudaGetLastError();
+    return with_ext_curved(c, [&](auto ex, auto cu) {
+        k_balance<Q, S, ex.value, cu.value><<<blocks, threads, 0, st>>>((const T*)P, c.cls, c.geo, kp_of<S>(c), vol,
+                                                                        partials);
+    });
 }
 
 template <int Q, class S>
@@ -1315,15 +1518,13 @@ cudaError_t launch_residual(const Ctx& c, const void* P, double* vref, int updat
 {
     using T = typename S::T;
     const long long N = (long long)c.geo.nx * c.geo.ny * c.geo.nz;
-    const int blocks = grid_for(N, RED_THREADS, MAX_PARTIAL_ROWS);
+    int threads;
+    const int blocks = red_grid(c, N, threads);
     *nblocks = blocks;
-    if (c.ext)
-        k_residual<Q, S, true><<<blocks, RED_THREADS, 0, st>>>((const T*)P, c.cls, c.geo, kp_of<S>(c), vref, update,
-                                                               partials);
-    else
-        k_residual<Q, S, false><<<blocks, RED_THREADS, 0, st>>>((const T*)P, c.cls, c.geo, kp_of<S>(c), vref, update,
-                                                                partials);
-    return cudaGetLastError();
+    return with_ext_curved(c, [&](auto ex, auto cu) {
+        k_residual<Q, S, ex.value, cu.value><<<blocks, threads, 0, st>>>((const T*)P, c.cls, c.geo, kp_of<S>(c), vref,
+                                                                         update, partials);
+    });
 }
 
 template <int Q, class S>
@@ -1334,14 +1535,11 @@ cudaError_t launch_stress(const Ctx& c, const void* cur, const void* prev, int v
     using R = typename S::R;
     const long long N = (long long)c.geo.nx * c.geo.ny * c.geo.nz;
     const int blocks = grid_for(N, NODE_THREADS, 65535ll * 16);
-    if (c.ext)
-        k_stress<Q, S, true><<<blocks, NODE_THREADS, 0, st>>>((const T*)cur, (const T*)prev, c.cls, c.geo,
-                                                              with_mag(kp_of<S>(c), c.mag[c.cur]), variant, (R*)sig,
-                                                              (R*)Sv, (R*)rho, (R*)v);
-    else
-        k_stress<Q, S, false><<<blocks, NODE_THREADS, 0, st>>>((const T*)cur, (const T*)prev, c.cls, c.geo, kp_of<S>(c),
-                                                               variant, (R*)sig, (R*)Sv, (R*)rho, (R*)v);
-    return cudaGetLastError();
+    return with_ext_curved(c, [&](auto ex, auto cu) {
+        k_stress<Q, S, ex.value, cu.value><<<blocks, NODE_THREADS, 0, st>>>(
+            (const T*)cur, (const T*)prev, c.cls, c.geo, with_mag(kp_of<S>(c), c.cfg.induced ? c.mag[c.cur] : nullptr),
+            variant, (R*)sig, (R*)Sv, (R*)rho, (R*)v);
+    });
 }
 
 template <int Q, class S>
@@ -1388,57 +1586,26 @@ cudaError_t launch_mag_field(const Ctx& c, double* B, cudaStream_t st)
 
 namespace lbm {
 
-template <class S> Dispatch make_dispatch()
+template <int Q, class S> Dispatch make_dispatch()
 {
     Dispatch d;
     d.step = [](const Ctx& c, const void* s, void* t, uint32_t seed, cudaStream_t st) {
-        return c.cfg.lattice == 9 ? launch_step<9, S>(c, s, t, seed, st) : launch_step<19, S>(c, s, t, seed, st);
+        return launch_step<Q, S>(c, s, t, seed, st);
     };
     d.step_force = [](const Ctx& c, const void* s, void* t, uint32_t seed, const StgForce& fw, cudaStream_t st) {
-        return c.cfg.lattice == 9 ? launch_step<9, S>(c, s, t, seed, st, &fw)
-                                  : launch_step<19, S>(c, s, t, seed, st, &fw);
+        return launch_step<Q, S>(c, s, t, seed, st, &fw);
     };
-    d.import_f = [](const Ctx& c, const void* s, int dt, void* t, cudaStream_t st) {
-        return c.cfg.lattice == 9 ? launch_import<9, S>(c, s, dt, t, st) : launch_import<19, S>(c, s, dt, t, st);
-    };
-    d.init_fields = [](const Ctx& c, const double* r, const double* u, const double* xi, void* t, cudaStream_t st) {
-        return c.cfg.lattice == 9 ? launch_init<9, S>(c, r, u, xi, t, st) : launch_init<19, S>(c, r, u, xi, t, st);
-    };
-    d.export_f = [](const Ctx& c, const void* P, void* o, int dt, cudaStream_t st) {
-        return c.cfg.lattice == 9 ? launch_export<9, S>(c, P, o, dt, st) : launch_export<19, S>(c, P, o, dt, st);
-    };
-    d.links = [](const Ctx& c, const void* P, long long b, long long e, unsigned fl, double* pa, int* nb,
-                 cudaStream_t st) {
-        return c.cfg.lattice == 9 ? launch_links<9, S>(c, P, b, e, fl, pa, nb, st)
-                                  : launch_links<19, S>(c, P, b, e, fl, pa, nb, st);
-    };
-    d.balance = [](const Ctx& c, const void* P, double* pa, int* nb, cudaStream_t st) {
-        return c.cfg.lattice == 9 ? launch_balance<9, S>(c, P, pa, nb, st) : launch_balance<19, S>(c, P, pa, nb, st);
-    };
-    d.residual = [](const Ctx& c, const void* P, double* vr, int up, double* pa, int* nb, cudaStream_t st) {
-        return c.cfg.lattice == 9 ? launch_residual<9, S>(c, P, vr, up, pa, nb, st)
-                                  : launch_residual<19, S>(c, P, vr, up, pa, nb, st);
-    };
-    d.stress = [](const Ctx& c, const void* cu, const void* pr, int var, void* sg, void* Sv, void* rh, void* v,
-                  cudaStream_t st) {
-        return c.cfg.lattice == 9 ? launch_stress<9, S>(c, cu, pr, var, sg, Sv, rh, v, st)
-                                  : launch_stress<19, S>(c, cu, pr, var, sg, Sv, rh, v, st);
-    };
-    d.mhd_step = [](const Ctx& c, const void* s, void* t, const void* G, void* Gn, uint32_t seed, cudaStream_t st) {
-        return c.cfg.lattice == 9 ? launch_mhd_step<9, S>(c, s, t, G, Gn, seed, st)
-                                  : launch_mhd_step<19, S>(c, s, t, G, Gn, seed, st);
-    };
-    d.mag_init = [](const Ctx& c, cudaStream_t st) {
-        return c.cfg.lattice == 9 ? launch_mag_init<9, S>(c, st) : launch_mag_init<19, S>(c, st);
-    };
-    d.mag_field = [](const Ctx& c, double* B, cudaStream_t st) {
-        return c.cfg.lattice == 9 ? launch_mag_field<9, S>(c, B, st) : launch_mag_field<19, S>(c, B, st);
-    };
-    d.adjoint = [](const Ctx& c, const void* Pp, const void* pn, void* po, int w, const double* dir, double sw,
-                   double* pa, cudaStream_t st) {
-        return c.cfg.lattice == 9 ? launch_adjoint<9, S>(c, Pp, pn, po, w, dir, sw, pa, st)
-                                  : launch_adjoint<19, S>(c, Pp, pn, po, w, dir, sw, pa, st);
-    };
+    d.import_f = launch_import<Q, S>;
+    d.init_fields = launch_init<Q, S>;
+    d.export_f = launch_export<Q, S>;
+    d.links = launch_links<Q, S>;
+    d.balance = launch_balance<Q, S>;
+    d.residual = launch_residual<Q, S>;
+    d.stress = launch_stress<Q, S>;
+    d.mhd_step = launch_mhd_step<Q, S>;
+    d.mag_init = launch_mag_init<Q, S>;
+    d.mag_field = launch_mag_field<Q, S>;
+    d.adjoint = launch_adjoint<Q, S>;
     return d;
 }
 
