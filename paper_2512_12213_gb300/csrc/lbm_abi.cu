@@ -198,15 +198,18 @@ void build_geometry(const lbm_config* c, const uint8_t* wid, int nxp, std::vecto
 
 // the 4-node chunks of the padded layout that hold a node other than a bulk
 // fluid node or a node whose only wall links cross a closed box face (a
-// solid neighbour, a solid node, padding): the first node of each, in order.
-// The staged step leaves them to its boundary warps.
+// solid neighbour, a solid node, the end of a ragged row; not padding alone):
+// the first node of each, in order.  The staged step leaves them to its
+// boundary warps.
 std::vector<uint32_t> special_chunks(const std::vector<uint8_t>& cls)
 {
     std::vector<uint32_t> out;
     auto plain = [](uint8_t c) { return c == NC_BULK || c == NC_FACE; };
-    for (size_t i = 0; i + 3 < cls.size(); i += 4)
+    for (size_t i = 0; i + 3 < cls.size(); i += 4) {
+        if (cls[i] == NC_PAD) continue;
         if (!plain(cls[i]) || !plain(cls[i + 1]) || !plain(cls[i + 2]) || !plain(cls[i + 3]))
             out.push_back((uint32_t)i);
+    }
     return out;
 }
 

@@ -923,6 +923,20 @@ __device__ __forceinline__ R ladd_of(const KP<R>& p, int a, int wall)
 {
     return R(WD<Q>(a)) * (R(EX<Q>(a)) * p.LW[wall][0] + R(EY<Q>(a)) * p.LW[wall][1] + R(EZ<Q>(a)) * p.LW[wall][2]);
 }
+// v plus (ladd_on) or minus (ladd_off) that term, rounded once: every kernel
+// forms a bounced population this way, so they agree bit for bit
+template <int Q, typename R>
+__device__ __forceinline__ R ladd_on(R v, const KP<R>& p, int a, int wall)
+{
+    return fma(R(WD<Q>(a)),
+               R(EX<Q>(a)) * p.LW[wall][0] + R(EY<Q>(a)) * p.LW[wall][1] + R(EZ<Q>(a)) * p.LW[wall][2], v);
+}
+template <int Q, typename R>
+__device__ __forceinline__ R ladd_off(R v, const KP<R>& p, int a, int wall)
+{
+    return fma(R(-WD<Q>(a)),
+               R(EX<Q>(a)) * p.LW[wall][0] + R(EY<Q>(a)) * p.LW[wall][1] + R(EZ<Q>(a)) * p.LW[wall][2], v);
+}
 
 // Box-face bounce-back inside the vectorised path (FACES = some axis is
 // closed).  For direction a at a chunk of row (y, z): the pull-source row is
@@ -1010,9 +1024,8 @@ __device__ __forceinline__ typename S::R bounced(const typename S::T* __restrict
     using R = typename S::R;
     auto cv = [](typename S::T v) { return RAW ? S::to_raw(v) : S::to_r(v); };
     const int a = OPP<Q>(b);
-    const R L = R(WD<Q>(b)) * (R(EX<Q>(b)) * p.LW[wall][0] + R(EY<Q>(b)) * p.LW[wall][1] + R(EZ<Q>(b)) * p.LW[wall][2]);
     const R Pa = cv(P[(long long)a * g.sq + own]);
-    const R out = Pa + L;
+    const R out = ladd_on<Q, R>(Pa, p, b, wall);
     if (!CURVED || !g.phi) return out;
     const long long s = link_target(g, x, y, z, EX<Q>(a), EY<Q>(a), EZ<Q>(a));
     if (s < 0 || !nc_solid(cls[s])) return out;            // a closed box face
@@ -1022,7 +1035,7 @@ __device__ __forceinline__ typename S::R bounced(const typename S::T* __restrict
     long long ff;
     int w2;
     if (!pull_source(g, cls, x, y, z, EX<Q>(a), EY<Q>(a), EZ<Q>(a), ff, w2)) return out;
-    return R(2) * q * Pa + (R(1) - R(2) * q) * cv(P[(long long)a * g.sq + ff]) + L;
+    return ladd_on<Q, R>(R(2) * q * Pa + (R(1) - R(2) * q) * cv(P[(long long)a * g.sq + ff]), p, b, wall);
 }
 
 // canonical post-propagation deviations at node (x,y,z) from a stored
@@ -1098,6 +1111,33 @@ __device__ __forceinline__ bool any_closed(const Geo& g, int Q)
     return !(g.periodic[0] && g.periodic[1] && (Q == 9 || g.periodic[2]));
 }
 
+// the canonical populations of any fluid node with halfway walls: the class
+// bytes of its 18 sources loaded together, then the 18 values
+template <int Q, class S, bool RAW>
+__device__ __forceinline__ void pull_walls(const typename S::T* __restrict__ P, const uint8_t* __restrict__ cls,
+                                           const Geo& g, const KP<typename S::R>& p, const Around<Q>& ar,
+                                           typename S::R (&d)[Q])
+{
+    using T = typename S::T;
+    using R = typename S::R;
+    auto cv = [](T v) { return RAW ? S::to_raw(v) : S::to_r(v); };
+    const unsigned own = ar.own();
+    uint8_t cs[Q];
+    T v[Q];
+#pragma unroll
+    for (int b = 1; b < Q; ++b) cs[b] = ar.out(b) ? nc_make_solid(ar.face(g, b)) : cls[ar.at(b)];
+    v[0] = P[own];
+#pragma unroll
+    for (int b = 1; b < Q; ++b)
+        v[b] = P[nc_solid(cs[b]) ? (long long)OPP<Q>(b) * g.sq + own : (long long)b * g.sq + ar.at(b)];
+    d[0] = cv(v[0]);
+#pragma unroll
+    for (int b = 1; b < Q; ++b) {
+        d[b] = cv(v[b]);
+        if (nc_solid(cs[b])) d[b] = ladd_on<Q, R>(d[b], p, b, nc_wall(cs[b]));
+    }
+}
+
 // gather_node for kernels that visit every node, given the node's class byte:
 // the class decides once how the 19 loads are formed, so that they are issued
 // together instead of each behind its own class lookup and branch (the
@@ -1105,9 +1145,8 @@ __device__ __forceinline__ bool any_closed(const Geo& g, int Q)
 // bandwidth).  Bulk nodes add nine row offsets and three x positions; in a
 // box with closed faces, bulk and face nodes alike pick the source or the
 // node's own opposite population by the node's position (no class bytes; one
-// path, so warps at the row ends do not diverge); nodes beside a solid load
-// their 18 sources' class bytes together, then the 18 values.  CURVED: nodes
-// beside a solid take gather_node (interpolated bounce-back).  Same values as
+// path, so warps at the row ends do not diverge); nodes beside a solid take
+// pull_walls, or (CURVED) gather_node with its interpolated bounce-back.  Same values as
 // gather_node, bit for bit.
 template <int Q, class S, bool RAW, bool CURVED>
 __device__ __forceinline__ void pull_node(const typename S::T* __restrict__ P, const uint8_t* __restrict__ cls,
@@ -1143,23 +1182,41 @@ __device__ __forceinline__ void pull_node(const typename S::T* __restrict__ P, c
         if (c == NC_FACE && p.face_ladd) {
 #pragma unroll
             for (int b = 1; b < Q; ++b)
-                if (ar.out(b)) d[b] += ladd_of<Q, R>(p, b, ar.face(g, b));
+                if (ar.out(b)) d[b] = ladd_on<Q, R>(d[b], p, b, ar.face(g, b));
         }
         return;
     }
-    uint8_t cs[Q];
-    T v[Q];
+    pull_walls<Q, S, RAW>(P, cls, g, p, ar, d);
+}
+
+// The mirror of pull_node: stores a node's canonical populations d where its
+// pulls read them, so that pull_node on the stored state gives d back: the
+// link source's P_b, or through a wall the node's own P_opp(b), less Ladd's
+// term.  Every entry of a fluid node in P has one writer.  Nodes beside a
+// solid load their sources' class bytes together.  Halfway walls.
+template <int Q, class S>
+__device__ __forceinline__ void push_node(typename S::T* __restrict__ P, const uint8_t* __restrict__ cls, const Geo& g,
+                                          const KP<typename S::R>& p, uint8_t c, int x, int y, int z,
+                                          const typename S::R (&d)[Q])
+{
+    using R = typename S::R;
+    const Around<Q> ar(g, x, y, z);
+    if (!any_closed(g, Q) && c == NC_BULK) {
 #pragma unroll
-    for (int b = 1; b < Q; ++b) cs[b] = ar.out(b) ? nc_make_solid(ar.face(g, b)) : cls[ar.at(b)];
-    v[0] = P[own];
+        for (int b = 0; b < Q; ++b) P[(long long)b * g.sq + ar.at(b)] = S::from_r(d[b]);
+        return;
+    }
+    const unsigned own = ar.own();
+    P[own] = S::from_r(d[0]);
+    uint8_t cs[Q];
 #pragma unroll
     for (int b = 1; b < Q; ++b)
-        v[b] = P[nc_solid(cs[b]) ? (long long)OPP<Q>(b) * g.sq + own : (long long)b * g.sq + ar.at(b)];
-    d[0] = cv(v[0]);
+        cs[b] = ar.out(b) ? nc_make_solid(ar.face(g, b)) : (c == NC_BOUND ? cls[ar.at(b)] : (uint8_t)NC_BULK);
 #pragma unroll
     for (int b = 1; b < Q; ++b) {
-        d[b] = cv(v[b]);
-        if (nc_solid(cs[b])) d[b] += ladd_of<Q, R>(p, b, nc_wall(cs[b]));
+        const bool hit = nc_solid(cs[b]);
+        const R v = hit ? ladd_off<Q, R>(d[b], p, b, nc_wall(cs[b])) : d[b];
+        P[hit ? (long long)OPP<Q>(b) * g.sq + own : (long long)b * g.sq + ar.at(b)] = S::from_r(v);
     }
 }
 

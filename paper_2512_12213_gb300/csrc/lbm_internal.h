@@ -163,8 +163,8 @@ struct Ctx {
     long long n_fluid;
 };
 
-// blocks of the staged step: one per SM, at most one per tile (each writes
-// one partial row of the fused wall force)
+// blocks of the staged step: one per SM, at most one per tile (each boundary
+// warp writes one partial row of the fused wall force)
 inline int staged_blocks(const Ctx& c) { return (int)(c.stage_tiles < c.sm_count ? c.stage_tiles : c.sm_count); }
 
 }  // namespace lbm

@@ -82,8 +82,13 @@ __device__ __forceinline__ void block_sum(double (&v)[W], double* smem /* >= W *
 // warp edge.  16-bit formats stay packed two to a register (the x shift is a
 // byte permute) and are relaxed two nodes at a time.  A chunk that holds a
 // boundary, solid or padding node is recomputed node by node with explicit
-// bounce-back.  Populations are in storage units (kernel parameters scaled
-// to match).
+// bounce-back, the warp's such nodes spread over its lanes: one lane walking
+// its chunk held the warp for up to four round trips, and a box of ragged
+// rows has such a chunk in every row (sphere 250 x 121 x 99 in FP32: 141 ->
+// 92 us).  Chunks of padding alone are not touched
+// unless zero_pad asks for it (a destination that is not the context's own,
+// whose padding is zero already).  Populations are in storage units (kernel
+// parameters scaled to match).
 // blocks of 128 threads per SM the register allocation must allow: FP64 3
 // (168 registers), else 4 (128; for 16-bit storage measured faster than 5
 // blocks at 96 registers, which spill with the FP32x2 node pairs)
@@ -107,7 +112,7 @@ template <class S, bool EXT, bool FACES = false, bool FULL = false, bool LP = fa
 template <int Q, class S, bool EXT, bool FACES, bool SR, bool FULL = false, bool LP = false>
 __global__ void __launch_bounds__(STEP_THREADS, StepOcc<S, EXT, FACES, FULL, LP>::value)
 k_step(const typename S::T* __restrict__ src, typename S::T* __restrict__ dst,
-       const uint8_t* __restrict__ cls, const Geo g, const KP<typename S::R> p, uint32_t seed)
+       const uint8_t* __restrict__ cls, const Geo g, const KP<typename S::R> p, uint32_t seed, int zero_pad)
 {
     using T = typename S::T;
     using R = typename S::R;
@@ -127,6 +132,8 @@ k_step(const typename S::T* __restrict__ src, typename S::T* __restrict__ dst,
 
     // class bytes of the chunk: fast path if all are bulk (or, with FACES, face)
     bool special, face_chunk = false;
+    const bool pad = x0 >= g.nx;
+    const int xl = pad ? (g.nx - 1) / V * V : x0;     // a padding chunk repeats the row's last loads
     {
         const uint8_t* cp = cls + row * g.nxp + x0;
         unsigned long long cb;
@@ -180,7 +187,7 @@ k_step(const typename S::T* __restrict__ src, typename S::T* __restrict__ dst,
         for (int a = 0; a < Q; ++a) {
             const T* rp = src + (long long)a * g.sq + roff[EY<Q>(a) + 1][EZ<Q>(a) + 1];
             VecN<T, V> raw;
-            raw.raw = __ldg(reinterpret_cast<const RawT*>(rp + x0));
+            raw.raw = __ldg(reinterpret_cast<const RawT*>(rp + xl));
             const int ex = EX<Q>(a);
             T edge = raw.e[0];
             // periodic x: the wrap of a row edge and the warp edge are plain loads
@@ -236,7 +243,7 @@ k_step(const typename S::T* __restrict__ src, typename S::T* __restrict__ dst,
         for (int a = 0; a < Q; ++a) {
             int rwall = 0;
             const bool rout = row_out<Q>(fi, a, rwall);
-            raw[a].raw = __ldg(reinterpret_cast<const RawT*>(row_ptr(a, rout) + x0));
+            raw[a].raw = __ldg(reinterpret_cast<const RawT*>(row_ptr(a, rout) + xl));
         }
         // lanes at a warp edge or a row edge load the element the shuffle
         // cannot give them: the left neighbour of x0 (E_x = +1) or the right
@@ -304,8 +311,6 @@ k_step(const typename S::T* __restrict__ src, typename S::T* __restrict__ dst,
             }
         }
     }
-    // only the velocity rows of insulating walls need the lanes past the last chunk
-    if (!(EXT && FULL) && !active) return;
     // insulating walls: this thread's sum of the flow velocity v over the
     // fluid nodes it relaxes, summed over the warp by a fixed shuffle tree in
     // FP64 (every thread of the block reaches it, inactive ones with zero),
@@ -332,7 +337,7 @@ k_step(const typename S::T* __restrict__ src, typename S::T* __restrict__ dst,
             }
         }
     };
-    if (active) {
+    if (active && !special) {
 
         // Ladd terms of moving face walls, added after unpacking (face chunks only)
         const bool ladd = FACES && face_chunk && p.face_ladd;
@@ -345,7 +350,7 @@ k_step(const typename S::T* __restrict__ src, typename S::T* __restrict__ dst,
                     if (EX<Q>(a) == 1 && x0 + k == 0) { hit = true; wall = fi.wx_lo; }
                     if (EX<Q>(a) == -1 && x0 + k == g.nx - 1) { hit = true; wall = fi.wx_hi; }
                 }
-                if (hit) d[a] += ladd_of<Q, R>(p, a, wall);
+                if (hit) d[a] = ladd_on<Q, R>(d[a], p, a, wall);
             }
         };
 
@@ -362,8 +367,8 @@ k_step(const typename S::T* __restrict__ src, typename S::T* __restrict__ dst,
                     if (EX<Q>(a) == -1 && x0 + k == g.nx - 1) { h0 = true; w0 = fi.wx_hi; }
                     if (EX<Q>(a) == -1 && x0 + k + 1 == g.nx - 1) { h1 = true; w1 = fi.wx_hi; }
                 }
-                if (h0) d[a].v.x += ladd_of<Q, R>(p, a, w0);
-                if (h1) d[a].v.y += ladd_of<Q, R>(p, a, w1);
+                if (h0) d[a].v.x = ladd_on<Q, R>(d[a].v.x, p, a, w0);
+                if (h1) d[a].v.y = ladd_on<Q, R>(d[a].v.y, p, a, w1);
             }
         };
         // two nodes at a time in packed FP32x2 arithmetic (FP32 compute without
@@ -375,7 +380,7 @@ k_step(const typename S::T* __restrict__ src, typename S::T* __restrict__ dst,
     constexpr bool PAIRX = StepOcc<S, EXT, FACES, FULL, LP>::PAIRX;
 
         const long long base = row * g.nxp + x0;
-        if (!special) {
+        {
             if constexpr (PACKED && (PAIR2 || PAIRX)) {
 #pragma unroll
                 for (int i = 0; i < V / 2; ++i) {
@@ -518,33 +523,44 @@ k_step(const typename S::T* __restrict__ src, typename S::T* __restrict__ dst,
                     *reinterpret_cast<typename RawVec<sizeof(T) * V>::type*>(dst + (long long)a * g.sq + base) = o.raw;
                 }
             }
-        } else {
-            // chunk with a solid neighbour or padding: node by node
-            for (int k = 0; k < V; ++k) {
-                const int x = x0 + k;
-                const uint8_t c = cls[base + k];
-                if (x >= g.nx || nc_solid(c) || c == NC_PAD) {
-#pragma unroll
-                    for (int a = 0; a < Q; ++a) dst[(long long)a * g.sq + base + k] = S::from_raw(R(0));
-                    continue;
-                }
-                R d[Q];
-                gather_node<Q, S, true, FULL>(src, cls, g, p, x, y, z, d);
-                NodeM<R> m;
-                node_macro<R, Q, EXT, FULL>(d, p, m);
-                node_relax<R, Q, EXT>(d, p, m);
-                add_v(m);
-                if constexpr (SR) {
-                    NodeRng rng((uint32_t)(base + k), seed);
-#pragma unroll
-                    for (int a = 0; a < Q; ++a) dst[(long long)a * g.sq + base + k] = S::from_raw_sr(d[a], rng.bits(a));
-                } else {
-#pragma unroll
-                    for (int a = 0; a < Q; ++a) dst[(long long)a * g.sq + base + k] = S::from_raw(d[a]);
-                }
-            }
         }
     }
+    // the warp's chunks with a solid neighbour or padding, one node per lane
+    const unsigned todo = __ballot_sync(0xffffffffu, active && special && !pad);
+    for (int i = lane; i < V * __popc(todo); i += 32) {
+        unsigned rest = todo;
+        for (int k = i / V; k > 0; --k) rest &= rest - 1;      // the (i / V)-th special chunk
+        const unsigned sch = (unsigned)(tid - lane) + (unsigned)__ffs(rest) - 1u;
+        const unsigned sr = sch / (unsigned)ncx;
+        const int sx = (int)(sch - sr * (unsigned)ncx) * V + i % V;
+        const int sz = (int)(sr / (unsigned)g.ny), sy = (int)(sr - (unsigned)sz * (unsigned)g.ny);
+        const long long n = (long long)sr * g.nxp + sx;
+        const uint8_t c = cls[n];
+        if (nc_solid(c) || c == NC_PAD) {
+#pragma unroll
+            for (int a = 0; a < Q; ++a) dst[(long long)a * g.sq + n] = S::from_raw(R(0));
+            continue;
+        }
+        R d[Q];
+        if (FULL && g.phi && c == NC_BOUND) gather_node<Q, S, true, true>(src, cls, g, p, sx, sy, sz, d);
+        else pull_walls<Q, S, true>(src, cls, g, p, Around<Q>(g, sx, sy, sz), d);
+        NodeM<R> m;
+        node_macro<R, Q, EXT, FULL>(d, p, m);
+        node_relax<R, Q, EXT>(d, p, m);
+        add_v(m);
+        if constexpr (SR) {
+            NodeRng rng((uint32_t)n, seed);
+#pragma unroll
+            for (int a = 0; a < Q; ++a) dst[(long long)a * g.sq + n] = S::from_raw_sr(d[a], rng.bits(a));
+        } else {
+#pragma unroll
+            for (int a = 0; a < Q; ++a) dst[(long long)a * g.sq + n] = S::from_raw(d[a]);
+        }
+    }
+    if (zero_pad && active && pad)
+        for (int a = 0; a < Q; ++a)
+            *reinterpret_cast<RawT*>(dst + (long long)a * g.sq + row * g.nxp + x0) = RawT{};
+    __syncwarp();
     put_v();
 }
 
@@ -577,35 +593,89 @@ __device__ __forceinline__ float add_split(float d, float hi, float lo)
 }
 
 // ------------------------------------------ inverse propagation (import/init)
-// Stored state P with gather(P) = the given canonical f: P_a(y) = f_a(y + E_a)
-// if y + E_a is fluid, else f_opp(a)(y) - (Ladd term of opp(a)).
+// Stored state P with gather(P) = the given canonical f: every node stores its
+// own populations where its pulls read them (push_node), so a node's values
+// are formed once.  The sources give one value (src_value, for walls off the
+// half-grid) or all of a node's (node_values).
 struct SrcCanonD { const double* f; long long N; };
 struct SrcCanonF { const float* f; long long N; };
-struct SrcFields { const double* rho; const double* u; const double* xi; long long N; };
+struct SrcFields { const double* rho; const double* u; const double* xi; long long N; double ic; };   // ic = 1 / c
 
-template <int Q, typename R>
-__device__ __forceinline__ R src_value(const SrcCanonD& s, const KP<R>& p, int a, long long n)
+// the deviations f_a - w_a rho0 of node n
+template <int Q, typename R, class Src>
+__device__ __forceinline__ void node_values(const Src& s, const KP<R>&, const WRho& wr, long long n, R (&d)[Q])
 {
-    return R(s.f[(long long)a * s.N + n] - WD<Q>(a) * (double)p.rho0);
+    std::remove_cv_t<std::remove_pointer_t<decltype(s.f)>> f[Q];
+#pragma unroll
+    for (int a = 0; a < Q; ++a) f[a] = s.f[(long long)a * s.N + n];
+#pragma unroll
+    for (int a = 0; a < Q; ++a) {
+        const int k = SPEED2<Q>(a);
+        if constexpr (sizeof(R) == 4 && sizeof(f[0]) == 4) d[a] = add_split(f[a], -wr.hi[k], -wr.lo[k]);
+        else d[a] = R((double)f[a] - wr.c[k]);
+    }
 }
+// Eq. (1) (+ Eq. 10) in FP64, times 1 + xi.  The FP64 pipe bounds it (1.7
+// lanes per cycle and SM), so the node's terms are shared: with m = 3 rho W
+// and q_k = m_k W_k, an opposite pair is w (even +- odd), odd = E.m and
+// even = rho - rho0 - sum q / 2 + 3/2 (E.m)(E.W), the last product
+// q_i + q_j +- 2 m_i W_j for a diagonal pair: 67 operations a node.
 template <int Q, typename R>
-__device__ __forceinline__ R src_value(const SrcCanonF& s, const KP<R>& p, int a, long long n)
+__device__ __forceinline__ void node_values(const SrcFields& s, const KP<R>& p, const WRho& wr, long long n, R (&d)[Q])
 {
-    return R((double)s.f[(long long)a * s.N + n] - WD<Q>(a) * (double)p.rho0);
-}
-// Eq. (1) (+ Eq. 10) evaluated in double from the fields, times (1 + xi)
-template <int Q, typename R>
-__device__ __forceinline__ R src_value(const SrcFields& s, const KP<R>& p, int a, long long n)
-{
-    const double c = (double)p.c;
+    constexpr int D = LatDim<Q>::D;
     const double rho = s.rho[n];
-    const double W[3] = {s.u[n] / c, s.u[s.N + n] / c, (Q == 19) ? s.u[2 * s.N + n] / c : 0.0};
-    const double eu = EX<Q>(a) * W[0] + EY<Q>(a) * W[1] + EZ<Q>(a) * W[2];
-    const double ww = W[0] * W[0] + W[1] * W[1] + W[2] * W[2];
-    double fe = p.stokes ? rho * WD<Q>(a) * (1.0 + 3.0 * eu) : rho * WD<Q>(a) * (1.0 + 3.0 * eu + 4.5 * eu * eu - 1.5 * ww);
-    if (p.maxwell) fe += (double)p.mx[a];
-    if (s.xi) fe *= 1.0 + s.xi[(long long)a * s.N + n];
-    return R(fe - WD<Q>(a) * (double)p.rho0);
+    double W[3], m[3], q[3], sq = 0.0;
+#pragma unroll
+    for (int k = 0; k < D; ++k) W[k] = s.u[(long long)k * s.N + n] * s.ic;
+#pragma unroll
+    for (int k = 0; k < D; ++k) {
+        m[k] = 3.0 * rho * W[k];
+        q[k] = m[k] * W[k];
+        sq += q[k];
+    }
+    const double h = p.stokes ? 0.0 : 1.5;       // the linear equilibrium drops the quadratic terms
+    const double base = fma(-h / 3.0, sq, rho - (double)p.rho0);
+    auto put = [&](int a, double v) {
+        if (p.maxwell) v += (double)p.mx[a];
+        if (s.xi) v = fma(v + wr.c[SPEED2<Q>(a)], s.xi[(long long)a * s.N + n], v);
+        d[a] = R(v);
+    };
+    put(0, WD<Q>(0) * base);
+#pragma unroll
+    for (int k = 0; k < LatDim<Q>::NP; ++k) {
+        const int a = PAIR<Q>(k), b = OPP<Q>(a);
+        const double w = WD<Q>(a);
+        const int e[3] = {EX<Q>(a), EY<Q>(a), EZ<Q>(a)};
+        double em = 0.0, eq = 0.0, mw = 0.0;     // E.m, the q_k of its axes, m_i W_j signed
+        int first = -1;
+#pragma unroll
+        for (int c = 0; c < D; ++c) {
+            if (!e[c]) continue;
+            if (first < 0) {
+                em = e[c] > 0 ? m[c] : -m[c];
+                eq = q[c];
+                first = c;
+            } else {
+                em = e[c] > 0 ? em + m[c] : em - m[c];
+                eq += q[c];
+                mw = e[first] * e[c] > 0 ? m[first] * W[c] : -(m[first] * W[c]);
+            }
+        }
+        double even = fma(h * w, eq, w * base);
+        if (SPEED2<Q>(a) == 2) even = fma(2.0 * h * w, mw, even);
+        put(a, fma(w, em, even));
+        put(b, fma(-w, em, even));
+    }
+}
+
+// one of them (a is a constant: the others' terms are dropped)
+template <int Q, typename R, class Src>
+__device__ __forceinline__ R src_value(const Src& s, const KP<R>& p, const WRho& wr, int a, long long n)
+{
+    R d[Q];
+    node_values<Q, R>(s, p, wr, n, d);
+    return d[a];
 }
 
 // canonical index of a fluid node given by its padded index
@@ -621,13 +691,12 @@ __device__ __forceinline__ long long canon_of(const Geo& g, long long padded)
 // interpolated rule.  Every case is explicit except both opposite links of
 // x hitting solids with q >= 1/2, a 2 x 2 solve.
 template <int Q, typename R, class Src>
-__device__ R unbounced(const Src& s, const KP<R>& p, const Geo& g, const uint8_t* __restrict__ cls, int x, int y, int z,
+__device__ R unbounced(const Src& s, const KP<R>& p, const WRho& wr, const Geo& g, const uint8_t* __restrict__ cls, int x, int y, int z,
                        long long own, long long nd, int a, int wall)
 {
     const int b = OPP<Q>(a);
-    const R Lb = R(WD<Q>(b)) * (R(EX<Q>(b)) * p.LW[wall][0] + R(EY<Q>(b)) * p.LW[wall][1] + R(EZ<Q>(b)) * p.LW[wall][2]);
-    const R fb = src_value<Q, R>(s, p, b, nd);
-    const R half = fb - Lb;
+    const R fb = src_value<Q, R>(s, p, wr, b, nd);
+    const R half = ladd_off<Q, R>(fb, p, b, wall);
     if (!g.phi) return half;
     const long long sa = link_target(g, x, y, z, EX<Q>(a), EY<Q>(a), EZ<Q>(a));
     if (sa < 0 || !nc_solid(cls[sa])) return half;               // a closed box face
@@ -637,66 +706,72 @@ __device__ R unbounced(const Src& s, const KP<R>& p, const Geo& g, const uint8_t
     const bool b_fluid = pull_source(g, cls, x, y, z, EX<Q>(a), EY<Q>(a), EZ<Q>(a), nb, wb);   // x + E_b = x - E_a
     if (qa < R(0.5)) {
         if (!b_fluid) return half;
-        const R fa = src_value<Q, R>(s, p, a, nd);                // = P_a(x - E_a)
-        return (fb - Lb - (R(1) - R(2) * qa) * fa) / (R(2) * qa);
+        const R fa = src_value<Q, R>(s, p, wr, a, nd);                // = P_a(x - E_a)
+        return (half - (R(1) - R(2) * qa) * fa) / (R(2) * qa);
     }
     R Pb;
     if (b_fluid) {
-        Pb = src_value<Q, R>(s, p, b, canon_of(g, nb));           // node x + E_b pulls b from x
-        return R(2) * qa * fb - (R(2) * qa - R(1)) * Pb - Lb;
+        Pb = src_value<Q, R>(s, p, wr, b, canon_of(g, nb));           // node x + E_b pulls b from x
+        return ladd_off<Q, R>(R(2) * qa * fb - (R(2) * qa - R(1)) * Pb, p, b, wall);
     }
     // the link b of x hits a wall too (wall id wb)
-    const R La = R(WD<Q>(a)) * (R(EX<Q>(a)) * p.LW[wb][0] + R(EY<Q>(a)) * p.LW[wb][1] + R(EZ<Q>(a)) * p.LW[wb][2]);
-    const R fa = src_value<Q, R>(s, p, a, nd);
+    const R fa = src_value<Q, R>(s, p, wr, a, nd);
     const long long sb = link_target(g, x, y, z, EX<Q>(b), EY<Q>(b), EZ<Q>(b));
     const R qb = (sb >= 0 && nc_solid(cls[sb])) ? R(g.phi[own]) / (R(g.phi[own]) - R(g.phi[sb])) : R(0.5);
     if (qb < R(0.5) || !(sb >= 0 && nc_solid(cls[sb]))) {
         // b bounces halfway (its second node x + E_a is the solid, or a face)
-        Pb = fa - La;
-        return R(2) * qa * fb - (R(2) * qa - R(1)) * Pb - Lb;
+        Pb = ladd_off<Q, R>(fa, p, a, wb);
+        return ladd_off<Q, R>(R(2) * qa * fb - (R(2) * qa - R(1)) * Pb, p, b, wall);
     }
-    const R A1 = R(2) * qa * fb - Lb, k1 = R(2) * qa - R(1);
-    const R A2 = R(2) * qb * fa - La, k2 = R(2) * qb - R(1);
+    const R A1 = ladd_off<Q, R>(R(2) * qa * fb, p, b, wall), k1 = R(2) * qa - R(1);
+    const R A2 = ladd_off<Q, R>(R(2) * qb * fa, p, a, wb), k2 = R(2) * qb - R(1);
     return (A1 - k1 * A2) / (R(1) - k1 * k2);
 }
 
-template <int Q, class S, class Src>
+// one padded node per thread.  Before (each node pulling its 18 neighbours'
+// values, with their equilibria in FP64) a 192^3 binary16 box took 12.2 ms
+// from fields and 1.04 ms from FP32 populations; so 2.25 ms (the FP64 pipe)
+// and 0.225 ms (0.53 of the copy bandwidth).
+template <int Q, class S, class Src, bool CURVED>
 __global__ void __launch_bounds__(NODE_THREADS)
 k_inverse_stream(typename S::T* __restrict__ P, const uint8_t* __restrict__ cls, const Geo g,
-                 const KP<typename S::R> p, const Src s)
+                 const KP<typename S::R> p, const WRho wr, const Src s)
 {
     using R = typename S::R;
-    for (long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x; n < (long long)g.nxp * g.ny * g.nz;
-         n += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(n % g.nxp);
-        const long long r = n / g.nxp;
-        const int y = (int)(r % g.ny), z = (int)(r / g.ny);
-        const uint8_t c = cls[n];
-        if (x >= g.nx || nc_solid(c) || c == NC_PAD) {
+    const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (n >= g.sq) return;
+    const unsigned r = (unsigned)n / (unsigned)g.nxp;
+    const int x = (int)((unsigned)n - r * (unsigned)g.nxp);
+    const int z = (int)(r / (unsigned)g.ny), y = (int)(r - (unsigned)z * (unsigned)g.ny);
+    const uint8_t c = cls[n];
+    if (x >= g.nx || nc_solid(c) || c == NC_PAD) {
 #pragma unroll
-            for (int a = 0; a < Q; ++a) P[(long long)a * g.sq + n] = S::from_r(R(0));
-            continue;
-        }
-        const long long nd = ((long long)z * g.ny + y) * g.nx + x;
+        for (int a = 0; a < Q; ++a) P[(long long)a * g.sq + n] = S::from_r(R(0));
+        return;
+    }
+    const long long nd = (long long)r * g.nx + x;
+    R d[Q];
+    node_values<Q, R>(s, p, wr, nd, d);
+    if constexpr (CURVED) {
+        if (c == NC_BOUND) {
+            // walls off the half-grid: a link's value solves the interpolation
 #pragma unroll
-        for (int a = 0; a < Q; ++a) {
-            // the link from y along a is the pull source of direction opp(a) at y
-            long long srcp;
-            int wall;
-            R val;
-            if (a == 0) {
-                val = src_value<Q, R>(s, p, 0, nd);
-            } else if (pull_source(g, cls, x, y, z, EX<Q>(OPP<Q>(a)), EY<Q>(OPP<Q>(a)), EZ<Q>(OPP<Q>(a)), srcp, wall)) {
-                const int xs = (int)(srcp % g.nxp);
-                const long long rs = srcp / g.nxp;
-                const long long ns = rs * g.nx + xs;
-                val = src_value<Q, R>(s, p, a, ns);
-            } else {
-                val = unbounced<Q, R>(s, p, g, cls, x, y, z, n, nd, a, wall);
+            for (int a = 0; a < Q; ++a) {
+                // the link along a is the pull source of direction opp(a); the
+                // neighbour's population a, if fluid, is its to store
+                long long srcp;
+                int wall;
+                if (a == 0) P[n] = S::from_r(d[0]);
+                else if (pull_source(g, cls, x, y, z, EX<Q>(a), EY<Q>(a), EZ<Q>(a), srcp, wall))
+                    P[(long long)a * g.sq + srcp] = S::from_r(d[a]);
+                else
+                    P[(long long)OPP<Q>(a) * g.sq + n] =
+                        S::from_r(unbounced<Q, R>(s, p, wr, g, cls, x, y, z, n, nd, OPP<Q>(a), wall));
             }
-            P[(long long)a * g.sq + n] = S::from_r(val);
+            return;
         }
     }
+    push_node<Q, S>(P, cls, g, p, c, x, y, z, d);
 }
 
 // ---------------------------------------------------------------- export
@@ -1316,36 +1391,44 @@ template <class S> inline KP<typename S::R> kp_links_of(const Ctx& c)
     return with_mag(kp_of<S>(c), c.cfg.induced ? c.mag[1 - c.cur] : nullptr);
 }
 
+// whether a step into dst also zeroes the padding: in a buffer that is not
+// the context's own (theirs is zero from create on)
+inline int zero_padding(const Ctx& c, const void* dst)
+{
+    return c.geo.nxp > c.geo.nx && dst != c.pop[0] && dst != c.pop[1];
+}
+
 template <int Q, class S, bool EXT, bool SR>
 cudaError_t launch_step_q(const Ctx& c, const void* src, void* dst, uint32_t seed, cudaStream_t st)
 {
     using T = typename S::T;
     const long long nch = (long long)(c.geo.nxp / S::V) * c.geo.ny * c.geo.nz;
     const int blocks = grid_for(nch, STEP_THREADS, 1ll << 31);
+    const int zp = zero_padding(c, dst);
     const bool faces = !c.geo.periodic[0] || !c.geo.periodic[1] || (Q == 19 && !c.geo.periodic[2]);
     if constexpr (EXT && sizeof(typename S::T) == 2) {
         if (c.les_pair) {
             if (faces)
                 k_step<Q, S, EXT, true, SR, false, true><<<blocks, STEP_THREADS, 0, st>>>(
-                    (const T*)src, (T*)dst, c.cls, c.geo, kp_step_of<S>(c), seed);
+                    (const T*)src, (T*)dst, c.cls, c.geo, kp_step_of<S>(c), seed, zp);
             else
                 k_step<Q, S, EXT, false, SR, false, true><<<blocks, STEP_THREADS, 0, st>>>(
-                    (const T*)src, (T*)dst, c.cls, c.geo, kp_step_of<S>(c), seed);
+                    (const T*)src, (T*)dst, c.cls, c.geo, kp_step_of<S>(c), seed, zp);
             return cudaGetLastError();
         }
     }
     if ((c.cfg.curved || c.insulating) && faces)
         k_step<Q, S, EXT, true, SR, true><<<blocks, STEP_THREADS, 0, st>>>((const T*)src, (T*)dst, c.cls, c.geo,
-                                                                           kp_step_of<S>(c), seed);
+                                                                           kp_step_of<S>(c), seed, zp);
     else if (c.cfg.curved || c.insulating)
         k_step<Q, S, EXT, false, SR, true><<<blocks, STEP_THREADS, 0, st>>>((const T*)src, (T*)dst, c.cls, c.geo,
-                                                                            kp_step_of<S>(c), seed);
+                                                                            kp_step_of<S>(c), seed, zp);
     else if (faces)
         k_step<Q, S, EXT, true, SR><<<blocks, STEP_THREADS, 0, st>>>((const T*)src, (T*)dst, c.cls, c.geo,
-                                                                     kp_step_of<S>(c), seed);
+                                                                     kp_step_of<S>(c), seed, zp);
     else
         k_step<Q, S, EXT, false, SR><<<blocks, STEP_THREADS, 0, st>>>((const T*)src, (T*)dst, c.cls, c.geo,
-                                                                      kp_step_of<S>(c), seed);
+                                                                      kp_step_of<S>(c), seed, zp);
     return cudaGetLastError();
 }
 
@@ -1364,9 +1447,10 @@ cudaError_t launch_step_staged_k(const Ctx& c, const void* src, void* dst, uint3
         if (e != cudaSuccess) return e;
         c.stage_ready = true;
     }
-    kern<<<staged_blocks(c), STG_THREADS, c.stage_smem, st>>>((const T*)src, (T*)dst, c.cls, c.special, c.n_special,
+    kern<<<staged_blocks(c), 32 * (STG_CWARPS + 1 + staged_bwarps(c.n_special, c.geo.sq)), c.stage_smem, st>>>((const T*)src, (T*)dst, c.cls, c.special, c.n_special,
                                                               c.geo, kp_step_of<S>(c), seed, c.stage_R,
-                                                              c.stage_tiles, c.stage_n, c.errflag, fw);
+                                                              c.stage_tiles, c.stage_n, zero_padding(c, dst), c.errflag,
+                                                              fw);
     return cudaGetLastError();
 }
 
@@ -1426,33 +1510,31 @@ template <class F> inline cudaError_t with_ext_curved(const Ctx& c, F&& f)
     });
 }
 
+template <int Q, class S, class Src>
+cudaError_t launch_inverse(const Ctx& c, const Src& src, void* dst, cudaStream_t st)
+{
+    const int blocks = grid_for(c.geo.sq, NODE_THREADS, 1ll << 31);
+    const WRho wr = wrho_of<Q>((double)kp_of<S>(c).rho0);
+    return with_curved(c, [&](auto cu) {
+        k_inverse_stream<Q, S, Src, cu.value><<<blocks, NODE_THREADS, 0, st>>>((typename S::T*)dst, c.cls, c.geo,
+                                                                               kp_of<S>(c), wr, src);
+    });
+}
+
 template <int Q, class S>
 cudaError_t launch_import(const Ctx& c, const void* srcf, int dtype, void* dst, cudaStream_t st)
 {
-    using T = typename S::T;
-    const long long NP = (long long)c.geo.nxp * c.geo.ny * c.geo.nz;
-    const int blocks = grid_for(NP, NODE_THREADS, 65535ll * 16);
     const long long N = (long long)c.geo.nx * c.geo.ny * c.geo.nz;
-    if (dtype == 0)
-        k_inverse_stream<Q, S, SrcCanonD><<<blocks, NODE_THREADS, 0, st>>>((T*)dst, c.cls, c.geo, kp_of<S>(c),
-                                                                          SrcCanonD{(const double*)srcf, N});
-    else
-        k_inverse_stream<Q, S, SrcCanonF><<<blocks, NODE_THREADS, 0, st>>>((T*)dst, c.cls, c.geo, kp_of<S>(c),
-                                                                          SrcCanonF{(const float*)srcf, N});
-    return cudaGetLastError();
+    return dtype == 0 ? launch_inverse<Q, S>(c, SrcCanonD{(const double*)srcf, N}, dst, st)
+                      : launch_inverse<Q, S>(c, SrcCanonF{(const float*)srcf, N}, dst, st);
 }
 
 template <int Q, class S>
 cudaError_t launch_init(const Ctx& c, const double* rho, const double* u, const double* xi, void* dst,
                         cudaStream_t st)
 {
-    using T = typename S::T;
-    const long long NP = (long long)c.geo.nxp * c.geo.ny * c.geo.nz;
-    const int blocks = grid_for(NP, NODE_THREADS, 65535ll * 16);
     const long long N = (long long)c.geo.nx * c.geo.ny * c.geo.nz;
-    k_inverse_stream<Q, S, SrcFields><<<blocks, NODE_THREADS, 0, st>>>((T*)dst, c.cls, c.geo, kp_of<S>(c),
-                                                                      SrcFields{rho, u, xi, N});
-    return cudaGetLastError();
+    return launch_inverse<Q, S>(c, SrcFields{rho, u, xi, N, 1.0 / c.kpd.c}, dst, st);
 }
 
 template <int Q, class S>
@@ -1485,6 +1567,8 @@ inline int red_grid(const Ctx& c, long long N, int& threads)
     return grid_for(N, threads, std::min<long long>(MAX_PARTIAL_ROWS, most));
 }
 
+// blocks of two warps spread 10^4 links over the SMs (FP64 sums of a block's
+// warps share one SM's FP64 pipe); from 65,536 links full blocks
 template <int Q, class S>
 cudaError_t launch_links(const Ctx& c, const void* P, long long begin, long long end, unsigned flags,
                          double* partials, int* nblocks, cudaStream_t st)

@@ -35,10 +35,10 @@
 // copies that row instead), the element outside a closed x face is the
 // node's own opposite population (the producer stages these face values),
 // and moving faces add Ladd's term.  The 4-node chunks that touch a solid
-// node, a wall or the padding are not the pipeline's: a boundary warp per
-// block takes its share of their list (built on the host) and computes them
-// node by node from global memory with explicit bounce-back, exactly as
-// k_step does, beside the pipeline -- inline, one such chunk held up its
+// node, a wall or the end of a ragged row are not the pipeline's: the
+// boundary warps take their share of their list (built on the host) and
+// compute them node by node from global memory with explicit bounce-back,
+// exactly as k_step does, beside the pipeline -- inline, one such chunk held up its
 // stage and with it the in-order producer (the sphere box ran at half the
 // rate of the same box without the sphere).  The arithmetic and the
 // stochastic rounding stream are those of k_step, so the two kernels store
@@ -56,7 +56,13 @@ namespace lbm {
 constexpr int STG_GROUPS = 2;                         // consumer groups (alternate tiles)
 constexpr int STG_GROUP_WARPS = 8;                    // warps per group
 constexpr int STG_CWARPS = STG_GROUPS * STG_GROUP_WARPS;
-constexpr int STG_THREADS = 32 * (STG_CWARPS + 2);    // plus the producer and the boundary warp
+// boundary warps: one, or three where more than 0.5% of the chunks are special
+// (a ragged row has one in every row): three is the most that still leaves
+// five warps on each of the SM's four sub-partitions, so the register cap of
+// 96 stays, and the kernel takes the number from its block size
+constexpr int STG_BWARPS = 3;
+constexpr int STG_THREADS = 32 * (STG_CWARPS + 1 + STG_BWARPS);    // plus the producer
+inline int staged_bwarps(long long n_special, long long nodes) { return n_special * 200 > nodes / 4 ? STG_BWARPS : 1; }
 constexpr int STG_COPY_BYTES = 2048;                  // least bytes per direction and tile
 constexpr int STG_TASK_NODES = 64;                    // nodes per warp task (32 pairs)
 constexpr int STG_MAX_STAGES = 8;
@@ -237,12 +243,12 @@ __device__ __forceinline__ float2 stg_pair(const typename S::T* __restrict__ row
 // (25) of the step that produced the stored state, summed over the links of
 // one wall (wall < 0: every wall) in FP64; null `out`: not asked for
 struct StgForce {
-    double* out;          // one row of 3 doubles per block, or null
+    double* out;          // one row of 3 doubles per boundary warp, or null
     int wall;
     unsigned flags;       // LBM_MOVING_CORR
     double c, rho0, svol; // physical units
     float lw[MAXW + 1][3];  // 6 rho0 u_w / c per wall id (physical units)
-    // the last block to write its row sums the rows (ticket: zero between
+    // the last warp to write its row sums the rows (ticket: zero between
     // launches) into result: result = (accumulate ? result : 0) + weight sum
     unsigned* ticket;
     double* result;
@@ -256,7 +262,9 @@ struct StgForce {
 // P_opp(b)(x) plus Ladd's term of the solid's wall.  Every load is issued
 // before any is used (one memory round trip for the boundary warps).  With
 // a force asked for, each link (x, a' = opp(b)) into a solid adds
-// (dx^D/dt) [e_a' (fbar_a' + fbar_b) (+ u_w (fbar_b - fbar_a'))] to acc, with
+// [e_a' (fbar_a' + fbar_b) (+ u_w (fbar_b - fbar_a'))] / c to acc (the FP64
+// pipe takes a warp instruction in ~19 cycles: the common factor c dx^D/dt
+// waits for the warp's sum), with
 // fbar_a' = f^rel_a'(x, T-1) and fbar_b = f_b(x, T) its bounced population,
 // as the link kernel of lbm_wall_force does.
 template <int Q, class S>
@@ -282,21 +290,19 @@ __device__ __forceinline__ void gather_periodic(const typename S::T* __restrict_
     for (int b = 1; b < Q; ++b) {
         if (nc_solid(cs[b])) {
             const int wall = nc_wall(cs[b]);
-            const R L = R(WD<Q>(b)) * (R(EX<Q>(b)) * p.LW[wall][0] + R(EY<Q>(b)) * p.LW[wall][1] +
-                                       R(EZ<Q>(b)) * p.LW[wall][2]);
-            d[b] = S::to_raw(bv[b]) + L;
+            d[b] = ladd_on<Q, R>(S::to_raw(bv[b]), p, b, wall);
             if (fw.out && (fw.wall < 0 || fw.wall == wall)) {
+                // e_a' (fbar_a' + fbar_b) in lattice units, scaled by the caller
                 const float* lw = fw.lw[wall];
                 const double w = WD<Q>(b);
                 const float Lp = (float)w * ((float)EX<Q>(b) * lw[0] + (float)EY<Q>(b) * lw[1] + (float)EZ<Q>(b) * lw[2]);
-                const double fo = (double)S::to_r(bv[b]) + w * fw.rho0;
-                const double fi = (double)(S::to_r(bv[b]) + Lp) + w * fw.rho0;
+                const double vo = (double)S::to_r(bv[b]), vi = (double)(S::to_r(bv[b]) + Lp);
+                const double s = vo + vi + 2.0 * w * fw.rho0;
                 const int e[3] = {-EX<Q>(b), -EY<Q>(b), -EZ<Q>(b)};     // e_a', a' = opp(b)
 #pragma unroll
                 for (int k = 0; k < 3; ++k) {
-                    double t = fw.c * e[k] * (fo + fi);
-                    if (fw.flags & 1u) t += (double)lw[k] * fw.c / (6.0 * fw.rho0) * (fi - fo);
-                    acc[k] += fw.svol * t;
+                    if (e[k]) acc[k] = e[k] > 0 ? acc[k] + s : acc[k] - s;
+                    if (fw.flags & 1u) acc[k] += (double)lw[k] / (6.0 * fw.rho0) * (vi - vo);
                 }
             }
         } else {
@@ -315,8 +321,8 @@ template <int Q, class S, bool SR, bool EXT = false, bool FACES = false, bool LP
 __global__ void __launch_bounds__(STG_THREADS, 1)
 k_step_staged(const typename S::T* __restrict__ src, typename S::T* __restrict__ dst,
               const uint8_t* __restrict__ cls, const uint32_t* __restrict__ special, long long nspecial, const Geo g,
-              const KP<float> p, uint32_t seed, int R, int ntiles, int nstages, unsigned* __restrict__ errflag,
-              const StgForce fw)
+              const KP<float> p, uint32_t seed, int R, int ntiles, int nstages, int zero_pad,
+              unsigned* __restrict__ errflag, const StgForce fw)
 {
     using T = typename S::T;
     using Rt = typename S::R;
@@ -377,13 +383,23 @@ k_step_staged(const typename S::T* __restrict__ src, typename S::T* __restrict__
         return;
     }
 
-    if (warp == STG_CWARPS + 1) {
-        // boundary warp: the listed chunks, node by node (lane per node), and
+    if (warp > STG_CWARPS) {
+        // boundary warps: the listed chunks, node by node (lane per node), and
         // the wall force of their links when asked for (each lane sums its
-        // nodes in a fixed order, then a fixed shuffle tree, one row per block)
+        // nodes in a fixed order, then a fixed shuffle tree, one row per warp)
         double acc[3] = {0.0, 0.0, 0.0};
         const long long nn = 4 * nspecial;
-        for (long long j = (long long)blockIdx.x * 32 + lane; j < nn; j += (long long)gridDim.x * 32) {
+        const int per = (int)(blockDim.x >> 5) - STG_CWARPS - 1;          // boundary warps of a block
+        const int bw = (int)blockIdx.x * per + warp - STG_CWARPS - 1, nbw = (int)gridDim.x * per;
+        if (zero_pad) {
+            // a destination that is not the context's own: zero its padding
+            // (the special chunks cover the rest of a row's last chunk)
+            const int x1 = (g.nx + 3) & ~3;
+            const long long rows = (long long)Q * g.ny * g.nz;
+            for (long long r = (long long)bw * 32 + lane; r < rows; r += (long long)nbw * 32)
+                for (int xx = x1; xx < g.nxp; ++xx) dst[r * g.nxp + xx] = S::from_raw(Rt(0));
+        }
+        for (long long j = (long long)bw * 32 + lane; j < nn; j += (long long)nbw * 32) {
             const long long node = (long long)special[j >> 2] + (j & 3);
             const int x = (int)(node % g.nxp);
             const long long row = node / g.nxp;
@@ -395,7 +411,7 @@ k_step_staged(const typename S::T* __restrict__ src, typename S::T* __restrict__
                 continue;
             }
             Rt d[Q];
-            if constexpr (FACES) gather_node<Q, S, true, false>(src, cls, g, p, x, y, z, d);
+            if constexpr (FACES) pull_walls<Q, S, true>(src, cls, g, p, Around<Q>(g, x, y, z), d);
             else gather_periodic<Q, S>(src, cls, g, p, x, y, z, node, d, fw, acc);
             NodeM<Rt> m;
             node_macro<Rt, Q, EXT, false>(d, p, m);
@@ -412,23 +428,24 @@ k_step_staged(const typename S::T* __restrict__ src, typename S::T* __restrict__
         if (!FACES && fw.out) {
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
+                acc[k] *= fw.svol * fw.c;
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) acc[k] += __shfl_down_sync(0xffffffffu, acc[k], o);
-                if (lane == 0) fw.out[(long long)blockIdx.x * 3 + k] = acc[k];
+                if (lane == 0) fw.out[(long long)bw * 3 + k] = acc[k];
             }
-            // the last block's boundary warp sums the rows: lane l takes rows
+            // the last boundary warp sums the rows: lane l takes rows
             // l, l+32, ..., then a fixed shuffle tree (the order of the
             // library's fixed-order pass), and clears the ticket
             __threadfence();
             unsigned last = 0;
-            if (lane == 0) last = (atomicAdd(fw.ticket, 1u) == gridDim.x - 1) ? 1u : 0u;
+            if (lane == 0) last = (atomicAdd(fw.ticket, 1u) == (unsigned)nbw - 1u) ? 1u : 0u;
             last = __shfl_sync(0xffffffffu, last, 0);
             if (last) {
                 __threadfence();
 #pragma unroll
                 for (int k = 0; k < 3; ++k) {
                     double sum = 0.0;
-                    for (int r = lane; r < (int)gridDim.x; r += 32) sum += __ldcg(fw.out + (long long)r * 3 + k);
+                    for (int r = lane; r < nbw; r += 32) sum += __ldcg(fw.out + (long long)r * 3 + k);
 #pragma unroll
                     for (int o = 16; o > 0; o >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, o);
                     if (lane == 0) fw.result[k] = (fw.accumulate ? fw.result[k] : 0.0) + fw.weight * sum;
@@ -500,8 +517,8 @@ k_step_staged(const typename S::T* __restrict__ src, typename S::T* __restrict__
                         if (EX<Q>(a) == -1 && x0 == g.nx - 1) { h0 = true; w0 = fi.wx_hi; }
                         if (EX<Q>(a) == -1 && x0 + 1 == g.nx - 1) { h1 = true; w1 = fi.wx_hi; }
                     }
-                    if (h0) dd[a].v.x += ladd_of<Q, float>(p, a, w0);
-                    if (h1) dd[a].v.y += ladd_of<Q, float>(p, a, w1);
+                    if (h0) dd[a].v.x = ladd_on<Q, float>(dd[a].v.x, p, a, w0);
+                    if (h1) dd[a].v.y = ladd_on<Q, float>(dd[a].v.y, p, a, w1);
                 }
             }
             if constexpr (!EXT || LP || PAIRX) {
