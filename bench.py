@@ -100,7 +100,7 @@ def peaks():
 
 # sources that compile into the step kernel (host code, the adjoint and the
 # allocation-free wall force are left out)
-STEP_SOURCES = ("lbm_device.cuh", "lbm_kernels.cuh", "lbm_staged.cuh", "lbm_internal.h",
+STEP_SOURCES = ("lbm_device.cuh", "lbm_kernels.cuh", "lbm_staged.cuh", "lbm_step64.cuh", "lbm_internal.h",
                 *(f"inst_{s}_{q}.cu" for s in ("f64", "f32", "f16", "bf16") for q in ("d2q9", "d3q19")))
 
 

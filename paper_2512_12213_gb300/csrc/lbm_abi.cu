@@ -224,18 +224,13 @@ void count_links(const lbm_config* c, const uint8_t* wid, long long* per_wall /*
     *n_special = (long long)special_chunks(cls).size();
 }
 
-// threads of the register-tiled step kernel: one per vector chunk
-long long step_threads_of(const lbm_config* c)
-{
-    const int V = (c->storage == LBM_STORE_F64) ? 2 : 4;
-    return (long long)(pitch_of(c->nx) / V) * c->ny * c->nz;
-}
-
-// insulating walls: one velocity-sum row per warp of the step grid (blocks of
-// 128 threads; the warps past the last chunk write zero rows)
+// insulating walls: the step's velocity-sum rows: FP64 one per 64 nodes; else
+// one per warp of the step grid, a vector of 4 nodes per thread in blocks of
+// 128 (the warps past the last vector write zero rows)
 long long ins_rows_of(const lbm_config* c)
 {
-    return (step_threads_of(c) + 127) / 128 * 4;
+    const long long sq = (long long)pitch_of(c->nx) * c->ny * c->nz;
+    return c->storage == LBM_STORE_F64 ? sq / 64 : (sq / 4 + 127) / 128 * 4;
 }
 
 // contexts that may run the staged step keep the list of special chunks in
@@ -311,6 +306,7 @@ template <typename R> void cast_kp(const KP<double>& s, KP<R>& d)
     for (int k = 0; k < 3; ++k) {
         d.ueq_c[k] = (R)s.ueq_c[k];
         d.uf_c[k] = (R)s.uf_c[k];
+        d.cA[k] = (R)s.cA[k];
     }
     d.uf_u = (R)s.uf_u;
     d.Cf = (R)s.Cf;
@@ -337,6 +333,7 @@ template <int Q> void pair_consts(KP<double>& p)
     }
     p.uf_u = (p.model == MODEL_A) ? 0.0 : 1.0;
     p.Cf = (p.model == MODEL_E) ? 1.0 - h * p.om0 : 1.0;
+    for (int k = 0; k < 3; ++k) p.cA[k] = (p.model == MODEL_A) ? 0.0 : 2.0 * p.Cf * p.AG[k];
     for (int a = 0; a < 19; ++a) {
         p.pe[a] = (a < Q) ? EX<Q>(a) * p.AG[0] + EY<Q>(a) * p.AG[1] + EZ<Q>(a) * p.AG[2] : 0.0;
         p.peq[a] = (a < Q) ? EX<Q>(a) * p.ueq_c[0] + EY<Q>(a) * p.ueq_c[1] + EZ<Q>(a) * p.ueq_c[2] : 0.0;

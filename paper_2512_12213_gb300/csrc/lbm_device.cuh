@@ -277,6 +277,7 @@ template <typename R> struct KP {
     // E_a . ueq_c = peq[a], E_a . uf_c = pf[a]
     R ueq_c[3], uf_u, uf_c[3], Cf;
     R pe[19], peq[19], pf[19];
+    R cA[3];          // 2 C A for models whose force has a quadratic part (all but [a]), else 0
     // insulating walls: the force coefficient dt sigma_e (E x B) / c of the
     // current field, kept on the device (replaces AEB), and the per-thread
     // rows of the step kernel's flow-velocity sums; null otherwise

@@ -1398,6 +1398,12 @@ inline int zero_padding(const Ctx& c, const void* dst)
     return c.geo.nxp > c.geo.nx && dst != c.pop[0] && dst != c.pop[1];
 }
 
+}  // namespace lbm
+
+#include "lbm_step64.cuh"  // the FP64 step; uses pull_node
+
+namespace lbm {
+
 template <int Q, class S, bool EXT, bool SR>
 cudaError_t launch_step_q(const Ctx& c, const void* src, void* dst, uint32_t seed, cudaStream_t st)
 {
@@ -1476,22 +1482,25 @@ template <int Q, class S>
 cudaError_t launch_step(const Ctx& c, const void* src, void* dst, uint32_t seed, cudaStream_t st,
                         const StgForce* fw = nullptr)
 {
-    StgForce none{};
-    const StgForce& f = fw ? *fw : none;
-    if constexpr (sizeof(typename S::T) == 2) {
-        if (c.stage_R > 0)
-            return c.sr ? launch_step_staged<Q, S, true>(c, src, dst, seed, st, f)
-                        : launch_step_staged<Q, S, false>(c, src, dst, seed, st, f);
-    } else if constexpr (sizeof(typename S::T) == 4) {
-        if (c.stage_R > 0) return launch_step_staged<Q, S, false>(c, src, dst, seed, st, f);
+    if constexpr (sizeof(typename S::T) == 8) return launch_step64<Q>(c, src, dst, zero_padding(c, dst), st);
+    else {
+        StgForce none{};
+        const StgForce& f = fw ? *fw : none;
+        if constexpr (sizeof(typename S::T) == 2) {
+            if (c.stage_R > 0)
+                return c.sr ? launch_step_staged<Q, S, true>(c, src, dst, seed, st, f)
+                            : launch_step_staged<Q, S, false>(c, src, dst, seed, st, f);
+        } else if constexpr (sizeof(typename S::T) == 4) {
+            if (c.stage_R > 0) return launch_step_staged<Q, S, false>(c, src, dst, seed, st, f);
+        }
+        if constexpr (sizeof(typename S::T) == 2) {
+            if (c.sr)
+                return c.ext ? launch_step_q<Q, S, true, true>(c, src, dst, seed, st)
+                             : launch_step_q<Q, S, false, true>(c, src, dst, seed, st);
+        }
+        return c.ext ? launch_step_q<Q, S, true, false>(c, src, dst, seed, st)
+                     : launch_step_q<Q, S, false, false>(c, src, dst, seed, st);
     }
-    if constexpr (sizeof(typename S::T) == 2) {
-        if (c.sr)
-            return c.ext ? launch_step_q<Q, S, true, true>(c, src, dst, seed, st)
-                         : launch_step_q<Q, S, false, true>(c, src, dst, seed, st);
-    }
-    return c.ext ? launch_step_q<Q, S, true, false>(c, src, dst, seed, st)
-                 : launch_step_q<Q, S, false, false>(c, src, dst, seed, st);
 }
 
 // calls f with the kernel's compile-time flags: CURVED (interpolated walls)
