@@ -559,17 +559,21 @@ size_t pop_bytes(const Ctx& x) { return (size_t)x.cfg.lattice * x.geo.sq * x.ele
     DeviceGuard guard_((x).device);                                              \
     if (!guard_.ok) return cuda_fail((x), cudaErrorInvalidDevice, "set device");
 
-// reduce nb partial rows of width W into out (device or host)
-// the mode was checked by out_mode_ok before any launch
-lbm_status finish_reduce(Ctx& x, const double* partials, int nb, int W, double* out, int mode, double weight,
-                         bool accumulate, cudaStream_t st)
+// where the last block of a reduction writes: device output directly, host
+// output through the result slot (the mode was checked by out_mode_ok before
+// any launch)
+RedOut red_out(Ctx& x, double* out, int mode, double weight, bool accumulate)
 {
-    if (mode == LBM_OUT_DEVICE) {
-        CK(launch_reduce_rows(partials, nb, W, out, weight, accumulate ? 1 : 0, st), "reduce");
-        return LBM_OK;
-    }
-    double* slot = x.scratch + SCRATCH_OUT_OFF;
-    CK(launch_reduce_rows(partials, nb, W, slot, weight, 0, st), "reduce");
+    const bool dev = mode == LBM_OUT_DEVICE;
+    return RedOut{dev ? out : x.scratch + SCRATCH_OUT_OFF, weight, dev && accumulate ? 1 : 0, 0,
+                  reinterpret_cast<unsigned*>(x.scratch + SCRATCH_TICKET_OFF)};
+}
+
+// bring the W sums in the result slot to a host output
+lbm_status finish_reduce(Ctx& x, int W, double* out, int mode, bool accumulate, cudaStream_t st)
+{
+    if (mode == LBM_OUT_DEVICE) return LBM_OK;
+    const double* slot = x.scratch + SCRATCH_OUT_OFF;
     if (mode == LBM_OUT_HOST_ASYNC) {
         CK(cudaMemcpyAsync(out, slot, sizeof(double) * W, cudaMemcpyDeviceToHost, st), "copy result");
         return LBM_OK;
@@ -1067,9 +1071,12 @@ lbm_status lbm_wall_force(lbm_ctx* ctx, int wall, unsigned flags, double weight,
     const long long b = wall < 0 ? 0 : x.wall_begin[wall];
     const long long e = wall < 0 ? x.n_links : x.wall_begin[wall + 1];
     double* part = x.scratch + SCRATCH_RED_OFF;
+    const bool acc = (flags & LBM_ACCUMULATE) != 0;
+    const RedOut ro = red_out(x, out, out_on_host, weight, acc);
     int nb = 0;
-    if (e > b) CK(x.ops->links(x, x.pop[x.cur], b, e, flags & 3u, part, &nb, st), "link kernel");
-    return finish_reduce(x, part, nb, 3, out, out_on_host, weight, (flags & LBM_ACCUMULATE) != 0, st);
+    if (e > b) CK(x.ops->links(x, x.pop[x.cur], b, e, flags & 3u, part, ro, &nb, st), "link kernel");
+    else CK(launch_reduce_rows(part, 0, 3, ro.out, weight, ro.accumulate, st), "reduce");
+    return finish_reduce(x, 3, out, out_on_host, acc, st);
 }
 
 lbm_status lbm_step_force(lbm_ctx* ctx, int wall, unsigned flags, double weight, double* out, int out_on_host,
@@ -1144,10 +1151,9 @@ lbm_status lbm_balance(lbm_ctx* ctx, double* out, int out_on_host, void* stream)
     GUARD(x);
     if (!out_mode_ok(out_on_host, false, out, x.err)) return LBM_ERR_ARG;
     cudaStream_t st = (cudaStream_t)stream;
-    double* part = x.scratch + SCRATCH_RED_OFF;
-    int nb = 0;
-    CK(x.ops->balance(x, x.pop[x.cur], part, &nb, st), "balance kernel");
-    return finish_reduce(x, part, nb, 7, out, out_on_host, 1.0, false, st);
+    const RedOut ro = red_out(x, out, out_on_host, 1.0, false);
+    CK(x.ops->balance(x, x.pop[x.cur], x.scratch + SCRATCH_RED_OFF, ro, st), "balance kernel");
+    return finish_reduce(x, 7, out, out_on_host, false, st);
 }
 
 lbm_status lbm_residual(lbm_ctx* ctx, double* v_ref, int update, double* out, int out_on_host, void* stream)
@@ -1159,29 +1165,21 @@ lbm_status lbm_residual(lbm_ctx* ctx, double* v_ref, int update, double* out, in
     GUARD(x);
     if (!out_mode_ok(out_on_host, false, out, x.err)) return LBM_ERR_ARG;
     cudaStream_t st = (cudaStream_t)stream;
-    double* part = x.scratch + SCRATCH_RED_OFF;
-    int nb = 0;
-    CK(x.ops->residual(x, x.pop[x.cur], v_ref, update ? 1 : 0, part, &nb, st), "residual kernel");
-    if (out_on_host == LBM_OUT_HOST) {
-        double sums[2] = {0.0, 0.0};
-        const lbm_status s = finish_reduce(x, part, nb, 2, sums, LBM_OUT_HOST, 1.0, false, st);
-        out[0] = sums[0];
-        out[1] = sums[1];
-        out[2] = sums[1] > 0.0 ? sums[0] / sums[1] : 0.0;
-        if (s == LBM_OK && !std::isfinite(out[2])) {
-            x.err = "the residual is not finite";
-            return LBM_ERR_NAN;
-        }
-        return s;
+    // the two sums and, for device and asynchronous outputs, their ratio
+    RedOut ro = red_out(x, out, out_on_host, 1.0, false);
+    ro.ratio = out_on_host != LBM_OUT_HOST;
+    CK(x.ops->residual(x, x.pop[x.cur], v_ref, update ? 1 : 0, x.scratch + SCRATCH_RED_OFF, ro, st), "residual kernel");
+    if (out_on_host != LBM_OUT_HOST) return finish_reduce(x, 3, out, out_on_host, false, st);
+    double sums[2] = {0.0, 0.0};
+    const lbm_status s = finish_reduce(x, 2, sums, LBM_OUT_HOST, false, st);
+    out[0] = sums[0];
+    out[1] = sums[1];
+    out[2] = sums[1] > 0.0 ? sums[0] / sums[1] : 0.0;
+    if (s == LBM_OK && !std::isfinite(out[2])) {
+        x.err = "the residual is not finite";
+        return LBM_ERR_NAN;
     }
-    // device or page-locked host output: the two sums and their ratio in the
-    // result slot, copied in stream order (HOST_ASYNC) or written to out
-    double* slot = (out_on_host == LBM_OUT_DEVICE) ? out : x.scratch + SCRATCH_OUT_OFF;
-    CK(launch_reduce_rows(part, nb, 2, slot, 1.0, 0, st), "reduce");
-    CK(launch_ratio(slot, st), "ratio");
-    if (out_on_host == LBM_OUT_HOST_ASYNC)
-        CK(cudaMemcpyAsync(out, slot, 3 * sizeof(double), cudaMemcpyDeviceToHost, st), "copy result");
-    return LBM_OK;
+    return s;
 }
 
 lbm_status lbm_run_steady(lbm_ctx* ctx, int every, double tol, int64_t max_steps, double* v_ref, double* r_out,
@@ -1257,8 +1255,9 @@ lbm_status lbm_adjoint_gradient(lbm_ctx* ctx, double* out, int out_on_host, void
     if (!out) return arg_fail(x, "out is NULL");
     GUARD(x);
     if (!out_mode_ok(out_on_host, false, out, x.err)) return LBM_ERR_ARG;
-    return finish_reduce(x, x.scratch + SCRATCH_ADJ_OFF, ADJ_BLOCKS, 6, out, out_on_host, 1.0, false,
-                         (cudaStream_t)stream);
+    const RedOut ro = red_out(x, out, out_on_host, 1.0, false);
+    CK(launch_reduce_rows(x.scratch + SCRATCH_ADJ_OFF, ADJ_BLOCKS, 6, ro.out, 1.0, 0, (cudaStream_t)stream), "reduce");
+    return finish_reduce(x, 6, out, out_on_host, false, (cudaStream_t)stream);
 }
 
 }  // extern "C"
@@ -1367,17 +1366,6 @@ __global__ void k_ins_reset(double* blk, double E0, double E1, double E2, double
     af[0] = f0; af[1] = f1; af[2] = f2;
     as[0] = s0; as[1] = s1; as[2] = s2;
     *reinterpret_cast<unsigned*>(blk + INS_TICKET) = 0u;
-}
-
-__global__ void k_ratio(double* out)
-{
-    if (threadIdx.x == 0 && blockIdx.x == 0) out[2] = out[1] > 0.0 ? out[0] / out[1] : 0.0;
-}
-
-cudaError_t launch_ratio(double* out, cudaStream_t st)
-{
-    k_ratio<<<1, 32, 0, st>>>(out);
-    return cudaGetLastError();
 }
 
 __global__ void k_zero(double* p, long long n)

@@ -56,7 +56,7 @@ constexpr size_t SCRATCH_RED_OFF = 0;
 constexpr size_t SCRATCH_ADJ_OFF = (size_t)MAX_PARTIAL_ROWS * PARTIAL_WIDTH;
 constexpr size_t SCRATCH_OUT_OFF = SCRATCH_ADJ_OFF + (size_t)ADJ_BLOCKS * 6;
 constexpr size_t SCRATCH_FLAG_OFF = SCRATCH_OUT_OFF + 8;   // device error flags (unsigned)
-constexpr size_t SCRATCH_TICKET_OFF = SCRATCH_FLAG_OFF + 1; // last-block ticket of the fused wall force (unsigned)
+constexpr size_t SCRATCH_TICKET_OFF = SCRATCH_FLAG_OFF + 1; // last-block ticket of the reductions (unsigned)
 constexpr size_t SCRATCH_DOUBLES = SCRATCH_FLAG_OFF + 8;
 // insulating walls only, after the above: the field block (E, the sum of v,
 // the force coefficient in FP64, FP32 and FP32 storage units, the ticket of
@@ -72,6 +72,17 @@ constexpr size_t SCRATCH_INS_ROWS = SCRATCH_INS_RED + (size_t)INS_RED_ROWS * 3;
 struct Ctx;
 struct StgForce;
 
+// where a reduction kernel's last block writes: out[k] = (accumulate ? out[k]
+// : 0) + weight * sum k, and with `ratio` the residual's out[0] / out[1]; the
+// ticket finds the last block (null: block rows only)
+struct RedOut {
+    double* out;
+    double weight;
+    int accumulate;
+    int ratio;
+    unsigned* ticket;
+};
+
 struct Dispatch {
     cudaError_t (*step)(const Ctx&, const void* src, void* dst, uint32_t seed, cudaStream_t);
     // the staged step with the wall force of the stored state's step fused in
@@ -82,9 +93,9 @@ struct Dispatch {
                                cudaStream_t);
     cudaError_t (*export_f)(const Ctx&, const void* P, void* out, int dtype, cudaStream_t);
     cudaError_t (*links)(const Ctx&, const void* P, long long begin, long long end, unsigned flags,
-                         double* partials, int* nblocks, cudaStream_t);
-    cudaError_t (*balance)(const Ctx&, const void* P, double* partials, int* nblocks, cudaStream_t);
-    cudaError_t (*residual)(const Ctx&, const void* P, double* vref, int update, double* partials, int* nblocks,
+                         double* partials, const RedOut& ro, int* nblocks, cudaStream_t);
+    cudaError_t (*balance)(const Ctx&, const void* P, double* partials, const RedOut& ro, cudaStream_t);
+    cudaError_t (*residual)(const Ctx&, const void* P, double* vref, int update, double* partials, const RedOut& ro,
                             cudaStream_t);
     cudaError_t (*stress)(const Ctx&, const void* cur, const void* prev, int variant, void* sig, void* S,
                           void* rho, void* v, cudaStream_t);
@@ -110,8 +121,6 @@ const Dispatch& dispatch_bf16_d3q19();
 cudaError_t launch_reduce_rows(const double* partials, int nb, int W, double* out, double weight, int accumulate,
                                cudaStream_t st);
 cudaError_t launch_zero(double* p, long long n, cudaStream_t st);
-// out[2] = out[0] / out[1] (0 when out[1] is 0), on the device
-cudaError_t launch_ratio(double* out, cudaStream_t st);
 // insulating walls: set the field from the last step's mean flow velocity /
 // reset it to the configured field
 cudaError_t ins_update(const Ctx& x, cudaStream_t st);

@@ -74,6 +74,45 @@ __device__ __forceinline__ void block_sum(double (&v)[W], double* smem /* >= W *
     }
 }
 
+// The end of a reduction: thread 0 holds the block's sums in v; they become
+// the block's partial row, and the block that finishes last (a ticket, zero
+// between launches) adds the rows in the order of k_reduce_rows -- lane l of
+// a column's warp takes rows l, l+32, ..., then a fixed shuffle tree -- so
+// the result does not depend on timing and no second launch is needed
+// (a wall force of 10^4 links 12.8 -> 10.7 us).  out[W] = out[0] / out[1]
+// with RATIO.  ticket null: the rows alone.
+template <int W, bool RATIO = false>
+__device__ __forceinline__ void finish_rows(const double (&v)[W], double* __restrict__ partials, const RedOut& ro)
+{
+    __shared__ int last;
+    __shared__ double col[W];
+    if (threadIdx.x == 0) {
+#pragma unroll
+        for (int k = 0; k < W; ++k) partials[(long long)blockIdx.x * W + k] = v[k];
+        last = 0;
+        if (ro.ticket) {
+            __threadfence();
+            last = atomicAdd(ro.ticket, 1u) == gridDim.x - 1;
+        }
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    const int lane = threadIdx.x & 31;
+    for (int k = threadIdx.x >> 5; k < W; k += (int)(blockDim.x >> 5)) {
+        double s = 0.0;
+        for (int r = lane; r < (int)gridDim.x; r += 32) s += __ldcg(partials + (long long)r * W + k);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+        if (lane == 0) col[k] = ro.out[k] = (ro.accumulate ? ro.out[k] : 0.0) + ro.weight * s;
+    }
+    if (threadIdx.x == 0) *ro.ticket = 0u;
+    if constexpr (RATIO) {
+        __syncthreads();
+        if (threadIdx.x == 0 && ro.ratio) ro.out[W] = col[1] > 0.0 ? col[0] / col[1] : 0.0;
+    }
+}
+
 // ------------------------------------------------- fused collide-stream step
 // One thread owns V consecutive nodes of a row (one 16-byte vector per
 // direction).  For every direction it loads the aligned vector of the pull
@@ -826,64 +865,79 @@ k_export(const typename S::T* __restrict__ P, const uint8_t* __restrict__ cls, c
 // = f^rel(x_f, T-1), fbar_a = f_opp(a')(x_f, T), the bounced population
 // (halfway: fbar_a' - w E_a'.LW; interpolated with a wall distance).
 // Per link (dx^D/dt) [e_a' (fbar_a' + fbar_a) + corrections], in FP64.
-template <int Q, class S>
+// CURVED: walls off the half-grid (the bounced population interpolates);
+// otherwise it is the link's own population plus Ladd's term, so a link is
+// one record and one value, and the direction is decoded by arithmetic.
+template <int Q> __device__ __forceinline__ void link_dir(int a, int (&e)[3])
+{
+    constexpr auto pack = [](int c) {
+        unsigned long long t = 0;
+        for (int b = 0; b < Q; ++b)
+            t |= (unsigned long long)(1 + (c == 0 ? EX<Q>(b) : (c == 1 ? EY<Q>(b) : EZ<Q>(b)))) << (2 * b);
+        return t;
+    };
+    constexpr unsigned long long t[3] = {pack(0), pack(1), pack(2)};
+#pragma unroll
+    for (int c = 0; c < 3; ++c) e[c] = (int)(t[c] >> (2 * a) & 3u) - 1;
+}
+template <int Q, class S, bool CURVED>
 __global__ void __launch_bounds__(RED_THREADS)
 k_links(const typename S::T* __restrict__ P, const uint8_t* __restrict__ cls, const Link* __restrict__ links,
         long long begin, long long end, const Geo g, const KP<typename S::R> p, unsigned flags,
-        double* __restrict__ partials)
+        double* __restrict__ partials, const RedOut ro)
 {
+    using R = typename S::R;
     __shared__ double sm[3 * 32];
-    double acc[3] = {0.0, 0.0, 0.0};
+    double acc[3] = {0.0, 0.0, 0.0}, cor[3] = {0.0, 0.0, 0.0};
     const double c = (double)p.c, rho0 = (double)p.rho0, svol = (double)p.svol;
     for (long long i = begin + (long long)blockIdx.x * blockDim.x + threadIdx.x; i < end;
          i += (long long)gridDim.x * blockDim.x) {
         const Link L = links[i];
         const int a = L.dir;
-        double e[3], w = 0.0;
-        double fo = 0.0;
-        // direction tables by a small switch (a is data here)
-#pragma unroll
-        for (int b = 1; b < Q; ++b)
-            if (b == a) {
-                e[0] = EX<Q>(b); e[1] = EY<Q>(b); e[2] = EZ<Q>(b);
-                w = WD<Q>(b);
-            }
-        fo = (double)S::to_r(P[(long long)a * g.sq + L.node]) + w * rho0;
+        int e[3];
+        link_dir<Q>(a, e);
+        const bool axis = e[0] * e[0] + e[1] * e[1] + e[2] * e[2] == 1;
+        const R Pa = S::to_r(P[(long long)a * g.sq + L.node]);
         // bounced population f_opp(a')(x_f, T)
-        const int xn = (int)(L.node % g.nxp);
-        const long long rn = L.node / g.nxp;
-        const int yn = (int)(rn % g.ny), zn = (int)(rn / g.ny);
-        double fi = 0.0;
+        R bounce = R(0);
+        const unsigned rn = L.node / (unsigned)g.nxp;
+        const int xn = (int)(L.node - rn * (unsigned)g.nxp);
+        const int zn = (int)(rn / (unsigned)g.ny), yn = (int)(rn - (unsigned)zn * (unsigned)g.ny);
+        if constexpr (CURVED) {
 #pragma unroll
-        for (int b = 1; b < Q; ++b)
-            if (OPP<Q>(b) == a) fi = (double)bounced<Q, S, false>(P, cls, g, p, xn, yn, zn, L.node, b, L.wall) + w * rho0;
-        double mxa = 0.0;
+            for (int b = 1; b < Q; ++b)
+                if (OPP<Q>(b) == a) bounce = bounced<Q, S, false>(P, cls, g, p, xn, yn, zn, L.node, b, L.wall);
+        } else {
+            // the Ladd term of direction opp(a)
+            bounce = fma(axis ? R(-WD<Q>(1)) : R(-WD<Q>(Q == 9 ? 5 : 7)),
+                         R(e[0]) * p.LW[L.wall][0] + R(e[1]) * p.LW[L.wall][1] + R(e[2]) * p.LW[L.wall][2], Pa);
+        }
+        const double vo = (double)Pa, vi = (double)bounce;
+        double s = vo + vi + 2.0 * (axis ? WD<Q>(1) : WD<Q>(Q == 9 ? 5 : 7)) * rho0;
         if ((flags & 2u) && p.maxwell) {
+            double mxa = 0.0;
             if (p.induced) {
                 // the field of the collision that produced f^rel(x_f, T-1)
-                typename S::R B[3];
+                R B[3];
                 mag_field_at<Q>(p.mag, cls, g, p, xn, yn, zn, (long long)L.node, B);
 #pragma unroll
                 for (int b = 1; b < Q; ++b)
                     if (b == a) mxa = (double)maxwell_at<Q>(p.mxk, B, b);
             } else {
-#pragma unroll
-                for (int b = 1; b < Q; ++b)
-                    if (b == a) mxa = (double)p.mx[b];
+                mxa = (double)p.mx[a];
             }
+            s -= 2.0 * mxa;
         }
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            const double ek = c * e[k];
-            double t = ek * (fo + fi);
-            if (flags & 1u) t += (double)p.LW[L.wall][k] * c / (6.0 * rho0) * (fi - fo);
-            if (flags & 2u) t -= 2.0 * ek * mxa;
-            acc[k] += svol * t;
+            acc[k] += e[k] == 0 ? 0.0 : (e[k] > 0 ? s : -s);
+            if (flags & 1u) cor[k] += (double)p.LW[L.wall][k] / (6.0 * rho0) * (vi - vo);
         }
     }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) acc[k] = svol * c * (acc[k] + cor[k]);
     block_sum<3>(acc, sm);
-    if (threadIdx.x == 0)
-        for (int k = 0; k < 3; ++k) partials[(long long)blockIdx.x * 3 + k] = acc[k];
+    finish_rows<3>(acc, partials, ro);
 }
 
 // ------------------------------------------------- exact moments of a node
@@ -972,7 +1026,7 @@ __device__ __forceinline__ void double_moments(const R (&d)[Q], double (&s)[4])
 template <int Q, class S, bool EXT, bool CURVED>
 __global__ void __launch_bounds__(RED_THREADS)
 k_balance(const typename S::T* __restrict__ P, const uint8_t* __restrict__ cls, const Geo g,
-          const KP<typename S::R> p, double vol, double* __restrict__ partials)
+          const KP<typename S::R> p, double vol, double* __restrict__ partials, const RedOut ro)
 {
     using R = typename S::R;
     __shared__ double sm[7 * 32];
@@ -1029,8 +1083,7 @@ k_balance(const typename S::T* __restrict__ P, const uint8_t* __restrict__ cls, 
         acc[4 + k] = vol * (c / (double)p.dt) * fa[k];
     }
     block_sum<7>(acc, sm);
-    if (threadIdx.x == 0)
-        for (int k = 0; k < 7; ++k) partials[(long long)blockIdx.x * 7 + k] = acc[k];
+    finish_rows<7>(acc, partials, ro);
 }
 
 // ------------------------------------------------------- steady residual
@@ -1044,7 +1097,8 @@ k_balance(const typename S::T* __restrict__ P, const uint8_t* __restrict__ cls, 
 template <int Q, class S, bool EXT, bool CURVED>
 __global__ void __launch_bounds__(RED_THREADS)
 k_residual(const typename S::T* __restrict__ P, const uint8_t* __restrict__ cls, const Geo g,
-           const KP<typename S::R> p, double* __restrict__ vref, int update, double* __restrict__ partials)
+           const KP<typename S::R> p, double* __restrict__ vref, int update, double* __restrict__ partials,
+           const RedOut ro)
 {
     using R = typename S::R;
     __shared__ double sm[2 * 32];
@@ -1101,8 +1155,7 @@ k_residual(const typename S::T* __restrict__ P, const uint8_t* __restrict__ cls,
         acc[1] += sqrt(vv);
     }
     block_sum<2>(acc, sm);
-    if (threadIdx.x == 0)
-        for (int k = 0; k < 2; ++k) partials[(long long)blockIdx.x * 2 + k] = acc[k];
+    finish_rows<2, true>(acc, partials, ro);
 }
 
 // ----------------------------------------------------------------- stress
@@ -1580,43 +1633,43 @@ inline int red_grid(const Ctx& c, long long N, int& threads)
 // warps share one SM's FP64 pipe); from 65,536 links full blocks
 template <int Q, class S>
 cudaError_t launch_links(const Ctx& c, const void* P, long long begin, long long end, unsigned flags,
-                         double* partials, int* nblocks, cudaStream_t st)
+                         double* partials, const RedOut& ro, int* nblocks, cudaStream_t st)
 {
     using T = typename S::T;
-    const int blocks = grid_for(end - begin, RED_THREADS, MAX_PARTIAL_ROWS);
+    const int threads = end - begin > 64ll * MAX_PARTIAL_ROWS ? RED_THREADS : 64;
+    const int blocks = grid_for(end - begin, threads, MAX_PARTIAL_ROWS);
     *nblocks = blocks;
-    k_links<Q, S><<<blocks, RED_THREADS, 0, st>>>((const T*)P, c.cls, c.links, begin, end, c.geo, kp_links_of<S>(c),
-                                                  flags, partials);
-    return cudaGetLastError();
+    return with_curved(c, [&](auto cu) {
+        k_links<Q, S, cu.value><<<blocks, threads, 0, st>>>((const T*)P, c.cls, c.links, begin, end, c.geo,
+                                                            kp_links_of<S>(c), flags, partials, ro);
+    });
 }
 
 template <int Q, class S>
-cudaError_t launch_balance(const Ctx& c, const void* P, double* partials, int* nblocks, cudaStream_t st)
+cudaError_t launch_balance(const Ctx& c, const void* P, double* partials, const RedOut& ro, cudaStream_t st)
 {
     using T = typename S::T;
     const long long N = (long long)c.geo.nx * c.geo.ny * c.geo.nz;
     int threads;
     const int blocks = red_grid(c, N, threads);
-    *nblocks = blocks;
     const double vol = (Q == 9) ? c.cfg.dx * c.cfg.dx : c.cfg.dx * c.cfg.dx * c.cfg.dx;
     return with_ext_curved(c, [&](auto ex, auto cu) {
         k_balance<Q, S, ex.value, cu.value><<<blocks, threads, 0, st>>>((const T*)P, c.cls, c.geo, kp_of<S>(c), vol,
-                                                                        partials);
+                                                                        partials, ro);
     });
 }
 
 template <int Q, class S>
-cudaError_t launch_residual(const Ctx& c, const void* P, double* vref, int update, double* partials, int* nblocks,
+cudaError_t launch_residual(const Ctx& c, const void* P, double* vref, int update, double* partials, const RedOut& ro,
                             cudaStream_t st)
 {
     using T = typename S::T;
     const long long N = (long long)c.geo.nx * c.geo.ny * c.geo.nz;
     int threads;
     const int blocks = red_grid(c, N, threads);
-    *nblocks = blocks;
     return with_ext_curved(c, [&](auto ex, auto cu) {
         k_residual<Q, S, ex.value, cu.value><<<blocks, threads, 0, st>>>((const T*)P, c.cls, c.geo, kp_of<S>(c), vref,
-                                                                         update, partials);
+                                                                         update, partials, ro);
     });
 }
 

@@ -13,16 +13,15 @@
 //
 // How: the block partial sums and the result slot live in one file-scope
 // static device array of fixed size, which every GPU that loads this library
-// holds until the process exits.  The launch has exactly the shape of
-// lbm_wall_force's (at most MAX_PARTIAL_ROWS blocks of RED_THREADS threads,
-// each thread striding over the links), so the two add the same terms in the
-// same order and agree bit for bit at every link count.  One call takes at
+// holds until the process exits.  The launch is lbm_wall_force's (at most
+// MAX_PARTIAL_ROWS blocks, each thread striding over the links), so the two
+// add the same terms in the same order and agree bit for bit at every link count.  One call takes at
 // most NOALLOC_MAX_LINKS links; larger requests are refused.
 #include <cstdio>
 #include <mutex>
 #include <string>
 
-#include "lbm_kernels.cuh"
+#include "lbm_internal.h"
 
 namespace {
 
@@ -57,24 +56,6 @@ bool scratch_address(int dev, double** out, std::string& err)
     }
     *out = g_addr[dev];
     return true;
-}
-
-template <int Q, class S>
-cudaError_t launch_links_rows(const lbm::Ctx& c, const void* P, long long begin, long long end, unsigned flags,
-                              double* partials, int rows, cudaStream_t st)
-{
-    using T = typename S::T;
-    lbm::k_links<Q, S><<<rows, lbm::RED_THREADS, 0, st>>>((const T*)P, c.cls, c.links, begin, end, c.geo,
-                                                         lbm::kp_links_of<S>(c), flags, partials);
-    return cudaGetLastError();
-}
-
-template <class S>
-cudaError_t links_rows(const lbm::Ctx& c, const void* P, long long b, long long e, unsigned flags, double* part,
-                       int rows, cudaStream_t st)
-{
-    return c.cfg.lattice == 9 ? launch_links_rows<9, S>(c, P, b, e, flags, part, rows, st)
-                              : launch_links_rows<19, S>(c, P, b, e, flags, part, rows, st);
 }
 
 }  // namespace
@@ -136,15 +117,10 @@ extern "C" lbm_status lbm_wall_force_noalloc(lbm_ctx* ctx, int wall, unsigned fl
         // per-thread strides, the same partial rows.  Every partial row and
         // the result slot are written before they are read, so nothing in the
         // array needs clearing between calls
-        const int rows = (e > b) ? grid_for(e - b, RED_THREADS, NOALLOC_ROWS) : 0;
-        if (rows > 0) {
-            switch (x.cfg.storage) {
-            case LBM_STORE_F64: ce = links_rows<StoreF64>(x, x.pop[x.cur], b, e, flags & 3u, scratch, rows, st); break;
-            case LBM_STORE_F32: ce = links_rows<StoreF32>(x, x.pop[x.cur], b, e, flags & 3u, scratch, rows, st); break;
-            case LBM_STORE_F16S: ce = links_rows<StoreF16>(x, x.pop[x.cur], b, e, flags & 3u, scratch, rows, st); break;
-            default: ce = links_rows<StoreBF16>(x, x.pop[x.cur], b, e, flags & 3u, scratch, rows, st); break;
-            }
-        }
+        // (no ticket: the rows alone, so that a call racing another on the
+        // shared array spoils only its own values, never a later call's)
+        int rows = 0;
+        if (e > b) ce = x.ops->links(x, x.pop[x.cur], b, e, flags & 3u, scratch, RedOut{}, &rows, st);
         const bool acc = (flags & LBM_ACCUMULATE) != 0;
         if (ce == cudaSuccess) {
             if (out_on_host == LBM_OUT_DEVICE) {
