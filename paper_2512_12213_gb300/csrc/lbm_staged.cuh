@@ -198,44 +198,47 @@ __device__ __forceinline__ void stg_issue(const typename S::T* __restrict__ src,
     if (lane == 0) mbar_arrive(bar);
 }
 
-// the pair (x0, x0+1) of direction a from a staged row: the pull sources
-// x0 - ex and x0 + 1 - ex (ex = E_x, or 0 for a row that holds the node's own
-// opposite populations), wrapped at the row ends of a periodic x axis; at a
-// closed x face the element outside the box is the face value fl (x = 0) or
-// fr (x = nx - 1)
-template <class S>
-__device__ __forceinline__ float2 stg_pair(const typename S::T* __restrict__ row, int ex, int x0, int nx,
-                                           bool closed_x, typename S::T fl, typename S::T fr)
+// the pair (x0, x0+1) of a direction from a staged row: the pull sources
+// x0 - ex and x0 + 1 - ex.  `e` is the element beside the pair, x0 - 1
+// (ex = 1) or x0 + 2 (ex = -1), wrapped at the row ends of a periodic x axis,
+// or at a closed x face the node's own opposite population; `own` says that
+// the row holds the node's own opposite populations instead (a source row
+// outside a closed y or z face), which are not shifted.
+template <class S, int EX>
+__device__ __forceinline__ float2 stg_pair(const typename S::T* __restrict__ row, int x0,
+                                           const typename S::T* __restrict__ e, bool own)
 {
     using T = typename S::T;
     if constexpr (sizeof(T) == 2) {
         const uint32_t w = *reinterpret_cast<const uint32_t*>(row + x0);
-        if (ex == 0) return S::unpack2(w);
-        const unsigned short* h = reinterpret_cast<const unsigned short*>(row);
-        union { T t; unsigned short u; } cv;
-        if (ex == 1) {                                    // values x0-1, x0
-            uint32_t e;
-            if (x0 == 0) {
-                cv.t = fl;
-                e = closed_x ? (uint32_t)cv.u : (uint32_t)h[nx - 1];
-            } else {
-                e = h[x0 - 1];
-            }
-            return S::unpack2(__byte_perm(e, w, 0x5410));
-        }
-        uint32_t e;                                       // values x0+1, x0+2
-        if (x0 + 2 >= nx) {
-            cv.t = fr;
-            e = closed_x ? (uint32_t)cv.u : (uint32_t)h[x0 + 2 - nx];
-        } else {
-            e = h[x0 + 2];
-        }
-        return S::unpack2(__byte_perm(w, e, 0x5432));
+        if (EX == 0) return S::unpack2(w);
+        const uint32_t b = *reinterpret_cast<const unsigned short*>(e);
+        // bytes 0-3 of the permute are the element's, 4-7 the word's
+        return S::unpack2(EX == 1 ? __byte_perm(b, w, own ? 0x7654 : 0x5410) : __byte_perm(b, w, own ? 0x7654 : 0x1076));
     } else {
         const float2 v = *reinterpret_cast<const float2*>(row + x0);
-        if (ex == 0) return v;
-        if (ex == 1) return make_float2(x0 == 0 ? (closed_x ? fl : row[nx - 1]) : row[x0 - 1], v.x);
-        return make_float2(v.y, x0 + 2 >= nx ? (closed_x ? fr : row[x0 + 2 - nx]) : row[x0 + 2]);
+        if (EX == 0) return v;
+        const float b = *e;
+        if (EX == 1) return make_float2(own ? v.x : b, own ? v.y : v.x);
+        return make_float2(own ? v.x : v.y, own ? v.y : b);
+    }
+}
+
+// all directions' pairs; row0: the row of direction 0, pitch: elements between
+// directions; el, er and their pitches: the elements beside the pair, one
+// load each (loading the row's and both face values and selecting spent 38
+// shared loads a pair in closed boxes; with the division of the task index
+// gone too, sphere 256 x 128 x 128 58.3 -> 56.2 us, cavity 256^3 519 -> 511)
+template <int Q, class S, bool FACES, int A = 0>
+__device__ __forceinline__ void stg_load_pairs(F2 (&dd)[Q], const typename S::T* __restrict__ row0, int pitch, int x0,
+                                               const typename S::T* __restrict__ el, int pl,
+                                               const typename S::T* __restrict__ er, int pr, const FaceInfo& fi)
+{
+    if constexpr (A < Q) {
+        int wall = 0;
+        const bool own = FACES && row_out<Q>(fi, A, wall);
+        dd[A] = F2{stg_pair<S, EX<Q>(A)>(row0 + A * pitch, x0, EX<Q>(A) == 1 ? el + A * pl : er + A * pr, own)};
+        stg_load_pairs<Q, S, FACES, A + 1>(dd, row0, pitch, x0, el, pl, er, pr, fi);
     }
 }
 
@@ -457,7 +460,10 @@ k_step_staged(const typename S::T* __restrict__ src, typename S::T* __restrict__
     }
 
     const int group = warp / STG_GROUP_WARPS, gw = warp % STG_GROUP_WARPS;
+    // a warp's tasks of a tile, gw, gw + 8, ...: row and task of the row
     const int tasks_per_row = g.nxp / STG_TASK_NODES;
+    const int r_first = gw / tasks_per_row, xt_first = gw % tasks_per_row;
+    const int r_step = STG_GROUP_WARPS / tasks_per_row, xt_step = STG_GROUP_WARPS % tasks_per_row;
     const long long sq = g.sq;
     const bool closed_x = FACES && !g.periodic[0];
     for (int k = group; k < my_tiles; k += STG_GROUPS) {
@@ -472,9 +478,12 @@ k_step_staged(const typename S::T* __restrict__ src, typename S::T* __restrict__
         const T* sp = reinterpret_cast<const T*>(smem + (size_t)s * stage_bytes);
         const uint8_t* sc = smem + (size_t)s * stage_bytes + stg_cls_off(Q, R, g.nxp, sizeof(T));
         const T* fa = reinterpret_cast<const T*>(smem + (size_t)s * stage_bytes + stg_face_off(Q, R, g.nxp, sizeof(T)));
-        for (int task = gw; task < nr * tasks_per_row; task += STG_GROUP_WARPS) {
-            const int r = task / tasks_per_row;
-            const int x0 = (task - r * tasks_per_row) * STG_TASK_NODES + 2 * lane;
+        for (int r = r_first, xt = xt_first; r < nr; r += r_step, xt += xt_step) {
+            if (xt >= tasks_per_row) {
+                xt -= tasks_per_row;
+                if (++r >= nr) break;
+            }
+            const int x0 = xt * STG_TASK_NODES + 2 * lane;
             const int y = y0 + r;
             const long long base = ((long long)z * g.ny + y) * g.nxp + x0;
             // the pair path serves pairs whose aligned 4-node chunk holds only
@@ -494,16 +503,18 @@ k_step_staged(const typename S::T* __restrict__ src, typename S::T* __restrict__
                 fi.wy_lo = g.face_wall[2]; fi.wy_hi = g.face_wall[3];
                 fi.wz_lo = g.face_wall[4]; fi.wz_hi = g.face_wall[5];
             }
+            // the element beside the pair on either side: in the row, wrapped
+            // at a periodic row end, or (closed x) among the face values, which
+            // then replace the row's base and pitch for this lane
+            const bool le = x0 == 0, re = x0 + 2 >= g.nx;
+            const bool lf = closed_x && le, rf = closed_x && re;
+            const T* el = lf ? fa + r : sp + (size_t)r * g.nxp + (le ? g.nx - 1 : x0 - 1);
+            const T* er = rf ? fa + Q * R + r : sp + (size_t)r * g.nxp + (re ? x0 + 2 - g.nx : x0 + 2);
+            const int pl = lf ? R : R * g.nxp, pr = rf ? R : R * g.nxp;
+            const T* row0 = sp + (size_t)r * g.nxp;
             F2 dd[Q];
-#pragma unroll
-            for (int a = 0; a < Q; ++a) {
-                int wall = 0;
-                const bool rout = FACES && row_out<Q>(fi, a, wall);
-                const T fl = closed_x ? fa[a * R + r] : T(0);
-                const T fr = closed_x ? fa[(Q + a) * R + r] : T(0);
-                dd[a] = F2{stg_pair<S>(sp + ((size_t)a * R + r) * g.nxp, rout ? 0 : EX<Q>(a), x0, g.nx, closed_x, fl,
-                                       fr)};
-            }
+            // (a fold over the directions: the shift is a template argument)
+            stg_load_pairs<Q, S, FACES>(dd, row0, R * g.nxp, x0, el, pl, er, pr, fi);
             if (FACES && p.face_ladd && (cb & 0x02020202u)) {
                 // Ladd terms of moving face walls (k_step's add_ladd2)
 #pragma unroll
