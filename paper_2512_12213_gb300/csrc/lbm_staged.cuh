@@ -56,13 +56,16 @@ namespace lbm {
 constexpr int STG_GROUPS = 2;                         // consumer groups (alternate tiles)
 constexpr int STG_GROUP_WARPS = 8;                    // warps per group
 constexpr int STG_CWARPS = STG_GROUPS * STG_GROUP_WARPS;
-// boundary warps: one, or three where more than 0.5% of the chunks are special
-// (a ragged row has one in every row): three is the most that still leaves
-// five warps on each of the SM's four sub-partitions, so the register cap of
-// 96 stays, and the kernel takes the number from its block size
-constexpr int STG_BWARPS = 3;
-constexpr int STG_THREADS = 32 * (STG_CWARPS + 1 + STG_BWARPS);    // plus the producer
-inline int staged_bwarps(long long n_special, long long nodes) { return n_special * 200 > nodes / 4 ? STG_BWARPS : 1; }
+// boundary warps: one, or more where more than 0.5% of the chunks are special
+// (a ragged row has one in every row): at most the three, with a face warp
+// two, that still leave five warps on each of the SM's four sub-partitions,
+// so the register cap of 96 stays.  The kernel takes the number from its
+// block size.
+constexpr int STG_THREADS = 32 * (STG_CWARPS + 4);    // at most: consumers, producer, three others
+inline int staged_warps(long long n_special, long long nodes, bool closed_x)
+{
+    return n_special * 200 > nodes / 4 ? STG_THREADS / 32 : STG_CWARPS + 2 + (closed_x ? 1 : 0);
+}
 constexpr int STG_COPY_BYTES = 2048;                  // least bytes per direction and tile
 constexpr int STG_TASK_NODES = 64;                    // nodes per warp task (32 pairs)
 constexpr int STG_MAX_STAGES = 8;
@@ -140,13 +143,11 @@ __host__ __device__ inline size_t stg_stage_bytes(int Q, int R, int nxp, int ele
 }
 
 // producer warp: stage the source rows of tile t (plane z, rows y0 .. y0+nr-1).
-// Lane 0 arms the full barrier with the tile's copy bytes (its first
-// arrival); lane a < Q copies direction a's rows and lane Q the class bytes,
-// so the copies of a tile are issued in parallel.  A source row outside a
-// closed y or z face is replaced by the node's own row of the opposite
-// direction (the bounced population, k_step's rule).  With a closed x face
-// the lanes then load the face values (plain loads) and lane 0 arrives a
-// second time once they are in the stage.
+// Lane 0 arms the full barrier with the tile's copy bytes (its arrival); lane
+// a < Q copies direction a's rows and lane Q the class bytes, so the copies
+// of a tile are issued in parallel.  A source row outside a closed y or z
+// face is replaced by the node's own row of the opposite direction (the
+// bounced population, k_step's rule).
 template <int Q, class S, bool FACES>
 __device__ __forceinline__ void stg_issue(const typename S::T* __restrict__ src, const uint8_t* __restrict__ cls,
                                           const Geo& g, int R, int nty, int t, unsigned char* stage, uint64_t* bar,
@@ -185,17 +186,50 @@ __device__ __forceinline__ void stg_issue(const typename S::T* __restrict__ src,
         bulk_g2s(stage + stg_cls_off(Q, R, g.nxp, sizeof(T)), cls + ((long long)z * g.ny + y0) * g.nxp,
                  (uint32_t)nr * g.nxp, bar);
     }
-    if (FACES && !g.periodic[0]) {
-        // face values: own opposite population at x = 0 (side 0) and nx - 1
-        T* fa = reinterpret_cast<T*>(stage + stg_face_off(Q, R, g.nxp, sizeof(T)));
-        for (int i = lane; i < 2 * Q * nr; i += 32) {
-            const int side = i / (Q * nr), rem = i - side * Q * nr, a = rem / nr, r = rem - a * nr;
-            const long long row = ((long long)z * g.ny + y0 + r) * g.nxp;
-            fa[(side * Q + a) * R + r] = src[(long long)OPP<Q>(a) * g.sq + row + (side ? g.nx - 1 : 0)];
+}
+
+// face warp (boxes closed in x): the face values of tile t, the node's own
+// opposite populations at x = 0 for the directions that enter there (E_x = 1)
+// and at x = nx - 1 (E_x = -1), by plain loads issued together.  In the
+// producer warp their round trip stood before every further copy (binary16
+// cavity, stochastic rounding, 256^3: 511 -> 335 us).
+template <int Q, class S>
+__device__ __forceinline__ void stg_faces(const typename S::T* __restrict__ src, const Geo& g, int R, int nty, int t,
+                                          unsigned char* stage, int lane)
+{
+    using T = typename S::T;
+    constexpr int NF = Q == 9 ? 6 : 10;           // entering directions of both faces
+    const int z = t / nty, y0 = (t - z * nty) * R;
+    const int nr = min(R, g.ny - y0);
+    T* fa = reinterpret_cast<T*>(stage + stg_face_off(Q, R, g.nxp, sizeof(T)));
+    const T* rows = src + ((long long)z * g.ny + y0) * g.nxp;
+    for (int i0 = 0; i0 < NF * nr; i0 += 64) {
+        T v[2];
+        int at[2] = {-1, -1};
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const int i = i0 + 32 * k + lane;
+            if (i < NF * nr) {
+                const int f = i / nr, r = i - f * nr;
+                int a = 0, oa = 0, side = 0, n = 0;
+#pragma unroll
+                for (int b = 1; b < Q; ++b)
+                    if (EX<Q>(b) != 0) {
+                        if (n == f) {
+                            a = b;
+                            oa = OPP<Q>(b);
+                            side = EX<Q>(b) < 0;
+                        }
+                        ++n;
+                    }
+                v[k] = rows[(long long)oa * g.sq + (long long)r * g.nxp + (side ? g.nx - 1 : 0)];
+                at[k] = (side * Q + a) * R + r;
+            }
         }
+#pragma unroll
+        for (int k = 0; k < 2; ++k)
+            if (at[k] >= 0) fa[at[k]] = v[k];
     }
-    __syncwarp();
-    if (lane == 0) mbar_arrive(bar);
 }
 
 // the pair (x0, x0+1) of a direction from a staged row: the pull sources
@@ -343,9 +377,10 @@ k_step_staged(const typename S::T* __restrict__ src, typename S::T* __restrict__
         return;
     }
 
+    const bool face_warp = FACES && !g.periodic[0];
     if (threadIdx.x == 0) {
         for (int s = 0; s < nstages; ++s) {
-            mbar_init(&full[s], 2);          // the producer's two arrivals (copies armed, face values in)
+            mbar_init(&full[s], face_warp ? 2 : 1);      // copies armed, and face values in
             mbar_init(&empty[s], STG_GROUP_WARPS);
         }
         mbar_fence_init();
@@ -386,14 +421,30 @@ k_step_staged(const typename S::T* __restrict__ src, typename S::T* __restrict__
         return;
     }
 
+    if (face_warp && warp == STG_CWARPS + 1) {
+        // the face warp refills a stage's face values as the producer does its rows
+        for (int k = 0; k < my_tiles; ++k) {
+            const int s = k % nstages, use = k / nstages;
+            if (use > 0 && !mbar_wait_bounded(&empty[s], (uint32_t)(use - 1) & 1u)) {
+                if (lane == 0) atomicOr(errflag, STG_ERR_TIMEOUT);
+                return;
+            }
+            stg_faces<Q, S>(src, g, R, nty, (int)blockIdx.x + k * (int)gridDim.x, smem + (size_t)s * stage_bytes, lane);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&full[s]);
+        }
+        return;
+    }
+
     if (warp > STG_CWARPS) {
         // boundary warps: the listed chunks, node by node (lane per node), and
         // the wall force of their links when asked for (each lane sums its
         // nodes in a fixed order, then a fixed shuffle tree, one row per warp)
         double acc[3] = {0.0, 0.0, 0.0};
         const long long nn = 4 * nspecial;
-        const int per = (int)(blockDim.x >> 5) - STG_CWARPS - 1;          // boundary warps of a block
-        const int bw = (int)blockIdx.x * per + warp - STG_CWARPS - 1, nbw = (int)gridDim.x * per;
+        const int first = STG_CWARPS + 1 + (face_warp ? 1 : 0);
+        const int per = (int)(blockDim.x >> 5) - first;                   // boundary warps of a block
+        const int bw = (int)blockIdx.x * per + warp - first, nbw = (int)gridDim.x * per;
         if (zero_pad) {
             // a destination that is not the context's own: zero its padding
             // (the special chunks cover the rest of a row's last chunk)
