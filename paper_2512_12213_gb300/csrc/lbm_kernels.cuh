@@ -1506,7 +1506,7 @@ cudaError_t launch_step_staged_k(const Ctx& c, const void* src, void* dst, uint3
         if (e != cudaSuccess) return e;
         c.stage_ready = true;
     }
-    kern<<<staged_blocks(c), 32 * (STG_CWARPS + 1 + staged_bwarps(c.n_special, c.geo.sq)), c.stage_smem, st>>>((const T*)src, (T*)dst, c.cls, c.special, c.n_special,
+    kern<<<staged_blocks(c), 32 * staged_warps(c.n_special, c.geo.sq, !c.geo.periodic[0]), c.stage_smem, st>>>((const T*)src, (T*)dst, c.cls, c.special, c.n_special,
                                                               c.geo, kp_step_of<S>(c), seed, c.stage_R,
                                                               c.stage_tiles, c.stage_n, zero_padding(c, dst), c.errflag,
                                                               fw);
