@@ -660,13 +660,11 @@ __device__ __forceinline__ void node_values(const Src& s, const KP<R>&, const WR
 // even = rho - rho0 - sum q / 2 + 3/2 (E.m)(E.W), the last product
 // q_i + q_j +- 2 m_i W_j for a diagonal pair: 67 operations a node.
 template <int Q, typename R>
-__device__ __forceinline__ void node_values(const SrcFields& s, const KP<R>& p, const WRho& wr, long long n, R (&d)[Q])
+__device__ __forceinline__ void fields_values64(const SrcFields& s, const KP<R>& p, const WRho& wr, long long n,
+                                                double rho, const double (&W)[3], R (&d)[Q])
 {
     constexpr int D = LatDim<Q>::D;
-    const double rho = s.rho[n];
-    double W[3], m[3], q[3], sq = 0.0;
-#pragma unroll
-    for (int k = 0; k < D; ++k) W[k] = s.u[(long long)k * s.N + n] * s.ic;
+    double m[3], q[3], sq = 0.0;
 #pragma unroll
     for (int k = 0; k < D; ++k) {
         m[k] = 3.0 * rho * W[k];
@@ -706,6 +704,123 @@ __device__ __forceinline__ void node_values(const SrcFields& s, const KP<R>& p, 
         put(a, fma(w, em, even));
         put(b, fma(-w, em, even));
     }
+}
+
+// Unevaluated FP32 sums h + l (|l| about 2^-24 |h|, 48 bits together): exact
+// products by the fused multiply-add, exact sums by Knuth's two-sum (Dekker
+// 1971); each operation keeps 2^-46 of its operands.
+struct FF {
+    float h, l;
+};
+__device__ __forceinline__ FF ff_add(FF x, FF y)
+{
+    const float s = __fadd_rn(x.h, y.h), b = __fsub_rn(s, x.h);
+    const float e = __fadd_rn(__fsub_rn(x.h, __fsub_rn(s, b)), __fsub_rn(y.h, b));
+    return FF{s, __fadd_rn(e, __fadd_rn(x.l, y.l))};
+}
+__device__ __forceinline__ FF ff_mul(FF x, FF y)
+{
+    const float p = __fmul_rn(x.h, y.h);
+    return FF{p, __fmaf_rn(x.l, y.h, __fmaf_rn(x.h, y.l, __fmaf_rn(x.h, y.h, -p)))};
+}
+__device__ __forceinline__ FF ff_neg(FF x) { return FF{-x.h, -x.l}; }
+__device__ __forceinline__ FF ff_scale(FF x, float c) { return FF{x.h * c, x.l * c}; }      // c a power of two
+__host__ __device__ constexpr FF ff_const(double c) { return FF{(float)c, (float)(c - (double)(float)c)}; }
+// x as h + l by its bits (the FP64 pipe converts as slowly as it adds): h the
+// leading 24 bits, l the other 29 rounded to 24; ok = false outside
+// 2^-73 .. 2^60 (zero is in)
+__device__ __forceinline__ FF ff_split(double x, bool& ok)
+{
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+    const unsigned e = (hi >> 20) & 0x7FFu, sign = hi & 0x80000000u;
+    if (((hi << 1) | lo) == 0u) return FF{0.0f, 0.0f};
+    if (e - 950u > 1083u - 950u) ok = false;
+    const float h = __uint_as_float(sign | ((((hi & 0x7FFFFFFFu) - 0x38000000u) << 3) | (lo >> 29)));
+    // 2^(exponent - 52), signed; e - 1023 - 52 + 127 = e - 948
+    const float u = __uint_as_float(sign | ((e - 948u) << 23));
+    return FF{h, __fmul_rn((float)(lo & 0x1FFFFFFFu), u)};
+}
+
+// the deviations of the equilibrium (without xi), for FP32 compute: as
+// fields_values64, in unevaluated FP32 sums, whose ~480 FP32 operations a node
+// cost a sixth of 67 FP64 ones.  With J = rho W, K_k = J_k W_k, X = J_i W_j
+// and Z = rho - rho0 - 3/2 sum K, the pairs are  w1 Z + 9/2 w1 K_k +- 3 w1 J_k
+// and  w2 Z + 9/2 w2 (K_i + K_j +- 2 X) +- 3 w2 (J_i +- J_j); 9/2 w is a power
+// of two.  Rounded to FP32 at the end, as the FP64 values were: the stored values'
+// error against 64 bits is the rounding's, 2.7e-8, at deviations of 1e-2 to
+// 1e-8 alike.  256 x 128 x 128: 1,335 us in FP64 -> 145 us (0.3 of the copy
+// bandwidth).  false (d not set): an input outside the range of ff_split.
+template <int Q>
+__device__ __forceinline__ bool fields_values32(const KP<float>& p, double rho, const double (&Wd)[3], float (&d)[Q])
+{
+    constexpr int D = LatDim<Q>::D;
+    constexpr double w1 = WD<Q>(1), w2 = WD<Q>(Q == 9 ? 5 : 7);
+    bool ok = true;
+    const FF dr = ff_split(rho - (double)p.rho0, ok);
+    const FF rh = ff_add(FF{p.rho0, 0.0f}, dr);
+    FF W[3], J[3], O[3], K[3], Z = dr;
+#pragma unroll
+    for (int k = 0; k < D; ++k) {
+        W[k] = ff_split(Wd[k], ok);
+        J[k] = ff_mul(rh, W[k]);
+        O[k] = ff_mul(J[k], ff_const(3.0 * w1));
+    }
+    if (!ok) return false;
+    const bool quad = !p.stokes;                 // the linear equilibrium drops the quadratic terms
+    if (quad) {
+        FF sum{0.0f, 0.0f};
+#pragma unroll
+        for (int k = 0; k < D; ++k) {
+            K[k] = ff_mul(J[k], W[k]);
+            sum = k ? ff_add(sum, K[k]) : K[k];
+        }
+        Z = ff_add(ff_add(Z, ff_neg(sum)), ff_scale(sum, -0.5f));
+    }
+    auto put = [&](int a, FF v) {
+        if (p.maxwell) v = ff_add(v, FF{p.mx[a], 0.0f});
+        d[a] = __fadd_rn(v.h, v.l);
+    };
+    put(0, ff_mul(Z, ff_const(WD<Q>(0))));
+    const FF Z1 = ff_mul(Z, ff_const(w1)), Z2 = ff_scale(Z1, (float)(w2 / w1));
+#pragma unroll
+    for (int k = 0; k < LatDim<Q>::NP; ++k) {
+        const int a = PAIR<Q>(k), b = OPP<Q>(a);
+        const int e[3] = {EX<Q>(a), EY<Q>(a), EZ<Q>(a)};
+        const int i = e[0] ? 0 : (e[1] ? 1 : 2);
+        FF even, odd;
+        if (SPEED2<Q>(a) == 1) {
+            even = quad ? ff_add(Z1, ff_scale(K[i], (float)(4.5 * w1))) : Z1;
+            odd = O[i];
+        } else {
+            const int j = e[2] ? 2 : 1;
+            const FF oi = ff_scale(O[i], (float)(e[i] * w2 / w1)), oj = ff_scale(O[j], (float)(e[j] * w2 / w1));
+            odd = ff_add(oi, oj);
+            even = Z2;
+            if (quad) {
+                even = ff_add(Z2, ff_scale(ff_add(K[i], K[j]), (float)(4.5 * w2)));
+                even = ff_add(even, ff_scale(ff_mul(J[i], W[j]), (float)(9.0 * w2 * e[i] * e[j])));
+            }
+        }
+        put(a, ff_add(even, odd));
+        put(b, ff_add(even, ff_neg(odd)));
+    }
+    return true;
+}
+
+template <int Q, typename R>
+__device__ __forceinline__ void node_values(const SrcFields& s, const KP<R>& p, const WRho& wr, long long n, R (&d)[Q])
+{
+    double W[3] = {0.0, 0.0, 0.0};
+    const double rho = s.rho[n];
+#pragma unroll
+    for (int k = 0; k < LatDim<Q>::D; ++k) {
+        W[k] = s.u[(long long)k * s.N + n];
+        if (s.ic != 1.0) W[k] *= s.ic;
+    }
+    if constexpr (sizeof(R) == 4) {
+        if (!s.xi && fields_values32<Q>(p, rho, W, d)) return;
+    }
+    fields_values64<Q, R>(s, p, wr, n, rho, W, d);
 }
 
 // one of them (a is a constant: the others' terms are dropped)
@@ -769,8 +884,8 @@ __device__ R unbounced(const Src& s, const KP<R>& p, const WRho& wr, const Geo& 
 
 // one padded node per thread.  Before (each node pulling its 18 neighbours'
 // values, with their equilibria in FP64) a 192^3 binary16 box took 12.2 ms
-// from fields and 1.04 ms from FP32 populations; so 2.25 ms (the FP64 pipe)
-// and 0.225 ms (0.53 of the copy bandwidth).
+// from fields and 1.04 ms from FP32 populations; so 0.345 ms and
+// 0.225 ms (0.53 of the copy bandwidth).
 template <int Q, class S, class Src, bool CURVED>
 __global__ void __launch_bounds__(NODE_THREADS)
 k_inverse_stream(typename S::T* __restrict__ P, const uint8_t* __restrict__ cls, const Geo g,
