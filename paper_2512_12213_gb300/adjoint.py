@@ -54,8 +54,11 @@ class DragProblem:
         for t in range(self.T):
             if t % self.k == 0:
                 lbm.lbm_save_state(s.ctx, self.ckpt[t // self.k], st)
-            lbm.lbm_step(s.ctx, 1, st)
-            lbm.lbm_wall_force(s.ctx, self.wall, lbm.ACCUMULATE, 1.0 / self.T, self.Facc, 0, st)
+            if t == 0:
+                lbm.lbm_step(s.ctx, 1, st)
+            else:                                # with the force of the step before, beside it
+                lbm.lbm_step_force(s.ctx, self.wall, lbm.ACCUMULATE, 1.0 / self.T, self.Facc, lbm.OUT_DEVICE, st)
+        lbm.lbm_wall_force(s.ctx, self.wall, lbm.ACCUMULATE, 1.0 / self.T, self.Facc, lbm.OUT_DEVICE, st)
         F = self.Facc.cpu().numpy()
         return float(np.dot(self.d, F))
 

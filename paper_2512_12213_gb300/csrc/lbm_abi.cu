@@ -732,6 +732,7 @@ lbm_status lbm_create(const lbm_config* cfg, const uint8_t* host_wall_id, void* 
     }
     choose_stage(x);
     x.adj_blocks = 0;
+    x.late_wait = false;
     cudaStream_t st = (cudaStream_t)stream;
     cudaError_t e = cudaMemcpyAsync(x.cls, cls.data(), cls.size(), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess && x.special && x.n_special)
@@ -1097,10 +1098,14 @@ lbm_status lbm_step_force(lbm_ctx* ctx, int wall, unsigned flags, double weight,
     if (x.stage_R <= 0 || !all_periodic(&x.cfg) || x.ext) {
         // the register-tiled step, or a staged step with closed faces (whose
         // face links the boundary warps do not see) or the EXT node code: the
-        // two calls in sequence
-        const lbm_status s = lbm_wall_force(ctx, wall, flags, weight, out, out_on_host, stream);
+        // two calls in sequence; with device output nothing lies between the
+        // two kernels, and the register step runs beside the link sum
+        lbm_status s = lbm_wall_force(ctx, wall, flags, weight, out, out_on_host, stream);
         if (s != LBM_OK) return s;
-        return lbm_step(ctx, 1, stream);
+        x.late_wait = out_on_host == LBM_OUT_DEVICE;
+        s = lbm_step(ctx, 1, stream);
+        x.late_wait = false;
+        return s;
     }
     StgForce fw;
     memset(&fw, 0, sizeof fw);
@@ -1296,6 +1301,8 @@ __global__ void k_ins_update(const double* __restrict__ rows, long long n, long 
                              double n_fluid, double c, double dt, double sigma, double B0, double B1, double B2,
                              double scale)
 {
+    pdl_trigger();
+    pdl_wait(rows);
     __shared__ double sm[3 * 32];
     __shared__ int last;
     unsigned* ticket = reinterpret_cast<unsigned*>(blk + INS_TICKET);
@@ -1387,10 +1394,10 @@ cudaError_t ins_update(const Ctx& x, cudaStream_t st)
     const long long chunk = std::max<long long>((n + INS_RED_ROWS - 1) / INS_RED_ROWS, 256);
     const int nb = (int)((n + chunk - 1) / chunk);
     const double scale = (x.cfg.storage == LBM_STORE_F16S) ? 4096.0 : 1.0;
-    k_ins_update<<<nb, 256, 0, st>>>(x.scratch + SCRATCH_INS_ROWS, n, chunk, x.scratch + SCRATCH_INS_RED,
-                                     x.scratch + SCRATCH_INS_OFF, (double)(x.n_fluid > 0 ? x.n_fluid : 1), x.kpd.c,
-                                     x.kpd.dt, x.cfg.sigma_e, x.cfg.B[0], x.cfg.B[1], x.cfg.B[2], scale);
-    return cudaGetLastError();
+    return launch_pdl(k_ins_update, nb, 256, 0, st, x.scratch + SCRATCH_INS_ROWS, n, chunk,
+                      x.scratch + SCRATCH_INS_RED, x.scratch + SCRATCH_INS_OFF,
+                      (double)(x.n_fluid > 0 ? x.n_fluid : 1), x.kpd.c, x.kpd.dt, x.cfg.sigma_e, x.cfg.B[0],
+                      x.cfg.B[1], x.cfg.B[2], scale);
 }
 
 // the configured field and its force coefficients (fill_params computed them)

@@ -38,6 +38,8 @@ k_adjoint(const typename S::T* __restrict__ Pprev, const typename S::R* __restri
           const KP<typename S::R> p, int target, const AdjConst<typename S::R> ac, double gscale,
           double* __restrict__ partials)
 {
+    pdl_trigger();
+    pdl_wait(Pprev, phin);
     using R = typename S::R;
     constexpr int D = LatDim<Q>::D;
     __shared__ double sm[6 * 32];
@@ -229,9 +231,8 @@ cudaError_t launch_adjoint(const Ctx& c, const void* Pprev, const void* phin, vo
         ac.seed[a] = R(seedw * 2.0 * pd.svol * de);
         ac.gl[a] = R(-6.0 * WD<Q>(a) * pd.rho0 / pd.c);
     }
-    k_adjoint<Q, S><<<blocks, RED_THREADS, 0, st>>>((const T*)Pprev, (const R*)phin, (R*)phio, c.cls, c.geo, p, wall,
-                                                    ac, pd.dt / pd.c, partials);
-    return cudaGetLastError();
+    return launch_pdl(k_adjoint<Q, S>, blocks, RED_THREADS, 0, st, (const T*)Pprev, (const R*)phin, (R*)phio, c.cls,
+                      c.geo, p, wall, ac, pd.dt / pd.c, partials);
 }
 
 }  // namespace lbm

@@ -19,7 +19,51 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 namespace lbm {
+
+// ------------------------------------------------ programmatic launches
+// The kernels of a step sequence are launched so that the next grid may be
+// scheduled while the one before drains (launch_pdl): its blocks then sit
+// ready, index arithmetic and class bytes done, and pdl_wait releases them
+// when the earlier grid has completed and its stores are visible.  Every
+// thread of such a grid calls pdl_wait before it touches anything an earlier
+// kernel of the stream writes, and before it exits, so the completion of a
+// grid implies that of all before it.  pdl_trigger lets the next grid start;
+// a kernel without it holds the next one back to its end, as without all
+// this.  (Steps: 2-D
+// cylinder 512 x 256 FP32 6.2 -> 4.2 us, FP64 channel 64 x 32 6.2 -> 4.0.)
+// (pointers of earlier kernels' data pass through the wait, so that the
+// compiler does not turn their loads into read-only ones: nothing keeps
+// ld.global.nc behind the wait, and such data is never read with it)
+template <class... P> __device__ __forceinline__ void pdl_wait(P&... p)
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    auto pass = [](auto& q) {
+        size_t a = __cvta_generic_to_global(q);          // a global address before and after
+        asm volatile("" : "+l"(a));
+        q = static_cast<std::remove_cv_t<std::remove_reference_t<decltype(q)>>>(__cvta_global_to_generic(a));
+    };
+    (pass(p), ...);
+}
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+template <class... P, class... A>
+inline cudaError_t launch_pdl(void (*kern)(P...), unsigned blocks, unsigned threads, size_t smem, cudaStream_t st,
+                              A&&... args)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
 
 // ---------------------------------------------------------------- lattices
 // D2Q9 : 0 (0,0) 1 (1,0) 2 (0,1) 3 (-1,0) 4 (0,-1) 5 (1,1) 6 (-1,1) 7 (-1,-1) 8 (1,-1)

@@ -151,8 +151,10 @@ template <class S, bool EXT, bool FACES = false, bool FULL = false, bool LP = fa
 template <int Q, class S, bool EXT, bool FACES, bool SR, bool FULL = false, bool LP = false>
 __global__ void __launch_bounds__(STEP_THREADS, StepOcc<S, EXT, FACES, FULL, LP>::value)
 k_step(const typename S::T* __restrict__ src, typename S::T* __restrict__ dst,
-       const uint8_t* __restrict__ cls, const Geo g, const KP<typename S::R> p, uint32_t seed, int zero_pad)
+       const uint8_t* __restrict__ cls, const Geo g, const KP<typename S::R> p, uint32_t seed, int zero_pad,
+       int late)
 {
+    pdl_trigger();
     using T = typename S::T;
     using R = typename S::R;
     constexpr int V = S::V;
@@ -213,6 +215,9 @@ k_step(const typename S::T* __restrict__ src, typename S::T* __restrict__ dst,
             roff[dy + 1][dz + 1] = ((long long)zs * g.ny + ys) * g.nxp;
         }
     const long long own = row * g.nxp;
+    // (late: the kernel before is the wall force's of the same state, which
+    // this step may run beside)
+    if (!late) pdl_wait(src);
 
     using RawT = typename RawVec<sizeof(T) * V>::type;
     // shifted source values: packed words for 16-bit formats, else elements
@@ -226,7 +231,7 @@ k_step(const typename S::T* __restrict__ src, typename S::T* __restrict__ dst,
         for (int a = 0; a < Q; ++a) {
             const T* rp = src + (long long)a * g.sq + roff[EY<Q>(a) + 1][EZ<Q>(a) + 1];
             VecN<T, V> raw;
-            raw.raw = __ldg(reinterpret_cast<const RawT*>(rp + xl));
+            raw.raw = *reinterpret_cast<const RawT*>(rp + xl);
             const int ex = EX<Q>(a);
             T edge = raw.e[0];
             // periodic x: the wrap of a row edge and the warp edge are plain loads
@@ -282,7 +287,7 @@ k_step(const typename S::T* __restrict__ src, typename S::T* __restrict__ dst,
         for (int a = 0; a < Q; ++a) {
             int rwall = 0;
             const bool rout = row_out<Q>(fi, a, rwall);
-            raw[a].raw = __ldg(reinterpret_cast<const RawT*>(row_ptr(a, rout) + xl));
+            raw[a].raw = *reinterpret_cast<const RawT*>(row_ptr(a, rout) + xl);
         }
         // lanes at a warp edge or a row edge load the element the shuffle
         // cannot give them: the left neighbour of x0 (E_x = +1) or the right
@@ -601,6 +606,7 @@ k_step(const typename S::T* __restrict__ src, typename S::T* __restrict__ dst,
             *reinterpret_cast<RawT*>(dst + (long long)a * g.sq + row * g.nxp + x0) = RawT{};
     __syncwarp();
     put_v();
+    if (late) pdl_wait();
 }
 
 // ------------------------------------------------- deviations and populations
@@ -891,6 +897,7 @@ __global__ void __launch_bounds__(NODE_THREADS)
 k_inverse_stream(typename S::T* __restrict__ P, const uint8_t* __restrict__ cls, const Geo g,
                  const KP<typename S::R> p, const WRho wr, const Src s)
 {
+    pdl_wait();
     using R = typename S::R;
     const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (n >= g.sq) return;
@@ -952,6 +959,7 @@ __global__ void __launch_bounds__(NODE_THREADS)
 k_export(const typename S::T* __restrict__ P, const uint8_t* __restrict__ cls, const Geo g,
          const KP<typename S::R> p, const WRho wr, OutT* __restrict__ out)
 {
+    pdl_wait(P);
     using R = typename S::R;
     const unsigned N = (unsigned)g.nx * (unsigned)g.ny * (unsigned)g.nz;
     for (unsigned n = blockIdx.x * blockDim.x + threadIdx.x; n < N; n += gridDim.x * blockDim.x) {
@@ -1001,6 +1009,8 @@ k_links(const typename S::T* __restrict__ P, const uint8_t* __restrict__ cls, co
         long long begin, long long end, const Geo g, const KP<typename S::R> p, unsigned flags,
         double* __restrict__ partials, const RedOut ro)
 {
+    pdl_wait(P);
+    pdl_trigger();      // after the wait: a step may run beside this kernel
     using R = typename S::R;
     __shared__ double sm[3 * 32];
     double acc[3] = {0.0, 0.0, 0.0}, cor[3] = {0.0, 0.0, 0.0};
@@ -1143,6 +1153,7 @@ __global__ void __launch_bounds__(RED_THREADS)
 k_balance(const typename S::T* __restrict__ P, const uint8_t* __restrict__ cls, const Geo g,
           const KP<typename S::R> p, double vol, double* __restrict__ partials, const RedOut ro)
 {
+    pdl_wait(P);
     using R = typename S::R;
     __shared__ double sm[7 * 32];
     double tot[4] = {0, 0, 0, 0}, fa[3] = {0, 0, 0};     // sums of d and E d; of rho A with EXT
@@ -1215,6 +1226,7 @@ k_residual(const typename S::T* __restrict__ P, const uint8_t* __restrict__ cls,
            const KP<typename S::R> p, double* __restrict__ vref, int update, double* __restrict__ partials,
            const RedOut ro)
 {
+    pdl_wait(P);
     using R = typename S::R;
     __shared__ double sm[2 * 32];
     double acc[2] = {0.0, 0.0};
@@ -1283,6 +1295,7 @@ k_stress(const typename S::T* __restrict__ cur, const typename S::T* __restrict_
          typename S::R* __restrict__ sig, typename S::R* __restrict__ Sout, typename S::R* __restrict__ rho_out,
          typename S::R* __restrict__ v_out)
 {
+    pdl_wait(cur, prev);
     using R = typename S::R;
     constexpr int D = LatDim<Q>::D;
     constexpr int NC = (D == 3) ? 6 : 3;
@@ -1580,30 +1593,17 @@ cudaError_t launch_step_q(const Ctx& c, const void* src, void* dst, uint32_t see
     const int blocks = grid_for(nch, STEP_THREADS, 1ll << 31);
     const int zp = zero_padding(c, dst);
     const bool faces = !c.geo.periodic[0] || !c.geo.periodic[1] || (Q == 19 && !c.geo.periodic[2]);
+    auto go = [&](auto fc, auto full, auto lp) {
+        return launch_pdl(k_step<Q, S, EXT, fc.value, SR, full.value, lp.value>, blocks, STEP_THREADS, 0, st,
+                          (const T*)src, (T*)dst, c.cls, c.geo, kp_step_of<S>(c), seed, zp, c.late_wait ? 1 : 0);
+    };
+    const std::true_type yes{};
+    const std::false_type no{};
     if constexpr (EXT && sizeof(typename S::T) == 2) {
-        if (c.les_pair) {
-            if (faces)
-                k_step<Q, S, EXT, true, SR, false, true><<<blocks, STEP_THREADS, 0, st>>>(
-                    (const T*)src, (T*)dst, c.cls, c.geo, kp_step_of<S>(c), seed, zp);
-            else
-                k_step<Q, S, EXT, false, SR, false, true><<<blocks, STEP_THREADS, 0, st>>>(
-                    (const T*)src, (T*)dst, c.cls, c.geo, kp_step_of<S>(c), seed, zp);
-            return cudaGetLastError();
-        }
+        if (c.les_pair) return faces ? go(yes, no, yes) : go(no, no, yes);
     }
-    if ((c.cfg.curved || c.insulating) && faces)
-        k_step<Q, S, EXT, true, SR, true><<<blocks, STEP_THREADS, 0, st>>>((const T*)src, (T*)dst, c.cls, c.geo,
-                                                                           kp_step_of<S>(c), seed, zp);
-    else if (c.cfg.curved || c.insulating)
-        k_step<Q, S, EXT, false, SR, true><<<blocks, STEP_THREADS, 0, st>>>((const T*)src, (T*)dst, c.cls, c.geo,
-                                                                            kp_step_of<S>(c), seed, zp);
-    else if (faces)
-        k_step<Q, S, EXT, true, SR><<<blocks, STEP_THREADS, 0, st>>>((const T*)src, (T*)dst, c.cls, c.geo,
-                                                                     kp_step_of<S>(c), seed, zp);
-    else
-        k_step<Q, S, EXT, false, SR><<<blocks, STEP_THREADS, 0, st>>>((const T*)src, (T*)dst, c.cls, c.geo,
-                                                                      kp_step_of<S>(c), seed, zp);
-    return cudaGetLastError();
+    if (c.cfg.curved || c.insulating) return faces ? go(yes, yes, no) : go(no, yes, no);
+    return faces ? go(yes, no, no) : go(no, no, no);
 }
 
 // the staged step (periodic boxes with the plain node code, 16-bit or FP32
@@ -1621,11 +1621,9 @@ cudaError_t launch_step_staged_k(const Ctx& c, const void* src, void* dst, uint3
         if (e != cudaSuccess) return e;
         c.stage_ready = true;
     }
-    kern<<<staged_blocks(c), 32 * staged_warps(c.n_special, c.geo.sq, !c.geo.periodic[0]), c.stage_smem, st>>>((const T*)src, (T*)dst, c.cls, c.special, c.n_special,
-                                                              c.geo, kp_step_of<S>(c), seed, c.stage_R,
-                                                              c.stage_tiles, c.stage_n, zero_padding(c, dst), c.errflag,
-                                                              fw);
-    return cudaGetLastError();
+    return launch_pdl(kern, staged_blocks(c), 32 * staged_warps(c.n_special, c.geo.sq, !c.geo.periodic[0]),
+                      c.stage_smem, st, (const T*)src, (T*)dst, c.cls, c.special, c.n_special, c.geo, kp_step_of<S>(c),
+                      seed, c.stage_R, (int)c.stage_tiles, c.stage_n, zero_padding(c, dst), c.errflag, fw);
 }
 
 // the staged step (the host chose the tile rows and stage count at create)
@@ -1674,16 +1672,13 @@ cudaError_t launch_step(const Ctx& c, const void* src, void* dst, uint32_t seed,
 // calls f with the kernel's compile-time flags: CURVED (interpolated walls)
 template <class F> inline cudaError_t with_curved(const Ctx& c, F&& f)
 {
-    if (c.cfg.curved) f(std::true_type{});
-    else f(std::false_type{});
-    return cudaGetLastError();
+    return c.cfg.curved ? f(std::true_type{}) : f(std::false_type{});
 }
 // and EXT, CURVED
 template <class F> inline cudaError_t with_ext_curved(const Ctx& c, F&& f)
 {
     return with_curved(c, [&](auto cu) {
-        if (c.ext) f(std::true_type{}, cu);
-        else f(std::false_type{}, cu);
+        return c.ext ? f(std::true_type{}, cu) : f(std::false_type{}, cu);
     });
 }
 
@@ -1693,8 +1688,8 @@ cudaError_t launch_inverse(const Ctx& c, const Src& src, void* dst, cudaStream_t
     const int blocks = grid_for(c.geo.sq, NODE_THREADS, 1ll << 31);
     const WRho wr = wrho_of<Q>((double)kp_of<S>(c).rho0);
     return with_curved(c, [&](auto cu) {
-        k_inverse_stream<Q, S, Src, cu.value><<<blocks, NODE_THREADS, 0, st>>>((typename S::T*)dst, c.cls, c.geo,
-                                                                               kp_of<S>(c), wr, src);
+        return launch_pdl(k_inverse_stream<Q, S, Src, cu.value>, blocks, NODE_THREADS, 0, st, (typename S::T*)dst,
+                          c.cls, c.geo, kp_of<S>(c), wr, src);
     });
 }
 
@@ -1723,11 +1718,10 @@ cudaError_t launch_export(const Ctx& c, const void* P, void* out, int dtype, cud
     const WRho wr = wrho_of<Q>((double)kp_of<S>(c).rho0);
     return with_curved(c, [&](auto cu) {
         if (dtype == 0)
-            k_export<Q, S, double, cu.value><<<blocks, NODE_THREADS, 0, st>>>((const T*)P, c.cls, c.geo, kp_of<S>(c),
-                                                                               wr, (double*)out);
-        else
-            k_export<Q, S, float, cu.value><<<blocks, NODE_THREADS, 0, st>>>((const T*)P, c.cls, c.geo, kp_of<S>(c),
-                                                                              wr, (float*)out);
+            return launch_pdl(k_export<Q, S, double, cu.value>, blocks, NODE_THREADS, 0, st, (const T*)P, c.cls, c.geo,
+                              kp_of<S>(c), wr, (double*)out);
+        return launch_pdl(k_export<Q, S, float, cu.value>, blocks, NODE_THREADS, 0, st, (const T*)P, c.cls, c.geo,
+                          kp_of<S>(c), wr, (float*)out);
     });
 }
 
@@ -1755,8 +1749,8 @@ cudaError_t launch_links(const Ctx& c, const void* P, long long begin, long long
     const int blocks = grid_for(end - begin, threads, MAX_PARTIAL_ROWS);
     *nblocks = blocks;
     return with_curved(c, [&](auto cu) {
-        k_links<Q, S, cu.value><<<blocks, threads, 0, st>>>((const T*)P, c.cls, c.links, begin, end, c.geo,
-                                                            kp_links_of<S>(c), flags, partials, ro);
+        return launch_pdl(k_links<Q, S, cu.value>, blocks, threads, 0, st, (const T*)P, c.cls, c.links, begin, end,
+                          c.geo, kp_links_of<S>(c), flags, partials, ro);
     });
 }
 
@@ -1769,8 +1763,8 @@ cudaError_t launch_balance(const Ctx& c, const void* P, double* partials, const 
     const int blocks = red_grid(c, N, threads);
     const double vol = (Q == 9) ? c.cfg.dx * c.cfg.dx : c.cfg.dx * c.cfg.dx * c.cfg.dx;
     return with_ext_curved(c, [&](auto ex, auto cu) {
-        k_balance<Q, S, ex.value, cu.value><<<blocks, threads, 0, st>>>((const T*)P, c.cls, c.geo, kp_of<S>(c), vol,
-                                                                        partials, ro);
+        return launch_pdl(k_balance<Q, S, ex.value, cu.value>, blocks, threads, 0, st, (const T*)P, c.cls, c.geo,
+                          kp_of<S>(c), vol, partials, ro);
     });
 }
 
@@ -1783,8 +1777,8 @@ cudaError_t launch_residual(const Ctx& c, const void* P, double* vref, int updat
     int threads;
     const int blocks = red_grid(c, N, threads);
     return with_ext_curved(c, [&](auto ex, auto cu) {
-        k_residual<Q, S, ex.value, cu.value><<<blocks, threads, 0, st>>>((const T*)P, c.cls, c.geo, kp_of<S>(c), vref,
-                                                                         update, partials, ro);
+        return launch_pdl(k_residual<Q, S, ex.value, cu.value>, blocks, threads, 0, st, (const T*)P, c.cls, c.geo,
+                          kp_of<S>(c), vref, update, partials, ro);
     });
 }
 
@@ -1797,9 +1791,10 @@ cudaError_t launch_stress(const Ctx& c, const void* cur, const void* prev, int v
     const long long N = (long long)c.geo.nx * c.geo.ny * c.geo.nz;
     const int blocks = grid_for(N, NODE_THREADS, 65535ll * 16);
     return with_ext_curved(c, [&](auto ex, auto cu) {
-        k_stress<Q, S, ex.value, cu.value><<<blocks, NODE_THREADS, 0, st>>>(
-            (const T*)cur, (const T*)prev, c.cls, c.geo, with_mag(kp_of<S>(c), c.cfg.induced ? c.mag[c.cur] : nullptr),
-            variant, (R*)sig, (R*)Sv, (R*)rho, (R*)v);
+        return launch_pdl(k_stress<Q, S, ex.value, cu.value>, blocks, NODE_THREADS, 0, st, (const T*)cur,
+                          (const T*)prev, c.cls, c.geo,
+                          with_mag(kp_of<S>(c), c.cfg.induced ? c.mag[c.cur] : nullptr), variant, (R*)sig, (R*)Sv,
+                          (R*)rho, (R*)v);
     });
 }
 

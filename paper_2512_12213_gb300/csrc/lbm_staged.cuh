@@ -365,6 +365,7 @@ k_step_staged(const typename S::T* __restrict__ src, typename S::T* __restrict__
     using Rt = typename S::R;
     static_assert(sizeof(Rt) == 4, "the staged step computes in FP32");
     constexpr bool PAIRX = EXT && !LP && FACES && sizeof(T) == 4;
+    pdl_trigger();
     extern __shared__ __align__(128) unsigned char smem[];
     const size_t stage_bytes = stg_stage_bytes(Q, R, g.nxp, sizeof(T));
     uint64_t* full = reinterpret_cast<uint64_t*>(smem + (size_t)nstages * stage_bytes);
@@ -373,6 +374,7 @@ k_step_staged(const typename S::T* __restrict__ src, typename S::T* __restrict__
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // the barrier protocol needs an even number of stages (see above)
     if (nstages < 2 || (nstages & 1) || nstages > STG_MAX_STAGES) {
+        pdl_wait();
         if (threadIdx.x == 0) atomicOr(errflag, STG_ERR_CONFIG);
         return;
     }
@@ -386,6 +388,7 @@ k_step_staged(const typename S::T* __restrict__ src, typename S::T* __restrict__
         mbar_fence_init();
     }
     __syncthreads();
+    pdl_wait(src);
     const int my_tiles = ((int)blockIdx.x < ntiles) ? (ntiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
 
     if (warp == STG_CWARPS) {

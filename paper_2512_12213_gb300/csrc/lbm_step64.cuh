@@ -190,16 +190,16 @@ constexpr int STEP64_THREADS = 128;
 template <int Q, bool EXT, bool FULL>
 __global__ void __launch_bounds__(STEP64_THREADS, 4)
 k_step64(const double* __restrict__ src, double* __restrict__ dst, const uint8_t* __restrict__ cls, const Geo g,
-         const KP<double> p, int zero_pad)
+         const KP<double> p, int zero_pad, int late)
 {
     const unsigned n = blockIdx.x * blockDim.x + threadIdx.x;
     const bool active = n < (unsigned)g.sq;      // the same for 64 threads: the padded node count is a multiple of 64
-    if (!(EXT && FULL) && !active) return;
     const unsigned r = n / (unsigned)g.nxp;
     const int x = (int)(n - r * (unsigned)g.nxp);
     const int z = (int)(r / (unsigned)g.ny), y = (int)(r - (unsigned)z * (unsigned)g.ny);
     const uint8_t c = active ? cls[n] : (uint8_t)NC_PAD;
     double v[3] = {0.0, 0.0, 0.0};
+    if (!late) pdl_wait(src);          // late: as in k_step
     if (c == NC_PAD || nc_solid(c)) {
         if (active && (c != NC_PAD || zero_pad))
 #pragma unroll
@@ -211,6 +211,10 @@ k_step64(const double* __restrict__ src, double* __restrict__ dst, const uint8_t
 #pragma unroll
         for (int k = 0; k < 3; ++k) aeb[k] = (FULL && p.aeb_dev) ? p.aeb_dev[k] : p.AEB[k];
         node_update64<Q, EXT>(d, p, aeb, v);
+        // not earlier: blocks of the next step that are placed while this one
+        // computes crowd some SMs' FP64 pipes (Hartmann 256 x 128: 27 us a
+        // step with the trigger at entry, 8.9 here, 11.0 without)
+        pdl_trigger();
 #pragma unroll
         for (int a = 0; a < Q; ++a) dst[(long long)a * g.sq + n] = d[a];
     }
@@ -233,6 +237,7 @@ k_step64(const double* __restrict__ src, double* __restrict__ dst, const uint8_t
                 for (int k = 0; k < 3; ++k) p.ins_rows[(long long)(n >> 6) * 3 + k] = v[k] + half[w >> 1][k];
         }
     }
+    if (late) pdl_wait();
 }
 
 // blocks of one warp (insulating walls: two) until every SM has the 20 warps
@@ -243,13 +248,14 @@ cudaError_t launch_step64(const Ctx& c, const void* src, void* dst, int zero_pad
     const bool full = c.cfg.curved || c.insulating;
     const int threads = c.geo.sq < 640ll * c.sm_count ? (full ? 64 : 32) : STEP64_THREADS;
     const unsigned blocks = (unsigned)((c.geo.sq + threads - 1) / threads);
-    auto go = [&](auto ex, auto full) {
-        k_step64<Q, ex.value, full.value><<<blocks, threads, 0, st>>>((const double*)src, (double*)dst, c.cls, c.geo,
-                                                                      c.kpd, zero_pad);
+    auto go = [&](auto ex, auto fu) {
+        return launch_pdl(k_step64<Q, ex.value, fu.value>, blocks, threads, 0, st, (const double*)src, (double*)dst,
+                          c.cls, c.geo, c.kpd, zero_pad, c.late_wait ? 1 : 0);
     };
-    if (c.ext) full ? go(std::true_type{}, std::true_type{}) : go(std::true_type{}, std::false_type{});
-    else full ? go(std::false_type{}, std::true_type{}) : go(std::false_type{}, std::false_type{});
-    return cudaGetLastError();
+    const std::true_type yes{};
+    const std::false_type no{};
+    if (c.ext) return full ? go(yes, yes) : go(yes, no);
+    return full ? go(no, yes) : go(no, no);
 }
 
 }  // namespace lbm
