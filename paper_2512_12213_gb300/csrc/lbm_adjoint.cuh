@@ -22,15 +22,18 @@ template <typename R> struct AdjConst {
 // plus the drag seed through a link into the target wall; then
 // phi_b = (1 - om) psi_b + A_rho + E_b . B_j, where A_rho and B_j collect the
 // derivatives of G = f^eq/tau + F with respect to rho and j, formed from the
-// weighted moments s0 = sum w psi, s1 = sum w psi E, s2 = sum w psi E E.
-// One node per thread, psi in registers.  Bulk nodes (every link to a fluid
-// node, periodic wrap allowed) address their neighbours through nine
-// precomputed row offsets and three x positions, without branches; nodes
-// next to a wall or a closed face take the general path.  Gradient terms are
-// summed per thread in the compute precision and per block in FP64.
-// blocks of RED_THREADS per SM: FP64 1; FP32 compute D3Q19 3 (80 registers,
-// a few dozen bytes of spill; 18% faster than 2 blocks at 126 registers on
-// the 128^3 sphere), D2Q9 2 (the 512 x 256 cylinder ran 23% slower at 3)
+// weighted moments s0 = sum w psi, s1 = sum w psi E, s2 = sum w psi E E, which
+// like the state's moments come from the sums and differences of the opposite
+// pairs, each speed class weighted once.  One node per thread, psi in
+// registers.  Bulk nodes (every link to a fluid node, periodic wrap allowed)
+// address their neighbours without branches; nodes next to a wall or a closed
+// face load their sources' class bytes together and then the values.  Bound by
+// memory: 128^3 FP32 117 us a step before the pairs (940 instructions a node)
+// -> 76, of 71 for its bytes.  Gradient terms are summed per thread
+// in the compute precision and per block in FP64.
+// blocks of RED_THREADS per SM: FP64 1; FP32 compute D3Q19 3 (80 registers;
+// 18% faster than 2 blocks at 126 registers on the 128^3 sphere), D2Q9 2 (the
+// 512 x 256 cylinder ran 23% slower at 3)
 template <int Q, class S>
 __global__ void __launch_bounds__(RED_THREADS, sizeof(typename S::R) == 8 ? 1 : (Q == 19 ? 3 : 2))
 k_adjoint(const typename S::T* __restrict__ Pprev, const typename S::R* __restrict__ phin,
@@ -41,96 +44,113 @@ k_adjoint(const typename S::T* __restrict__ Pprev, const typename S::R* __restri
     pdl_trigger();
     pdl_wait(Pprev, phin);
     using R = typename S::R;
-    constexpr int D = LatDim<Q>::D;
+    using T = typename S::T;
+    constexpr int D = LatDim<Q>::D, NP = LatDim<Q>::NP;
     __shared__ double sm[6 * 32];
     R accg[3] = {0, 0, 0}, accw[3] = {0, 0, 0};
-    const long long NP = (long long)g.nxp * g.ny * g.nz;
     // node indices fit in 32 bits (the padded node count is below 2^31)
     const unsigned nxp = (unsigned)g.nxp, ny = (unsigned)g.ny;
-    for (long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x; n < NP; n += (long long)gridDim.x * blockDim.x) {
-        const unsigned un = (unsigned)n, ur = un / nxp;
-        const int x = (int)(un - ur * nxp);
+    for (unsigned n = blockIdx.x * blockDim.x + threadIdx.x; n < (unsigned)g.sq; n += gridDim.x * blockDim.x) {
+        const unsigned ur = n / nxp;
+        const int x = (int)(n - ur * nxp);
         const int z = (int)(ur / ny), y = (int)(ur - (unsigned)z * ny);
         const uint8_t cl = cls[n];
-        if (x >= g.nx || nc_solid(cl) || cl == NC_PAD) {
+        if (nc_solid(cl) || cl == NC_PAD) {
 #pragma unroll
             for (int a = 0; a < Q; ++a) phio[(long long)a * g.sq + n] = R(0);
             continue;
         }
-        Mom<R> mo;
-        mom_zero(mo);
-        R psi[Q];
+        R psi[Q], d[Q];
+        const Around<Q> ar(g, x, y, z);          // x + E_a is the source of opp(a)
         if (cl == NC_BULK) {
-            // rows (y + dy, z + dz) and x +- 1, wrapped (bulk nodes wrap only on periodic axes)
-            unsigned rows[3][3];
+            T v[Q];
 #pragma unroll
-            for (int dy = -1; dy <= 1; ++dy)
+            for (int a = 0; a < Q; ++a) v[a] = Pprev[(long long)a * g.sq + ar.at(a)];
 #pragma unroll
-                for (int dz = -1; dz <= 1; ++dz) {
-                    const int yy = wrapi(y + dy, g.ny);
-                    const int zz = (Q == 19) ? wrapi(z + dz, g.nz) : 0;
-                    rows[dy + 1][dz + 1] = ((unsigned)zz * ny + (unsigned)yy) * nxp;
-                }
-            const unsigned xs[3] = {(unsigned)(x == 0 ? g.nx - 1 : x - 1), (unsigned)x,
-                                    (unsigned)(x == g.nx - 1 ? 0 : x + 1)};
-            auto at = [&](int ex, int ey, int ez) -> unsigned { return rows[ey + 1][ez + 1] + xs[ex + 1]; };
+            for (int a = 0; a < Q; ++a) psi[a] = phin ? phin[(long long)a * g.sq + ar.at(OPP<Q>(a))] : R(0);
 #pragma unroll
-            for (int a = 0; a < Q; ++a)
-                mom_add<R, Q, false>(mo, a, S::to_r(Pprev[(long long)a * g.sq + at(-EX<Q>(a), -EY<Q>(a), -EZ<Q>(a))]));
-#pragma unroll
-            for (int a = 0; a < Q; ++a) psi[a] = phin ? phin[(long long)a * g.sq + at(EX<Q>(a), EY<Q>(a), EZ<Q>(a))] : R(0);
+            for (int a = 0; a < Q; ++a) d[a] = S::to_r(v[a]);
         } else {
+            uint8_t cs[Q];
 #pragma unroll
-            for (int a = 0; a < Q; ++a) {
-                R v;
-                long long sidx;
-                int wall;
-                if (a == 0) v = S::to_r(Pprev[n]);
-                else if (pull_source(g, cls, x, y, z, EX<Q>(a), EY<Q>(a), EZ<Q>(a), sidx, wall))
-                    v = S::to_r(Pprev[(long long)a * g.sq + sidx]);
-                else
-                    v = S::to_r(Pprev[(long long)OPP<Q>(a) * g.sq + n]) + ladd_of<Q, R>(p, a, wall);
-                mom_add<R, Q, false>(mo, a, v);
+            for (int b = 1; b < Q; ++b) cs[b] = ar.out(b) ? nc_make_solid(ar.face(g, b)) : cls[ar.at(b)];
+            d[0] = S::to_r(Pprev[n]);
+            psi[0] = phin ? phin[n] : R(0);
+#pragma unroll
+            for (int b = 1; b < Q; ++b) {
+                const int a = OPP<Q>(b);
+                const bool hit = nc_solid(cs[b]);
+                d[b] = S::to_r(Pprev[hit ? (long long)a * g.sq + n : (long long)b * g.sq + ar.at(b)]);
+                psi[a] = phin ? phin[hit ? (long long)b * g.sq + n : (long long)a * g.sq + ar.at(b)] : R(0);
             }
 #pragma unroll
-            for (int a = 0; a < Q; ++a) {
-                long long dn;
-                int wall;
-                if (a == 0) {
-                    psi[0] = phin ? phin[n] : R(0);
-                } else if (pull_source(g, cls, x, y, z, EX<Q>(OPP<Q>(a)), EY<Q>(OPP<Q>(a)), EZ<Q>(OPP<Q>(a)), dn,
-                                       wall)) {
-                    psi[a] = phin ? phin[(long long)a * g.sq + dn] : R(0);
-                } else {
-                    const R back = phin ? phin[(long long)OPP<Q>(a) * g.sq + n] : R(0);
-                    psi[a] = back;
-                    if (wall == target) {
-                        psi[a] += ac.seed[a];
-                        // u_w enters f(t+1) and F_t through the Ladd term
-                        const R gl = ac.gl[a] * (back + R(0.5) * ac.seed[a]);
-                        accw[0] += gl * R(EX<Q>(a));
-                        accw[1] += gl * R(EY<Q>(a));
-                        accw[2] += gl * R(EZ<Q>(a));
-                    }
+            for (int b = 1; b < Q; ++b) {
+                const int a = OPP<Q>(b);
+                if (!nc_solid(cs[b])) continue;
+                const int wall = nc_wall(cs[b]);
+                d[b] += ladd_of<Q, R>(p, b, wall);
+                if (wall == target) {
+                    // u_w enters f(t+1) and F_t through the Ladd term
+                    const R gl = ac.gl[a] * (psi[a] + R(0.5) * ac.seed[a]);
+                    psi[a] += ac.seed[a];
+                    accw[0] += gl * R(EX<Q>(a));
+                    accw[1] += gl * R(EY<Q>(a));
+                    accw[2] += gl * R(EZ<Q>(a));
                 }
             }
         }
         NodeM<R> m;
-        macro_from_moments<R, Q, false>(mo, p, m);
-        // omega-weighted moments of psi
-        R s0 = 0, s1[3] = {0, 0, 0}, s2[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
+        {
+            Mom<R> mo;
+            mom_zero(mo);
+            mo.drho = d[0];
 #pragma unroll
-        for (int a = 0; a < Q; ++a) {
-            const R wp = R(WD<Q>(a)) * psi[a];
-            const int e[3] = {EX<Q>(a), EY<Q>(a), EZ<Q>(a)};
-            s0 += wp;
+            for (int k = 0; k < NP; ++k) {
+                const int a = PAIR<Q>(k), b = OPP<Q>(a);
+                const int e[3] = {EX<Q>(a), EY<Q>(a), EZ<Q>(a)};
+                const R df = d[a] - d[b];
+                mo.drho += d[a] + d[b];
 #pragma unroll
-            for (int i = 0; i < D; ++i) {
-                if (e[i]) s1[i] += R(e[i]) * wp;
-#pragma unroll
-                for (int j = 0; j < D; ++j)
-                    if (e[i] * e[j]) s2[i][j] += R(e[i] * e[j]) * wp;
+                for (int c = 0; c < 3; ++c)
+                    if (e[c]) mo.j[c] = e[c] > 0 ? mo.j[c] + df : mo.j[c] - df;
             }
+            macro_from_moments<R, Q, false>(mo, p, m);
+        }
+        // weighted moments of psi: per speed class, then w_axis and w_diag
+        R s0, s1[3], s2[3][3];
+        {
+            constexpr R wa = R(WD<Q>(1)), wd = R(WD<Q>(Q == 9 ? 5 : 7));
+            R ax = R(0), dg = R(0), j2[3] = {R(0), R(0), R(0)}, p2[3] = {R(0), R(0), R(0)}, x2[3] = {R(0), R(0), R(0)};
+            R j1[3] = {R(0), R(0), R(0)}, p1[3] = {R(0), R(0), R(0)};
+#pragma unroll
+            for (int k = 0; k < NP; ++k) {
+                const int a = PAIR<Q>(k), b = OPP<Q>(a);
+                const int e[3] = {EX<Q>(a), EY<Q>(a), EZ<Q>(a)};
+                const R sp = psi[a] + psi[b], df = psi[a] - psi[b];
+                if (SPEED2<Q>(a) == 1) {
+                    const int c = e[0] ? 0 : (e[1] ? 1 : 2);
+                    ax += sp;
+                    p1[c] = sp;
+                    j1[c] = e[c] > 0 ? df : -df;
+                } else {
+                    const int i = e[0] ? 0 : 1, j = e[2] ? 2 : 1, q = i == 1 ? 2 : (j == 2 ? 1 : 0);   // xy xz yz
+                    dg += sp;
+                    p2[i] += sp;
+                    p2[j] += sp;
+                    x2[q] = e[i] * e[j] > 0 ? x2[q] + sp : x2[q] - sp;
+                    j2[i] = e[i] > 0 ? j2[i] + df : j2[i] - df;
+                    j2[j] = e[j] > 0 ? j2[j] + df : j2[j] - df;
+                }
+            }
+            s0 = R(WD<Q>(0)) * psi[0] + wa * ax + wd * dg;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                s1[c] = wa * j1[c] + wd * j2[c];
+                s2[c][c] = wa * p1[c] + wd * p2[c];
+            }
+            s2[0][1] = s2[1][0] = wd * x2[0];
+            s2[0][2] = s2[2][0] = wd * x2[1];
+            s2[1][2] = s2[2][1] = wd * x2[2];
         }
         // sum psi f^eq(rho, W) = rho Psi_e(W); grad_W = rho (3 s1 + 9 s2 W - 3 s0 W)
         // sum psi F = C rho Psi_f; grad_Wf = C rho (9 s2 A - 3 s0 A); grad_A = C rho (3 s1 - 3 s0 Wf + 9 s2 Wf)
@@ -177,11 +197,19 @@ k_adjoint(const typename S::T* __restrict__ Pprev, const typename S::R* __restri
             Arho -= (Ge[i] + Gf[i]) * m.u[i] * ir;
             Bj[i] = (Ge[i] + Gf[i]) * ir;
         }
+        const R om1 = R(1) - m.om;
+        phio[n] = fma(om1, psi[0], Arho);
 #pragma unroll
-        for (int b = 0; b < Q; ++b) {
-            const R phib = (R(1) - m.om) * psi[b] + Arho + R(EX<Q>(b)) * Bj[0] + R(EY<Q>(b)) * Bj[1] +
-                           R(EZ<Q>(b)) * Bj[2];
-            phio[(long long)b * g.sq + n] = phib;
+        for (int k = 0; k < NP; ++k) {
+            const int a = PAIR<Q>(k), b = OPP<Q>(a);
+            R t = R(0);
+#pragma unroll
+            for (int c = 0; c < D; ++c) {
+                const int e = c == 0 ? EX<Q>(a) : (c == 1 ? EY<Q>(a) : EZ<Q>(a));
+                if (e) t = e > 0 ? t + Bj[c] : t - Bj[c];
+            }
+            phio[(long long)a * g.sq + n] = fma(om1, psi[a], Arho + t);
+            phio[(long long)b * g.sq + n] = fma(om1, psi[b], Arho - t);
         }
         // dJ/dg: A = dt g / c; W^eq moves with A/2 for [e]; W^F with tau/2 ([c]) or 1/2 ([d], [e])
         const R keq = (p.model == MODEL_E) ? R(0.5) : R(0);

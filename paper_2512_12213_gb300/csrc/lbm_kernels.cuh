@@ -50,27 +50,41 @@ template <class T> __device__ __forceinline__ T shfl_down1(T v)
     }
 }
 
-// sum W doubles over the block; thread 0 gets the totals in out[]
+// sum W doubles over the block; thread 0 gets the totals in v[].  The FP64
+// pipe takes a warp addition in ~19 cycles, so the values are reduced
+// together: the first steps halve the values a lane carries along with the
+// lanes that carry them (9 additions a warp for 8 values, not 40).
 template <int W>
 __device__ __forceinline__ void block_sum(double (&v)[W], double* smem /* >= W * 32 */)
 {
-#pragma unroll
-    for (int k = 0; k < W; ++k)
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
+    constexpr int P = W <= 2 ? 2 : (W <= 4 ? 4 : 8), G = 32 / P;
+    static_assert(W <= 8, "at most 8 values");
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-    if (lane == 0)
+    double t[P];
 #pragma unroll
-        for (int k = 0; k < W; ++k) smem[k * 32 + wid] = v[k];
+    for (int k = 0; k < P; ++k) t[k] = k < W ? v[k] : 0.0;
+#pragma unroll
+    for (int n = P / 2; n >= 1; n /= 2) {
+        const int o = n * G;                     // 16, 8, ...
+        const bool up = lane & o;
+#pragma unroll
+        for (int i = 0; i < n; ++i) {
+            const double keep = up ? t[i + n] : t[i], send = up ? t[i] : t[i + n];
+            t[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+    }
+#pragma unroll
+    for (int o = G / 2; o > 0; o /= 2) t[0] += __shfl_xor_sync(0xffffffffu, t[0], o);
+    const int k = lane / G, sub = lane % G;      // this lane's value
+    if (sub == 0 && k < W) smem[k * 32 + wid] = t[0];
     __syncthreads();
     if (wid == 0) {
+        double s = 0.0;
+        for (int j = sub; j < nw; j += G) s += k < W ? smem[k * 32 + j] : 0.0;
 #pragma unroll
-        for (int k = 0; k < W; ++k) {
-            double s = (lane < nw) ? smem[k * 32 + lane] : 0.0;
+        for (int o = G / 2; o > 0; o /= 2) s += __shfl_xor_sync(0xffffffffu, s, o);
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-            v[k] = s;
-        }
+        for (int i = 0; i < W; ++i) v[i] = __shfl_sync(0xffffffffu, s, i * G);
     }
 }
 
@@ -1221,7 +1235,7 @@ k_balance(const typename S::T* __restrict__ P, const uint8_t* __restrict__ cls, 
 // node's v replaces v_ref (each thread reads its own entries before it writes
 // them; solid nodes get 0).
 template <int Q, class S, bool EXT, bool CURVED>
-__global__ void __launch_bounds__(RED_THREADS)
+__global__ void __launch_bounds__(RED_THREADS, 3)
 k_residual(const typename S::T* __restrict__ P, const uint8_t* __restrict__ cls, const Geo g,
            const KP<typename S::R> p, double* __restrict__ vref, int update, double* __restrict__ partials,
            const RedOut ro)
@@ -1725,16 +1739,14 @@ cudaError_t launch_export(const Ctx& c, const void* P, void* out, int dtype, cud
     });
 }
 
-// grid of a reduction over nodes: at most the two blocks per SM that its
-// registers allow at once, so that there is no second wave and each block's
-// FP64 tail (~1.3 us of an SM's FP64 pipe) is paid twice an SM; fewer threads
-// per block, a warp at least, where a box is too small for a block of 256
-// nodes on every SM
-inline int red_grid(const Ctx& c, long long N, int& threads)
+// grid of a reduction over nodes: at most the blocks per SM that its registers
+// allow at once, so that there is no second wave; fewer threads per block, a
+// warp at least, where a box is too small for a block of 256 nodes on every SM
+inline int red_grid(const Ctx& c, long long N, int per_sm, int& threads)
 {
     threads = RED_THREADS;
     while (threads > 32 && N < (long long)threads * c.sm_count) threads /= 2;
-    const long long most = N / (8ll * threads) > c.sm_count ? 2ll * c.sm_count : c.sm_count;
+    const long long most = N / (8ll * threads) > c.sm_count ? (long long)per_sm * c.sm_count : c.sm_count;
     return grid_for(N, threads, std::min<long long>(MAX_PARTIAL_ROWS, most));
 }
 
@@ -1760,7 +1772,7 @@ cudaError_t launch_balance(const Ctx& c, const void* P, double* partials, const 
     using T = typename S::T;
     const long long N = (long long)c.geo.nx * c.geo.ny * c.geo.nz;
     int threads;
-    const int blocks = red_grid(c, N, threads);
+    const int blocks = red_grid(c, N, 2, threads);
     const double vol = (Q == 9) ? c.cfg.dx * c.cfg.dx : c.cfg.dx * c.cfg.dx * c.cfg.dx;
     return with_ext_curved(c, [&](auto ex, auto cu) {
         return launch_pdl(k_balance<Q, S, ex.value, cu.value>, blocks, threads, 0, st, (const T*)P, c.cls, c.geo,
@@ -1775,7 +1787,7 @@ cudaError_t launch_residual(const Ctx& c, const void* P, double* vref, int updat
     using T = typename S::T;
     const long long N = (long long)c.geo.nx * c.geo.ny * c.geo.nz;
     int threads;
-    const int blocks = red_grid(c, N, threads);
+    const int blocks = red_grid(c, N, 3, threads);
     return with_ext_curved(c, [&](auto ex, auto cu) {
         return launch_pdl(k_residual<Q, S, ex.value, cu.value>, blocks, threads, 0, st, (const T*)P, c.cls, c.geo,
                           kp_of<S>(c), vref, update, partials, ro);
