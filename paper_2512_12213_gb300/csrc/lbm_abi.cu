@@ -450,7 +450,7 @@ void fill_params(Ctx& x)
 // shape of the staged step: tiles of R rows such that each direction's copy
 // moves at least 2 KB (R nxp = 1024 nodes for 16-bit storage, 512 for FP32:
 // a bulk copy costs the copy engine a fixed time, so small copies starve the
-// pipeline), and as many stages (an even count, 4..8) as the shared memory
+// pipeline), and as many stages (4..8) as the shared memory
 // holds; stage_R = 0
 // where the kernel does not apply, was not asked for, or fewer than 4 stages
 // fit (rows of more than ~1,100 16-bit or ~550 FP32 nodes): the
@@ -481,8 +481,8 @@ void choose_stage(Ctx& x)
                                                             (size_t)x.cfg.ny));
     const size_t stage = stg_stage_bytes((int)Q, R, (int)nxp, (int)x.elem);
     const size_t budget = (size_t)x.smem_optin - 1024;
-    // an even count: each consumer group owns every other stage
-    const int n = (int)std::min<size_t>(8, budget / (stage + 2 * sizeof(uint64_t))) & ~1;
+    int n = (int)std::min<size_t>(STG_MAX_STAGES, budget / (stage + 2 * sizeof(uint64_t)));
+    n -= n % (x.ext ? StgShape<true>::G : StgShape<false>::G);      // every stage belongs to one consumer group
     if (n < 4) return;
     const long long tiles = (long long)((x.cfg.ny + R - 1) / R) * x.cfg.nz;
     // automatic choice with closed faces or the EXT node code (longer tiles):

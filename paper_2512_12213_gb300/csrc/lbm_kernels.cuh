@@ -1635,7 +1635,7 @@ cudaError_t launch_step_staged_k(const Ctx& c, const void* src, void* dst, uint3
         if (e != cudaSuccess) return e;
         c.stage_ready = true;
     }
-    return launch_pdl(kern, staged_blocks(c), 32 * staged_warps(c.n_special, c.geo.sq, !c.geo.periodic[0]),
+    return launch_pdl(kern, staged_blocks(c), 32 * staged_warps(StgShape<EXT>::CW, c.n_special, c.geo.sq, !c.geo.periodic[0]),
                       c.stage_smem, st, (const T*)src, (T*)dst, c.cls, c.special, c.n_special, c.geo, kp_step_of<S>(c),
                       seed, c.stage_R, (int)c.stage_tiles, c.stage_n, zero_padding(c, dst), c.errflag, fw);
 }

@@ -19,15 +19,15 @@
 // stores, which cost the copy engine nothing.
 //
 // One producer warp keeps up to 8 stages in flight (lane a copies direction
-// a): it refills a stage as soon as the consumer warps that read it have
-// released it (full / empty mbarriers, the full one with the copies'
-// transaction bytes).  Consumer warps form two groups that take alternate
-// tiles.  The stage count is even, so tile k uses stage k mod n and every
-// stage belongs to one group, which consumes its uses in order: a warp can
-// then only wait on the phase of a use whose predecessor its group has
-// finished, and a parity wait cannot mistake a phase two uses old for the
-// current one (with an odd count a stage alternates between the groups and
-// a group running ahead could do exactly that).  A thread relaxes one pair
+// a): it refills a stage as soon as the consumer warps have released it (full
+// / empty mbarriers, the full one with the copies' transaction bytes).  The
+// consumer warps form groups that take alternate tiles, a group's warps its
+// 64-node tasks in turn.  The number of stages is a multiple of the number of
+// groups, so every stage belongs to one group, and every warp of a group
+// waits for and releases each of its tiles, with a task in it or not: a warp
+// can then only wait on the use of a stage whose predecessor it has released
+// itself, and a parity wait cannot mistake a phase two uses old for the
+// current one.  A thread relaxes one pair
 // of nodes of a 64-node warp task at a time (one 32-bit word per direction
 // for 16-bit storage, one float2 for FP32) with k_step's node code for the
 // configuration.  Closed faces follow k_step: a source row outside a closed
@@ -53,25 +53,33 @@
 
 namespace lbm {
 
-constexpr int STG_GROUPS = 2;                         // consumer groups (alternate tiles)
-constexpr int STG_GROUP_WARPS = 8;                    // warps per group
-constexpr int STG_CWARPS = STG_GROUPS * STG_GROUP_WARPS;
-// boundary warps: one, or more where more than 0.5% of the chunks are special
-// (a ragged row has one in every row): at most the three, with a face warp
-// two, that still leave five warps on each of the SM's four sub-partitions,
-// so the register cap of 96 stays.  The kernel takes the number from its
-// block size.
-constexpr int STG_THREADS = 32 * (STG_CWARPS + 4);    // at most: consumers, producer, three others
-inline int staged_warps(long long n_special, long long nodes, bool closed_x)
+// Consumer warps, in G groups of W that take alternate tiles.  Without the EXT
+// terms two groups of 8: with the producer and up to three others that is
+// five warps on each of the SM's four sub-partitions, 96 registers, which the
+// plain node code fits, and while one group starts a tile the other is in the
+// middle of one (binary16 sphere 256 x 128 x 128 54.5 us; one group of 16
+// 58.1, of 12 55.0; bfloat16 250 x 121 x 99 54.1, 62.8, 61.1).  The LES and
+// EXT node codes spill at 96: one group of 12, four warps a sub-partition,
+// 128 registers (cavity 256^3: binary16 327 us against 334 for two groups of
+// 8, FP32 427 against 441; Brinkman box FP32 100 against 106).
+template <bool EXT> struct StgShape {
+    static constexpr int G = EXT ? 1 : 2, W = EXT ? 12 : 8;
+    static constexpr int CW = G * W;
+    static constexpr int MAXW = CW + 4;          // warps of a block at most
+};
+// boundary warps: one, or as many as the block may hold where more than 0.5%
+// of the chunks are special (a ragged row has one in every row).  The kernel
+// takes the number from its block size.
+inline int staged_warps(int cw, long long n_special, long long nodes, bool closed_x)
 {
-    return n_special * 200 > nodes / 4 ? STG_THREADS / 32 : STG_CWARPS + 2 + (closed_x ? 1 : 0);
+    return n_special * 200 > nodes / 4 ? cw + 4 : cw + 2 + (closed_x ? 1 : 0);
 }
 constexpr int STG_COPY_BYTES = 2048;                  // least bytes per direction and tile
 constexpr int STG_TASK_NODES = 64;                    // nodes per warp task (32 pairs)
 constexpr int STG_MAX_STAGES = 8;
 constexpr unsigned long long STG_WAIT_NS = 1000000000ull;   // bounded waits: 1 s
 constexpr unsigned STG_ERR_TIMEOUT = 1u;
-constexpr unsigned STG_ERR_CONFIG = 2u;                     // a launch with an odd stage count
+constexpr unsigned STG_ERR_CONFIG = 2u;                     // a launch with a stage count out of range
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -355,7 +363,7 @@ __device__ __forceinline__ void gather_periodic(const typename S::T* __restrict_
 // scalar EXT code node by node; LP: the FP32x2 pair code specialised for
 // LES (LES-only contexts).
 template <int Q, class S, bool SR, bool EXT = false, bool FACES = false, bool LP = false>
-__global__ void __launch_bounds__(STG_THREADS, 1)
+__global__ void __launch_bounds__(32 * StgShape<EXT>::MAXW, 1)
 k_step_staged(const typename S::T* __restrict__ src, typename S::T* __restrict__ dst,
               const uint8_t* __restrict__ cls, const uint32_t* __restrict__ special, long long nspecial, const Geo g,
               const KP<float> p, uint32_t seed, int R, int ntiles, int nstages, int zero_pad,
@@ -365,6 +373,7 @@ k_step_staged(const typename S::T* __restrict__ src, typename S::T* __restrict__
     using Rt = typename S::R;
     static_assert(sizeof(Rt) == 4, "the staged step computes in FP32");
     constexpr bool PAIRX = EXT && !LP && FACES && sizeof(T) == 4;
+    constexpr int G = StgShape<EXT>::G, W = StgShape<EXT>::W, CW = StgShape<EXT>::CW;
     pdl_trigger();
     extern __shared__ __align__(128) unsigned char smem[];
     const size_t stage_bytes = stg_stage_bytes(Q, R, g.nxp, sizeof(T));
@@ -372,8 +381,7 @@ k_step_staged(const typename S::T* __restrict__ src, typename S::T* __restrict__
     uint64_t* empty = full + nstages;
     const int nty = (g.ny + R - 1) / R;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    // the barrier protocol needs an even number of stages (see above)
-    if (nstages < 2 || (nstages & 1) || nstages > STG_MAX_STAGES) {
+    if (nstages < 2 || nstages % G || nstages > STG_MAX_STAGES) {    // every stage belongs to one group
         pdl_wait();
         if (threadIdx.x == 0) atomicOr(errflag, STG_ERR_CONFIG);
         return;
@@ -383,7 +391,7 @@ k_step_staged(const typename S::T* __restrict__ src, typename S::T* __restrict__
     if (threadIdx.x == 0) {
         for (int s = 0; s < nstages; ++s) {
             mbar_init(&full[s], face_warp ? 2 : 1);      // copies armed, and face values in
-            mbar_init(&empty[s], STG_GROUP_WARPS);
+            mbar_init(&empty[s], W);
         }
         mbar_fence_init();
     }
@@ -391,8 +399,8 @@ k_step_staged(const typename S::T* __restrict__ src, typename S::T* __restrict__
     pdl_wait(src);
     const int my_tiles = ((int)blockIdx.x < ntiles) ? (ntiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
 
-    if (warp == STG_CWARPS) {
-        // producer warp: refill a stage once the group that read it released it
+    if (warp == CW) {
+        // producer warp: refill a stage once every consumer warp released it
         int ey = 0, ez = 0, oa = 0;          // the pull shift and opposite of this lane's direction
 #pragma unroll
         for (int b = 0; b < Q; ++b)
@@ -424,7 +432,7 @@ k_step_staged(const typename S::T* __restrict__ src, typename S::T* __restrict__
         return;
     }
 
-    if (face_warp && warp == STG_CWARPS + 1) {
+    if (face_warp && warp == CW + 1) {
         // the face warp refills a stage's face values as the producer does its rows
         for (int k = 0; k < my_tiles; ++k) {
             const int s = k % nstages, use = k / nstages;
@@ -439,13 +447,13 @@ k_step_staged(const typename S::T* __restrict__ src, typename S::T* __restrict__
         return;
     }
 
-    if (warp > STG_CWARPS) {
+    if (warp > CW) {
         // boundary warps: the listed chunks, node by node (lane per node), and
         // the wall force of their links when asked for (each lane sums its
         // nodes in a fixed order, then a fixed shuffle tree, one row per warp)
         double acc[3] = {0.0, 0.0, 0.0};
         const long long nn = 4 * nspecial;
-        const int first = STG_CWARPS + 1 + (face_warp ? 1 : 0);
+        const int first = CW + 1 + (face_warp ? 1 : 0);
         const int per = (int)(blockDim.x >> 5) - first;                   // boundary warps of a block
         const int bw = (int)blockIdx.x * per + warp - first, nbw = (int)gridDim.x * per;
         if (zero_pad) {
@@ -513,30 +521,42 @@ k_step_staged(const typename S::T* __restrict__ src, typename S::T* __restrict__
         return;
     }
 
-    const int group = warp / STG_GROUP_WARPS, gw = warp % STG_GROUP_WARPS;
-    // a warp's tasks of a tile, gw, gw + 8, ...: row and task of the row
+    // a consumer warp's tasks: every W-th of its group's, R x tasks_per_row to
+    // a tile (row and task of the row, carried over the tiles)
+    const int group = warp / W, gw = warp % W;
     const int tasks_per_row = g.nxp / STG_TASK_NODES;
-    const int r_first = gw / tasks_per_row, xt_first = gw % tasks_per_row;
-    const int r_step = STG_GROUP_WARPS / tasks_per_row, xt_step = STG_GROUP_WARPS % tasks_per_row;
+    const int r_step = W / tasks_per_row, xt_step = W % tasks_per_row;
+    int r = gw / tasks_per_row, xt = gw % tasks_per_row;
     const long long sq = g.sq;
     const bool closed_x = FACES && !g.periodic[0];
-    for (int k = group; k < my_tiles; k += STG_GROUPS) {
-        const int s = k % nstages, use = k / nstages;
-        if (!mbar_wait_bounded(&full[s], (uint32_t)use & 1u)) {
+    auto advance = [&]() {
+        r += r_step;
+        xt += xt_step;
+        if (xt >= tasks_per_row) {
+            xt -= tasks_per_row;
+            ++r;
+        }
+    };
+    int s = group;
+    uint32_t phase = 0;
+    // plane and tile of the plane, stepped without divisions
+    const int t0 = (int)blockIdx.x + group * (int)gridDim.x;
+    int z = t0 / nty, ty = t0 - z * nty;
+    const int z_step = G * (int)gridDim.x / nty, ty_step = G * (int)gridDim.x - z_step * nty;
+    const size_t cls_off = stg_cls_off(Q, R, g.nxp, sizeof(T)), face_off = stg_face_off(Q, R, g.nxp, sizeof(T));
+    for (int k = group; k < my_tiles; k += G) {
+        if (!mbar_wait_bounded(&full[s], phase)) {
             if (lane == 0) atomicOr(errflag, STG_ERR_TIMEOUT);
             return;
         }
-        const int t = (int)blockIdx.x + k * (int)gridDim.x;
-        const int z = t / nty, y0 = (t - z * nty) * R;
+        const int y0 = ty * R;
         const int nr = min(R, g.ny - y0);
-        const T* sp = reinterpret_cast<const T*>(smem + (size_t)s * stage_bytes);
-        const uint8_t* sc = smem + (size_t)s * stage_bytes + stg_cls_off(Q, R, g.nxp, sizeof(T));
-        const T* fa = reinterpret_cast<const T*>(smem + (size_t)s * stage_bytes + stg_face_off(Q, R, g.nxp, sizeof(T)));
-        for (int r = r_first, xt = xt_first; r < nr; r += r_step, xt += xt_step) {
-            if (xt >= tasks_per_row) {
-                xt -= tasks_per_row;
-                if (++r >= nr) break;
-            }
+        const unsigned char* st = smem + (size_t)s * stage_bytes;
+        const T* sp = reinterpret_cast<const T*>(st);
+        const uint8_t* sc = st + cls_off;
+        const T* fa = reinterpret_cast<const T*>(st + face_off);
+        for (; r < R; advance()) {
+            if (r >= nr) continue;               // a ragged last tile
             const int x0 = xt * STG_TASK_NODES + 2 * lane;
             const int y = y0 + r;
             const long long base = ((long long)z * g.ny + y) * g.nxp + x0;
@@ -629,6 +649,18 @@ k_step_staged(const typename S::T* __restrict__ src, typename S::T* __restrict__
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(&empty[s]);     // this warp is done with stage s
+        r -= R;
+        z += z_step;
+        ty += ty_step;
+        if (ty >= nty) {
+            ty -= nty;
+            ++z;
+        }
+        s += G;
+        if (s >= nstages) {
+            s = group;
+            phase ^= 1u;
+        }
     }
 }
 
