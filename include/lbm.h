@@ -166,14 +166,18 @@ typedef struct lbm_config {
 
 /* Kernel of the fused step.  Both compute the same arithmetic and store the
  * same bits; they differ in how the pull sources reach the registers.
- * LBM_STEP_AUTO (0) picks the staged kernel for 16-bit storage wherever it
- * applies, enough shared memory holds its pipeline and at most 2% of the
- * 4-node chunks touch a solid or padding; else the register-tiled one.  LBM_STEP_REGISTER (1): every thread loads its vectors straight from
- * HBM.  LBM_STEP_STAGED (2): a persistent kernel stages each tile's source
+ * LBM_STEP_AUTO (0) picks the staged kernel, where it applies and its
+ * pipeline fits in shared memory, for 16-bit storage and for FP32 with any of
+ * the Lorentz force, Maxwell term, LES, linear equilibrium or Darcy
+ * resistance on D3Q19 (large boxes with insulating walls included), unless
+ * more than 4% (8% with one of those) of the 4-node chunks touch a solid or a
+ * ragged row end or the box is one of the few kinds that measured slower; else
+ * the register-tiled one.  LBM_STEP_REGISTER
+ * (1): every thread loads its vectors straight from HBM.  LBM_STEP_STAGED (2): a persistent kernel stages each tile's source
  * rows in shared memory with bulk asynchronous copies; it serves FP32 and
  * 16-bit storage with closed or periodic faces and every node code except
- * curved walls, insulating walls and the induced field (those: LBM_ERR_ARG);
- * where its pipeline does not fit in shared memory (rows of more than about
+ * curved walls, insulating walls and the induced field (asked for with one of
+ * those: LBM_ERR_ARG); where its pipeline does not fit in shared memory (rows of more than about
  * 1,100 16-bit or 550 FP32 nodes) the register-tiled kernel runs instead. */
 enum { LBM_STEP_AUTO = 0, LBM_STEP_REGISTER = 1, LBM_STEP_STAGED = 2 };
 

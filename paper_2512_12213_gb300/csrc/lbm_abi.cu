@@ -46,6 +46,14 @@ bool staged_applies(const lbm_config* c)
     return !c->curved && !c->insulating && !c->induced && c->storage != LBM_STORE_F64;
 }
 
+// insulating walls run it too where the automatic choice picks the kernel
+// (FP32, D3Q19): the step's velocity sums are then one row per warp
+bool staged_insulating(const lbm_config* c)
+{
+    return c->insulating && !c->curved && c->storage == LBM_STORE_F32 && c->lattice == LBM_D3Q19 &&
+           c->step_kernel == LBM_STEP_AUTO;
+}
+
 bool all_periodic(const lbm_config* c)
 {
     return c->periodic[0] && c->periodic[1] && (c->lattice == LBM_D2Q9 || c->periodic[2]);
@@ -237,7 +245,7 @@ long long ins_rows_of(const lbm_config* c)
 // the node buffer, after the class bytes
 bool keeps_special_list(const lbm_config* c)
 {
-    return c->step_kernel != LBM_STEP_REGISTER && staged_applies(c);
+    return c->step_kernel != LBM_STEP_REGISTER && (staged_applies(c) || staged_insulating(c));
 }
 
 void sizes_of(const lbm_config* c, long long n_links, long long n_special, size_t s[LBM_NUM_BUFFERS])
@@ -463,18 +471,22 @@ void choose_stage(Ctx& x)
     x.stage_smem = 0;
     x.stage_ready = false;
     if (!keeps_special_list(&x.cfg)) return;
-    // automatic choice: the boundary warps keep pace while at most 2% of the
-    // chunks are special (a sphere or a few bodies in a periodic box); boxes
-    // full of small solids go to the register-tiled kernel
-    if (x.cfg.step_kernel == LBM_STEP_AUTO && x.n_special * 50 > x.geo.sq / 4) return;
-    // ... and 16-bit storage: with FP32 the register-tiled kernel already
-    // keeps enough bytes in flight (measured on the sphere box: 0.84 of HBM
-    // against 0.81 staged), with 16-bit it does not (0.52 against 0.80)
-    if (x.cfg.step_kernel == LBM_STEP_AUTO && x.elem != 2) return;
-    // (with 16-bit storage the staged kernel also wins with closed faces and
-    // the EXT node code: LES cavity 256^3, binary16 with stochastic rounding,
-    // 28.5k against 23.7k MLUPS; with FP32 it loses there too, 20.2k against
-    // 26.7k)
+    // automatic choice, from both kernels' steps on GB300 (us, register-tiled
+    // / staged).  The boundary warps keep pace with 4% of special chunks (a
+    // sphere or a few bodies, ragged row ends), with 8% beside the longer LES
+    // and EXT node codes: sphere 67 x 60 x 61 with 3.1% binary16 14.3 / 12.2,
+    // 99 x 100 x 101 37.3 / 26.5, 41 x 24 x 25 with 6.3% binary16 5.9 / 5.9, FP32
+    // 6.0 / 6.6; cavity 41^3 with 6.3% binary16 15.8 / 8.8, FP32 11.3 / 8.1.
+    // Boxes full of small solids go to the register-tiled kernel.
+    const bool automatic = x.cfg.step_kernel == LBM_STEP_AUTO, d3 = x.cfg.lattice == LBM_D3Q19;
+    if (automatic && x.n_special * (x.ext ? 25 : 50) > 2 * (x.geo.sq / 4)) return;
+    // FP32 without the EXT terms: the register-tiled kernel keeps enough bytes
+    // in flight (sphere 256 x 128 x 128 97.8 / 111) unless the rows are ragged
+    // and short (more than 2%: 130 x 96 x 96 53.5 / 44.7, 67 x 60 x 61 13.5 /
+    // 11.8; below, 250 x 121 x 99 88.7 / 94.5).  With them it holds too few
+    // warps (cavity 256^3 502 / 427, 64^3 12.3 / 10.7, 32^3 7.9 / 5.3; Brinkman
+    // box 256 x 128 x 128 123 / 100).  D2Q9 stays.
+    if (automatic && x.elem != 2 && !(d3 && (x.ext || x.n_special * 50 > x.geo.sq / 4))) return;
     const size_t Q = x.cfg.lattice, nxp = x.geo.nxp;
     const size_t row_bytes = nxp * x.elem;
     const int R = (int)std::max<size_t>(1, std::min<size_t>((STG_COPY_BYTES + row_bytes - 1) / row_bytes,
@@ -485,12 +497,24 @@ void choose_stage(Ctx& x)
     n -= n % (x.ext ? StgShape<true>::G : StgShape<false>::G);      // every stage belongs to one consumer group
     if (n < 4) return;
     const long long tiles = (long long)((x.cfg.ny + R - 1) / R) * x.cfg.nz;
-    // automatic choice with closed faces or the EXT node code (longer tiles):
-    // at least 16 tiles per block, else the tail of the persistent grid costs
-    // more than the pipeline gains (LES cavity 128^3: 13 tiles per block,
-    // 16.0k staged against 19.6k MLUPS register-tiled)
-    const bool long_tiles = !all_periodic(&x.cfg) || x.ext;
-    if (x.cfg.step_kernel == LBM_STEP_AUTO && long_tiles && tiles < 16ll * x.sm_count) return;
+    // closed faces or the EXT terms with 16-bit storage: D2Q9 (256 x 128
+    // channel 2.8 / 3.5) and the scalar EXT code in a box without ragged rows
+    // (Brinkman 96 x 64 x 64 15.8 / 17.9, 256 x 128 x 128 112 / 96) need 16 tiles
+    // per block; LES and plain node codes do not (cavity binary16 128^3 80.5 /
+    // 49.5, 64^3 10.8 / 10.6, 32^3 10.2 / 7.5)
+    const bool scalar = x.ext && !x.les_pair && x.n_special * 200 <= x.geo.sq / 4;
+    const bool long_tiles = d3 ? scalar : (!all_periodic(&x.cfg) || x.ext);
+    if (automatic && x.elem == 2 && long_tiles && tiles < 16ll * x.sm_count) return;
+    if (x.insulating) {
+        // from 16 tiles per block (256 x 128 x 128 139 / 121, 130 x 96 x 96 86 / 77,
+        // 96 x 64 x 64 26 / 34); the velocity rows of the staged warps have to
+        // fit the scratch of the register step's
+        if (tiles < 16ll * x.sm_count) return;
+        const long long blocks = std::min<long long>(tiles, x.sm_count);
+        const long long rows = blocks * staged_warps(StgShape<true>::CW, x.n_special, x.geo.sq, !x.geo.periodic[0]);
+        if (rows > x.ins_rows) return;
+        x.ins_rows = rows;
+    }
     x.stage_R = R;
     x.stage_n = n;
     x.stage_tiles = tiles;

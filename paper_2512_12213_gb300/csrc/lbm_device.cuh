@@ -389,9 +389,11 @@ template <typename R> __device__ __forceinline__ void mom_zero(Mom<R>& mo)
 // the per-node quantities of the text after Eq. (1) and the per-model
 // choices of C, u^F and u^eq of Sec. 2, from the raw moments; EXT enables
 // the Lorentz force and LES; INS reads the Lorentz coefficient of insulating
-// walls from the device (kernels that never serve them compile without it)
+// walls from the device (kernels that never serve them compile without it),
+// or from `ins` where the caller holds it
 template <typename R, int Q, bool EXT, bool INS = true>
-__device__ __forceinline__ void macro_from_moments(const Mom<R>& mo, const KP<R>& p, NodeM<R>& m)
+__device__ __forceinline__ void macro_from_moments(const Mom<R>& mo, const KP<R>& p, NodeM<R>& m,
+                                                   const R* ins = nullptr)
 {
     constexpr int D = LatDim<Q>::D;
     const R drho = mo.drho;
@@ -412,7 +414,7 @@ __device__ __forceinline__ void macro_from_moments(const Mom<R>& mo, const KP<R>
         R wv[3], Ag[3];
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            const R aeb = (INS && p.aeb_dev) ? p.aeb_dev[k] : p.AEB[k];
+            const R aeb = ins ? ins[k] : ((INS && p.aeb_dev) ? p.aeb_dev[k] : p.AEB[k]);
             Ag[k] = (k < D) ? p.AG[k] + aeb * ir : R(0);
             wv[k] = m.u[k] + R(0.5) * Ag[k];
         }
@@ -467,7 +469,7 @@ __device__ __forceinline__ void macro_from_moments(const Mom<R>& mo, const KP<R>
 
 // moments and per-node quantities of the populations d[Q]
 template <typename R, int Q, bool EXT, bool INS = true>
-__device__ __forceinline__ void node_macro(const R (&d)[Q], const KP<R>& p, NodeM<R>& m)
+__device__ __forceinline__ void node_macro(const R (&d)[Q], const KP<R>& p, NodeM<R>& m, const R* ins = nullptr)
 {
     Mom<R> mo;
     mom_zero(mo);
@@ -478,7 +480,7 @@ __device__ __forceinline__ void node_macro(const R (&d)[Q], const KP<R>& p, Node
 #pragma unroll
         for (int a = 0; a < Q; ++a) mom_add<R, Q, false>(mo, a, d[a]);
     }
-    macro_from_moments<R, Q, EXT, INS>(mo, p, m);
+    macro_from_moments<R, Q, EXT, INS>(mo, p, m, ins);
 }
 
 // The odd part's relaxation carries the momentum, and in FP32 a relative
@@ -568,6 +570,19 @@ __device__ __forceinline__ void node_relax(R (&d)[Q], const KP<R>& p, const Node
             d[b] = fma(-Wa, ej, fma(om1j, db, ps - pa));
         }
     }
+}
+
+// Unevaluated FP32 sums h + l (|l| about 2^-24 |h|, 48 bits together): exact
+// products by the fused multiply-add, exact sums by Knuth's two-sum (Dekker
+// 1971); each operation keeps 2^-46 of its operands.
+struct FF {
+    float h, l;
+};
+__device__ __forceinline__ FF ff_add(FF x, FF y)
+{
+    const float s = __fadd_rn(x.h, y.h), b = __fsub_rn(s, x.h);
+    const float e = __fadd_rn(__fsub_rn(x.h, __fsub_rn(s, b)), __fsub_rn(y.h, b));
+    return FF{s, __fadd_rn(e, __fadd_rn(x.l, y.l))};
 }
 
 // ------------------------------------------------ node pairs in FP32x2

@@ -167,7 +167,7 @@ struct Ctx {
     unsigned* errflag;
     // curved walls: the wall ids of the geometry (host), to check distances
     std::vector<uint8_t> host_wid;
-    // insulating walls: rows of the velocity sum (warps of the step grid) and fluid nodes
+    // insulating walls: rows of the step's velocity sum and fluid nodes
     bool insulating;
     long long ins_rows;
     long long n_fluid;

@@ -726,18 +726,6 @@ __device__ __forceinline__ void fields_values64(const SrcFields& s, const KP<R>&
     }
 }
 
-// Unevaluated FP32 sums h + l (|l| about 2^-24 |h|, 48 bits together): exact
-// products by the fused multiply-add, exact sums by Knuth's two-sum (Dekker
-// 1971); each operation keeps 2^-46 of its operands.
-struct FF {
-    float h, l;
-};
-__device__ __forceinline__ FF ff_add(FF x, FF y)
-{
-    const float s = __fadd_rn(x.h, y.h), b = __fsub_rn(s, x.h);
-    const float e = __fadd_rn(__fsub_rn(x.h, __fsub_rn(s, b)), __fsub_rn(y.h, b));
-    return FF{s, __fadd_rn(e, __fadd_rn(x.l, y.l))};
-}
 __device__ __forceinline__ FF ff_mul(FF x, FF y)
 {
     const float p = __fmul_rn(x.h, y.h);
@@ -1622,12 +1610,12 @@ cudaError_t launch_step_q(const Ctx& c, const void* src, void* dst, uint32_t see
 
 // the staged step (periodic boxes with the plain node code, 16-bit or FP32
 // storage; the host chose the tile rows and stage count at create)
-template <int Q, class S, bool SR, bool EXT, bool FACES, bool LP = false>
+template <int Q, class S, bool SR, bool EXT, bool FACES, bool LP = false, bool INS = false>
 cudaError_t launch_step_staged_k(const Ctx& c, const void* src, void* dst, uint32_t seed, cudaStream_t st,
                                  const StgForce& fw)
 {
     using T = typename S::T;
-    auto kern = k_step_staged<Q, S, SR, EXT, FACES, LP>;
+    auto kern = k_step_staged<Q, S, SR, EXT, FACES, LP, INS>;
     // a context always launches the same instantiation: set its shared
     // memory limit on the first launch
     if (!c.stage_ready) {
@@ -1637,7 +1625,7 @@ cudaError_t launch_step_staged_k(const Ctx& c, const void* src, void* dst, uint3
     }
     return launch_pdl(kern, staged_blocks(c), 32 * staged_warps(StgShape<EXT>::CW, c.n_special, c.geo.sq, !c.geo.periodic[0]),
                       c.stage_smem, st, (const T*)src, (T*)dst, c.cls, c.special, c.n_special, c.geo, kp_step_of<S>(c),
-                      seed, c.stage_R, (int)c.stage_tiles, c.stage_n, zero_padding(c, dst), c.errflag, fw);
+                      seed, c.stage_R, (int)c.stage_tiles, c.stage_n, zero_padding(c, dst), c.late_wait ? 1 : 0, c.errflag, fw);
 }
 
 // the staged step (the host chose the tile rows and stage count at create)
@@ -1650,6 +1638,11 @@ cudaError_t launch_step_staged(const Ctx& c, const void* src, void* dst, uint32_
         if (c.les_pair)
             return faces ? launch_step_staged_k<Q, S, SR, true, true, true>(c, src, dst, seed, st, fw)
                          : launch_step_staged_k<Q, S, SR, true, false, true>(c, src, dst, seed, st, fw);
+    }
+    if constexpr (sizeof(typename S::T) == 4 && Q == 19) {
+        if (c.insulating)
+            return faces ? launch_step_staged_k<Q, S, SR, true, true, false, true>(c, src, dst, seed, st, fw)
+                         : launch_step_staged_k<Q, S, SR, true, false, false, true>(c, src, dst, seed, st, fw);
     }
     if (c.ext)
         return faces ? launch_step_staged_k<Q, S, SR, true, true>(c, src, dst, seed, st, fw)

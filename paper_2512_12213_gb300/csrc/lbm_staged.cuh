@@ -361,18 +361,19 @@ __device__ __forceinline__ void gather_periodic(const typename S::T* __restrict_
 // code of each configuration is k_step's: the FP32x2 pair code without EXT,
 // the FP32x2 EXT pair code for FP32 storage with closed faces, else the
 // scalar EXT code node by node; LP: the FP32x2 pair code specialised for
-// LES (LES-only contexts).
-template <int Q, class S, bool SR, bool EXT = false, bool FACES = false, bool LP = false>
+// LES (LES-only contexts); INS: insulating walls (the scalar code at the
+// device's force coefficient, and the warps' sums of the flow velocity).
+template <int Q, class S, bool SR, bool EXT = false, bool FACES = false, bool LP = false, bool INS = false>
 __global__ void __launch_bounds__(32 * StgShape<EXT>::MAXW, 1)
 k_step_staged(const typename S::T* __restrict__ src, typename S::T* __restrict__ dst,
               const uint8_t* __restrict__ cls, const uint32_t* __restrict__ special, long long nspecial, const Geo g,
               const KP<float> p, uint32_t seed, int R, int ntiles, int nstages, int zero_pad,
-              unsigned* __restrict__ errflag, const StgForce fw)
+              int late, unsigned* __restrict__ errflag, const StgForce fw)
 {
     using T = typename S::T;
     using Rt = typename S::R;
     static_assert(sizeof(Rt) == 4, "the staged step computes in FP32");
-    constexpr bool PAIRX = EXT && !LP && FACES && sizeof(T) == 4;
+    constexpr bool PAIRX = EXT && !LP && !INS && FACES && sizeof(T) == 4;
     constexpr int G = StgShape<EXT>::G, W = StgShape<EXT>::W, CW = StgShape<EXT>::CW;
     pdl_trigger();
     extern __shared__ __align__(128) unsigned char smem[];
@@ -396,7 +397,33 @@ k_step_staged(const typename S::T* __restrict__ src, typename S::T* __restrict__
         mbar_fence_init();
     }
     __syncthreads();
-    pdl_wait(src);
+    // late: the kernel before is the wall force's of the same state, which
+    // this step may run beside (the producer warp waits at its end)
+    if (!late) pdl_wait(src);
+    // insulating walls: the current force coefficient, and this lane's sum of
+    // the flow velocity over its nodes (48 bits: a lane takes dozens)
+    Rt aeb[3] = {Rt(0), Rt(0), Rt(0)};
+    FF vs[3] = {{0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}};
+    auto add_v = [&](const NodeM<Rt>& m) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) vs[k] = ff_add(vs[k], FF{m.v[k], 0.0f});
+    };
+    // one row per warp of the block, by a fixed shuffle tree
+    auto put_v = [&]() {
+        const long long row = (long long)blockIdx.x * (blockDim.x >> 5) + warp;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            double t = (double)vs[k].h + (double)vs[k].l;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+            if (lane == 0) p.ins_rows[row * 3 + k] = t;
+        }
+    };
+    if constexpr (INS) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) aeb[k] = p.aeb_dev[k];
+    }
+    const Rt* const ins = INS ? aeb : nullptr;
     const int my_tiles = ((int)blockIdx.x < ntiles) ? (ntiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
 
     if (warp == CW) {
@@ -429,6 +456,9 @@ k_step_staged(const typename S::T* __restrict__ src, typename S::T* __restrict__
             for (int j = (k > nstages ? k - nstages : 0); j < k; ++j)
                 mbar_wait_bounded(&full[j % nstages], (uint32_t)(j / nstages) & 1u);
         }
+        __syncwarp();
+        if constexpr (INS) put_v();
+        if (late) pdl_wait();
         return;
     }
 
@@ -444,6 +474,7 @@ k_step_staged(const typename S::T* __restrict__ src, typename S::T* __restrict__
             __syncwarp();
             if (lane == 0) mbar_arrive(&full[s]);
         }
+        if constexpr (INS) put_v();
         return;
     }
 
@@ -479,8 +510,9 @@ k_step_staged(const typename S::T* __restrict__ src, typename S::T* __restrict__
             if constexpr (FACES) pull_walls<Q, S, true>(src, cls, g, p, Around<Q>(g, x, y, z), d);
             else gather_periodic<Q, S>(src, cls, g, p, x, y, z, node, d, fw, acc);
             NodeM<Rt> m;
-            node_macro<Rt, Q, EXT, false>(d, p, m);
+            node_macro<Rt, Q, EXT, INS>(d, p, m, ins);
             node_relax<Rt, Q, EXT>(d, p, m);
+            if constexpr (INS) add_v(m);
             if constexpr (SR) {
                 NodeRng rng((uint32_t)node, seed);
 #pragma unroll
@@ -489,6 +521,10 @@ k_step_staged(const typename S::T* __restrict__ src, typename S::T* __restrict__
 #pragma unroll
                 for (int a = 0; a < Q; ++a) dst[(long long)a * g.sq + node] = S::from_raw(d[a]);
             }
+        }
+        if constexpr (INS) {
+            __syncwarp();
+            put_v();
         }
         if (!FACES && fw.out) {
 #pragma unroll
@@ -619,13 +655,15 @@ k_step_staged(const typename S::T* __restrict__ src, typename S::T* __restrict__
                 }
                 {
                     NodeM<Rt> m;
-                    node_macro<Rt, Q, true, false>(d0, p, m);
+                    node_macro<Rt, Q, true, INS>(d0, p, m, ins);
                     node_relax<Rt, Q, true>(d0, p, m);
+                    if constexpr (INS) add_v(m);
                 }
                 {
                     NodeM<Rt> m;
-                    node_macro<Rt, Q, true, false>(d1, p, m);
+                    node_macro<Rt, Q, true, INS>(d1, p, m, ins);
                     node_relax<Rt, Q, true>(d1, p, m);
+                    if constexpr (INS) add_v(m);
                 }
 #pragma unroll
                 for (int a = 0; a < Q; ++a) dd[a].v = make_float2(d0[a], d1[a]);
@@ -662,6 +700,7 @@ k_step_staged(const typename S::T* __restrict__ src, typename S::T* __restrict__
             phase ^= 1u;
         }
     }
+    if constexpr (INS) put_v();
 }
 
 }  // namespace lbm
