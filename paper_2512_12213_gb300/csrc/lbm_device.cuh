@@ -62,7 +62,9 @@ inline cudaError_t launch_pdl(void (*kern)(P...), unsigned blocks, unsigned thre
     at.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+    if (e != cudaSuccess) cudaGetLastError();        // reported here, not to the next caller
+    return e;
 }
 
 // ---------------------------------------------------------------- lattices
@@ -646,6 +648,47 @@ __device__ __forceinline__ float rcp_approx(float x)
 __device__ __forceinline__ F2 f2sqrta(F2 a) { return F2{make_float2(sqrt_approx(a.v.x), sqrt_approx(a.v.y))}; }
 __device__ __forceinline__ F2 f2rcpa(F2 a) { return F2{make_float2(rcp_approx(a.v.x), rcp_approx(a.v.y))}; }
 
+// FP32 <-> FP64 of a positive number in 2^-111 .. 2^112 by shifting its bits
+// (narrow truncates): the FP64 pipe converts as slowly as it multiplies
+__device__ __forceinline__ float narrow(double x)
+{
+    return __uint_as_float((((unsigned)__double2hiint(x) - 0x38000000u) << 3) | ((unsigned)__double2loint(x) >> 29));
+}
+__device__ __forceinline__ double widen(float x)
+{
+    const unsigned b = __float_as_uint(x);
+    return __hiloint2double((int)((b >> 3) + 0x38000000u), (int)(b << 29));
+}
+__device__ __forceinline__ bool narrow_range(double x)
+{
+    return (unsigned)__double2hiint(x) - 0x39000000u < 0x46F00000u - 0x39000000u;
+}
+// FP64 reciprocal: y0 = 1/x in FP32 (relative error 2^-23), then
+// y = y0 (1 + e + e^2) with e = 1 - x y0 (Halley; error e^3 = 2^-69, so the
+// rounding of the three operations decides).  Outside the FP32 range, and
+// for negative or non-finite x, the plain quotient.
+__device__ __forceinline__ double rcp64(double x)
+{
+    if (!narrow_range(x)) return 1.0 / x;
+    const double y0 = widen(rcp_approx(narrow(x)));
+    const double e = fma(-x, y0, 1.0);
+    return fma(y0, fma(e, e, e), y0);
+}
+// FP64 square root by Goldschmidt's iteration from the FP32 reciprocal square
+// root: g -> sqrt(x), h -> 1/(2 sqrt(x)) (relative error 2^-22, 2^-44), then
+// the remainder x - g^2 corrects g to its rounding.  Six operations.
+__device__ __forceinline__ double sqrt64(double x)
+{
+    if (!narrow_range(x)) return sqrt(x);
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(narrow(x)));
+    double g = x * widen(y), h = widen(0.5f * y);
+    const double r = fma(-g, h, 0.5);
+    g = fma(g, r, g);
+    h = fma(h, r, h);
+    return fma(fma(-g, g, x), h, g);
+}
+
 // Eq. (2) with Eqs. (1) and (3) for two nodes: d <- (1 - om) d + om d^eq + F,
 // per opposite pair d_a' = (1 - om) d_a + w (X + Y), d_opp' = (1 - om) d_opp
 // + w (X - Y) with X = base + 9/2 om rho t^2 + 9 C rho (E_a.u^F)(E_a.A),
@@ -1201,8 +1244,7 @@ __device__ __forceinline__ void pull_walls(const typename S::T* __restrict__ P, 
 // gather_node for kernels that visit every node, given the node's class byte:
 // the class decides once how the 19 loads are formed, so that they are issued
 // together instead of each behind its own class lookup and branch (the
-// canonical export of a 256^3 FP32 box: 2,254 -> 526 us, 0.72 of the copy
-// bandwidth).  Bulk nodes add nine row offsets and three x positions; in a
+// canonical export of a 256^3 FP32 box: 2,254 -> 526 us).  Bulk nodes add nine row offsets and three x positions; in a
 // box with closed faces, bulk and face nodes alike pick the source or the
 // node's own opposite population by the node's position (no class bytes; one
 // path, so warps at the row ends do not diverge); nodes beside a solid take

@@ -895,7 +895,7 @@ __device__ R unbounced(const Src& s, const KP<R>& p, const WRho& wr, const Geo& 
 // from fields and 1.04 ms from FP32 populations; so 0.345 ms and
 // 0.225 ms (0.53 of the copy bandwidth).
 template <int Q, class S, class Src, bool CURVED>
-__global__ void __launch_bounds__(NODE_THREADS)
+__global__ void __launch_bounds__(NODE_THREADS, CURVED ? 1 : 4)
 k_inverse_stream(typename S::T* __restrict__ P, const uint8_t* __restrict__ cls, const Geo g,
                  const KP<typename S::R> p, const WRho wr, const Src s)
 {
@@ -955,9 +955,12 @@ __device__ __forceinline__ NodeXYZ node_at(const Geo& g, unsigned n)
 }
 
 // f = d + w rho0, one node per thread: bound by its loads and stores (bulk
-// nodes: 19 independent loads, no class lookups; see pull_node)
+// nodes: 19 independent loads, no class lookups; see pull_node), so as many
+// warps as registers allow: five blocks per SM (256 x 128 x 128 FP32 100 us at
+// 48 registers, 107 with four blocks, 119 with three; 0.95 of the copy
+// bandwidth; binary16 94 us, 0.76)
 template <int Q, class S, typename OutT, bool CURVED>
-__global__ void __launch_bounds__(NODE_THREADS)
+__global__ void __launch_bounds__(NODE_THREADS, 5)
 k_export(const typename S::T* __restrict__ P, const uint8_t* __restrict__ cls, const Geo g,
          const KP<typename S::R> p, const WRho wr, OutT* __restrict__ out)
 {
@@ -1221,7 +1224,9 @@ k_balance(const typename S::T* __restrict__ P, const uint8_t* __restrict__ cls, 
 // exactly from the stored values, see above), |v - v_ref| and |v| (Euclidean
 // norms), block sums in FP64 for the fixed-order pass; with `update` the
 // node's v replaces v_ref (each thread reads its own entries before it writes
-// them; solid nodes get 0).
+// them; solid nodes get 0).  The FP64 pipe bounds it (~35 operations a node):
+// 256 x 128 x 128 FP32 423 us with the quotient and the library's square
+// roots, 366 with rcp64 and sqrt64; three blocks per SM (444 with two).
 template <int Q, class S, bool EXT, bool CURVED>
 __global__ void __launch_bounds__(RED_THREADS, 3)
 k_residual(const typename S::T* __restrict__ P, const uint8_t* __restrict__ cls, const Geo g,
@@ -1270,7 +1275,7 @@ k_residual(const typename S::T* __restrict__ P, const uint8_t* __restrict__ cls,
 #pragma unroll
             for (int k = 0; k < 3; ++k) A[k] = (k < LatDim<Q>::D) ? (double)p.AG[k] : 0.0;
         }
-        const double ir = c * unit / fma(s[0], unit, (double)p.rho0);
+        const double ir = c * unit * rcp64(fma(s[0], unit, (double)p.rho0));
         double dd = 0.0, vv = 0.0;
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
@@ -1280,18 +1285,20 @@ k_residual(const typename S::T* __restrict__ P, const uint8_t* __restrict__ cls,
             vv += vk * vk;
             if (update) vref[(long long)k * N + n] = vk;
         }
-        acc[0] += sqrt(dd);
-        acc[1] += sqrt(vv);
+        acc[0] += sqrt64(dd);
+        acc[1] += sqrt64(vv);
     }
     block_sum<2>(acc, sm);
     finish_rows<2, true>(acc, partials, ro);
 }
 
 // ----------------------------------------------------------------- stress
+// Four blocks per SM in FP32 (256 x 128 x 128 S2 117 us, 136 with three, 176
+// with two; S4 201, 205, 246), two in FP64, whose pipe bounds it.
 // Variants 1, 2 at f(T) = gather(cur); 3, 4 at the half step between T-1 and
 // T: fbar = (cur + gather(cur))/2 with the node's state at T-1 = gather(prev).
 template <int Q, class S, bool EXT, bool CURVED>
-__global__ void __launch_bounds__(NODE_THREADS)
+__global__ void __launch_bounds__(NODE_THREADS, sizeof(typename S::R) == 8 ? 2 : 4)
 k_stress(const typename S::T* __restrict__ cur, const typename S::T* __restrict__ prev,
          const uint8_t* __restrict__ cls, const Geo g, const KP<typename S::R> p, int variant,
          typename S::R* __restrict__ sig, typename S::R* __restrict__ Sout, typename S::R* __restrict__ rho_out,

@@ -16,27 +16,11 @@
 //   * One node per thread, in blocks of one warp while the box has few of
 //     them: the work then spreads evenly over the SMs' FP64 pipes (64 x 32
 //     nodes in two-node threads and blocks of 128 sat on 8 of 152 SMs).
-// Step before -> now: D2Q9 64 x 32 12.4 -> 6.2 us, 256 x 128 with the Lorentz
-// force 18.5 -> 11.0 us; D3Q19 128^3 890 -> 539 us.
+// Step before -> now: D2Q9 64 x 32 12.4 -> 3.9 us, 256 x 128 with the Lorentz
+// force 18.5 -> 8.9 us; D3Q19 128^3 890 -> 537 us.
 #pragma once
 
 namespace lbm {
-
-// FP64 reciprocal: y0 = 1/x in FP32 (relative error 2^-23; converted by
-// shifting the bits, the FP64 pipe converts as slowly as it multiplies), then
-// y = y0 (1 + e + e^2) with e = 1 - x y0 (Halley; error e^3 = 2^-69, so the
-// rounding of the three operations decides).  Outside the FP32 range, and
-// for negative or non-finite x, the plain quotient.
-__device__ __forceinline__ double rcp64(double x)
-{
-    const unsigned hi = (unsigned)__double2hiint(x);
-    if (hi - 0x39000000u >= 0x46F00000u - 0x39000000u) return 1.0 / x;      // 2^-111 .. 2^112
-    const float y = rcp_approx(__uint_as_float(((hi - 0x38000000u) << 3) | ((unsigned)__double2loint(x) >> 29)));
-    const unsigned b = __float_as_uint(y);
-    const double y0 = __hiloint2double((int)((b >> 3) + 0x38000000u), (int)(b << 29));
-    const double e = fma(-x, y0, 1.0);
-    return fma(y0, fma(e, e, e), y0);
-}
 
 // Eq. (2) for the FP64 deviations d of a node; v returns the flow velocity
 // with EXT.  AEB: the Lorentz coefficient (configured, or insulating walls').
