@@ -648,7 +648,8 @@ __device__ __forceinline__ float add_split(float d, float hi, float lo)
 {
     const float s = __fadd_rn(d, hi), b = __fsub_rn(s, d);
     const float e = __fadd_rn(__fsub_rn(d, __fsub_rn(s, b)), __fsub_rn(hi, b));
-    return __fadd_rn(s, __fadd_rn(e, lo));
+    const float r = __fadd_rn(s, __fadd_rn(e, lo));
+    return fabsf(s) <= 3.402823466e38f ? r : s;      // an infinite or undefined sum has no error term
 }
 
 // ------------------------------------------ inverse propagation (import/init)
@@ -1293,12 +1294,12 @@ k_residual(const typename S::T* __restrict__ P, const uint8_t* __restrict__ cls,
 }
 
 // ----------------------------------------------------------------- stress
-// Four blocks per SM in FP32 (256 x 128 x 128 S2 117 us, 136 with three, 176
-// with two; S4 201, 205, 246), two in FP64, whose pipe bounds it.
+// Three blocks per SM in FP32 (256 x 128 x 128 S2 136 us, 176 with two; S4 205,
+// 246), two in FP64, whose pipe bounds it.
 // Variants 1, 2 at f(T) = gather(cur); 3, 4 at the half step between T-1 and
 // T: fbar = (cur + gather(cur))/2 with the node's state at T-1 = gather(prev).
 template <int Q, class S, bool EXT, bool CURVED>
-__global__ void __launch_bounds__(NODE_THREADS, sizeof(typename S::R) == 8 ? 2 : 4)
+__global__ void __launch_bounds__(NODE_THREADS, sizeof(typename S::R) == 8 ? 2 : 3)
 k_stress(const typename S::T* __restrict__ cur, const typename S::T* __restrict__ prev,
          const uint8_t* __restrict__ cls, const Geo g, const KP<typename S::R> p, int variant,
          typename S::R* __restrict__ sig, typename S::R* __restrict__ Sout, typename S::R* __restrict__ rho_out,

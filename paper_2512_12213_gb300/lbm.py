@@ -413,6 +413,7 @@ class Sim:
         fields[:self.N].fill_(self.cfg.rho0)
         fields[self.N:].zero_()
         lbm_init_equilibrium(self.ctx, fields[:self.N], fields[self.N:], None, 0, self.stream)
+        self.torch.cuda.current_stream(self.device).synchronize()    # as with host arrays
 
     def import_f(self, f):
         if isinstance(f, np.ndarray):

@@ -67,6 +67,23 @@ def test_equilibrium_from_fields(box, scale, stokes):
     sim.close()
 
 
+# infinities and NaN pass through import and export unchanged in kind
+@pytest.mark.parametrize("storage", ["f32", "bf16s", "f64"])
+def test_non_finite_populations_pass(storage):
+    nx, ny, nz = 9, 4, 3
+    sim = lbm.Sim(dict(lattice=19, nx=nx, ny=ny, nz=nz, tau=0.8, force_model="e", storage=storage),
+                  inputs.empty_mask(nx, ny, nz), stage=False)
+    f = torch.full((19, nz, ny, nx), 0.05, dtype=torch.float64, device="cuda")
+    f[3, 1, 2, 4], f[7, 0, 0, 0], f[18, 2, 3, 8] = float("inf"), float("-inf"), float("nan")
+    for dtype in (torch.float32, torch.float64):
+        sim.import_f(f.to(dtype))
+        for out in (torch.float32, torch.float64):
+            g = sim.export_f(out).double()
+            assert torch.equal(torch.isnan(g), torch.isnan(f)) and torch.equal(torch.isinf(g), torch.isinf(f))
+            assert torch.equal(g[torch.isinf(f)], f[torch.isinf(f)])
+    sim.close()
+
+
 # the FP64 step scales exactly with the density unit except for 1/rho, whose
 # iteration serves 2^-111 .. 2^112 and the plain quotient the rest: an ulp or
 # two per step
