@@ -188,9 +188,9 @@ def bytes_per_node(Q, storage, induced=False):
 EXTENSIONS = {
     "curved": ("sphere_curved", "k_step<19,S,EXT=0,FULL=1> (interpolated bounce-back in boundary chunks)",
                "true sphere r=12.4 as the wall, linear interpolated bounce-back from the signed distance"),
-    "insulating": ("sphere_insulating", "k_step<19,S,EXT=1,FULL=1> + k_ins_update",
+    "insulating": ("sphere_insulating", "k_step_staged<19,S,EXT=1,INS=1> + k_ins_update",
                    "imposed field (0, 0.02, 0), sigma_e = 1, Lorentz force, insulating walls E = -<v> x B"),
-    "brinkman": ("sphere_brinkman", "k_step<19,S,EXT=1>",
+    "brinkman": ("sphere_brinkman", "k_step_staged<19,S,EXT=1>",
                  "linear (Stokes) equilibrium, Darcy resistance 1e-4 (Brinkman)"),
     "induced": ("sphere_induced", "k_mhd_step<19,S> (fluid D3Q19 + field D3Q7, one node per thread)",
                 "external field (0, 0.02, 0), induced field on D3Q7, eta = 0.05, Maxwell equilibrium at the local field"),
@@ -328,7 +328,9 @@ def run_ours(args):
     value = whole_job_mlups(ws, N, args.steps, total_ms)
     achieved = N * bpn / (kern_ms * 1e-3) / 1e9
     kname = {"f64": "StoreF64", "f32": "StoreF32", "f16s": "StoreF16", "bf16s": "StoreBF16"}[args.storage]
-    if args.workload in EXTENSIONS:
+    if args.storage == "f64" and args.workload != "induced":
+        kernel = "k_step64<19>"
+    elif args.workload in EXTENSIONS:
         kernel = EXTENSIONS[args.workload][1].replace(",S", "," + kname)
     elif step_kernel == "staged":
         kernel = f"k_step_staged<19,{kname},SR={int(sr)}>"
@@ -399,7 +401,7 @@ def run_ours(args):
                        "l2": f"inputs larger than L2: {N * (bpn - 1) / 2 / 1e6:.0f} MB of populations read and the same "
                   "written per step",
                        "parallelism": f"{ws} independent replica(s)"},
-            "roofline": roof, "gpu_launches": (1 if step_kernel == "staged" else 3) * args.steps,
+            "roofline": roof, "gpu_launches": (1 if step_kernel == "staged" else 2) * args.steps,
             "clocks": clocks.summary(),
             "repeats": {"blocks": args.repeats, "block_ms": [round(b, 4) for b in blocks_ms],
                         "value_from": "median block (no per-step events); the roofline's kernel time is the "
