@@ -138,18 +138,18 @@ __device__ __forceinline__ void finish_rows(const double (&v)[W], double* __rest
 // bounce-back, the warp's such nodes spread over its lanes: one lane walking
 // its chunk held the warp for up to four round trips, and a box of ragged
 // rows has such a chunk in every row (sphere 250 x 121 x 99 in FP32: 141 ->
-// 92 us).  Chunks of padding alone are not touched
-// unless zero_pad asks for it (a destination that is not the context's own,
-// whose padding is zero already).  Populations are in storage units (kernel
+// 92 us).  Chunks of padding alone are not touched unless zero_pad asks for it
+// (a destination that is not the context's own, whose padding is zero
+// already).  FP32 and 16-bit storage (lbm_step64.cuh: FP64).  Populations are in storage units (kernel
 // parameters scaled to match).
-// blocks of 128 threads per SM the register allocation must allow: FP64 3
-// (168 registers), else 4 (128; for 16-bit storage measured faster than 5
-// blocks at 96 registers, which spill with the FP32x2 node pairs)
+// blocks of 128 threads per SM the register allocation must allow: 4 (128
+// registers; for 16-bit storage measured faster than 5 blocks at 96, which
+// spill with the FP32x2 node pairs)
 // (the EXT node code in FP32x2 node pairs, 32-bit storage with closed faces:
 // 3, where it needs 158 registers without spill)
 template <class S, bool EXT, bool FACES = false, bool FULL = false, bool LP = false> struct StepOcc {
     static constexpr bool PAIRX = EXT && !FULL && !LP && FACES && sizeof(typename S::T) == 4;
-    static constexpr int value = (sizeof(typename S::T) == 8 || PAIRX) ? 3 : 4;
+    static constexpr int value = PAIRX ? 3 : 4;
 };
 
 // FULL: the boundary path interpolates at walls off the half-grid and the
@@ -173,6 +173,7 @@ k_step(const typename S::T* __restrict__ src, typename S::T* __restrict__ dst,
     using R = typename S::R;
     constexpr int V = S::V;
     constexpr bool PACKED = sizeof(T) == 2;
+    static_assert(V == 4, "FP64 has its own step");
     const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const int lane = threadIdx.x & 31;
     const int ncx = g.nxp / V;
@@ -191,20 +192,12 @@ k_step(const typename S::T* __restrict__ src, typename S::T* __restrict__ dst,
     const int xl = pad ? (g.nx - 1) / V * V : x0;     // a padding chunk repeats the row's last loads
     {
         const uint8_t* cp = cls + row * g.nxp + x0;
-        unsigned long long cb;
-        if constexpr (V == 8) {
-            const uint2 cv = *reinterpret_cast<const uint2*>(cp);
-            cb = ((unsigned long long)cv.y << 32) | cv.x;
-        } else if constexpr (V == 4) {
-            cb = *reinterpret_cast<const uint32_t*>(cp);
-        } else {
-            cb = *reinterpret_cast<const uint16_t*>(cp);
-        }
+        const uint32_t cb = *reinterpret_cast<const uint32_t*>(cp);
         if (FACES) {
-            special = (cb & ~0x0202020202020202ull) != 0ull;
-            face_chunk = (cb & 0x0202020202020202ull) != 0ull;
+            special = (cb & ~0x02020202u) != 0u;
+            face_chunk = (cb & 0x02020202u) != 0u;
         } else {
-            special = cb != 0ull;
+            special = cb != 0u;
         }
     }
     FaceInfo fi;
@@ -558,19 +551,6 @@ k_step(const typename S::T* __restrict__ src, typename S::T* __restrict__ dst,
                             f[a][2 * i] = S::from_raw(dd[a].v.x);
                             f[a][2 * i + 1] = S::from_raw(dd[a].v.y);
                         }
-                    }
-                } else {
-#pragma unroll
-                    for (int k = 0; k < V; ++k) {
-                        R d[Q];
-#pragma unroll
-                        for (int a = 0; a < Q; ++a) d[a] = S::to_raw(f[a][k]);
-                        if (ladd) add_ladd(d, k);
-                        NodeM<R> m;
-                        node_macro<R, Q, EXT, FULL>(d, p, m);
-                        node_relax<R, Q, EXT>(d, p, m);
-#pragma unroll
-                        for (int a = 0; a < Q; ++a) f[a][k] = S::from_raw(d[a]);
                     }
                 }
 #pragma unroll
