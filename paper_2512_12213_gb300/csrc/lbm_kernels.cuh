@@ -737,10 +737,14 @@ __device__ __forceinline__ FF ff_split(double x, bool& ok)
 // and  w2 Z + 9/2 w2 (K_i + K_j +- 2 X) +- 3 w2 (J_i +- J_j); 9/2 w is a power
 // of two.  Rounded to FP32 at the end, as the FP64 values were: the stored values'
 // error against 64 bits is the rounding's, 2.7e-8, at deviations of 1e-2 to
-// 1e-8 alike.  256 x 128 x 128: 1,335 us in FP64 -> 145 us (0.3 of the copy
-// bandwidth).  false (d not set): an input outside the range of ff_split.
+// 1e-8 alike.  256 x 128 x 128: 1,335 us in FP64 -> 185 us.  A value that lies within the two evaluations' errors of the
+// middle of two FP32 numbers (about one of 1e5) takes the FP64 formula, so
+// that the rounding is that of the FP64 evaluation; not in a flow whose
+// deviations are below 1e-8, where the sums here are the more exact.  false (d
+// not set): an input outside the range of ff_split.
 template <int Q>
-__device__ __forceinline__ bool fields_values32(const KP<float>& p, double rho, const double (&Wd)[3], float (&d)[Q])
+__device__ __forceinline__ bool fields_values32(const KP<float>& p, const WRho& wr, double rho, const double (&Wd)[3],
+                                                float (&d)[Q])
 {
     constexpr int D = LatDim<Q>::D;
     constexpr double w1 = WD<Q>(1), w2 = WD<Q>(Q == 9 ? 5 : 7);
@@ -765,9 +769,21 @@ __device__ __forceinline__ bool fields_values32(const KP<float>& p, double rho, 
         }
         Z = ff_add(ff_add(Z, ff_neg(sum)), ff_scale(sum, -0.5f));
     }
+    // errors, over w: 2^-43 of the terms here, 2^-50 of w rho in FP64
+    float tol = fabsf(dr.h);
+#pragma unroll
+    for (int k = 0; k < D; ++k) tol = fmaf(4.0f, fabsf(W[k].h), tol);
+    tol = fmaf(1.1368684e-13f, tol, 8.8817842e-16f * p.rho0);
+    unsigned redo = 0;
     auto put = [&](int a, FF v) {
         if (p.maxwell) v = ff_add(v, FF{p.mx[a], 0.0f});
-        d[a] = __fadd_rn(v.h, v.l);
+        const float r = __fadd_rn(v.h, v.l), t = tol * (float)WD<Q>(a);
+        d[a] = r;
+        // |v - r| near half a unit in the last place of r, or a quarter (the
+        // half below a power of two)
+        const float e = fabsf(__fadd_rn(__fsub_rn(v.h, r), v.l));
+        const float half = __uint_as_float(__float_as_uint(r) & 0x7F800000u) * 5.9604645e-8f;
+        if (t <= 0.0625f * half && (fabsf(e - half) <= t || fabsf(e - 0.5f * half) <= t)) redo |= 1u << a;
     };
     put(0, ff_mul(Z, ff_const(WD<Q>(0))));
     const FF Z1 = ff_mul(Z, ff_const(w1)), Z2 = ff_scale(Z1, (float)(w2 / w1));
@@ -793,6 +809,18 @@ __device__ __forceinline__ bool fields_values32(const KP<float>& p, double rho, 
         put(a, ff_add(even, odd));
         put(b, ff_add(even, ff_neg(odd)));
     }
+    if (redo) {
+        const double ww = Wd[0] * Wd[0] + Wd[1] * Wd[1] + Wd[2] * Wd[2];
+#pragma unroll
+        for (int a = 0; a < Q; ++a) {
+            if (!(redo >> a & 1u)) continue;
+            const double eu = EX<Q>(a) * Wd[0] + EY<Q>(a) * Wd[1] + EZ<Q>(a) * Wd[2];
+            double fe = p.stokes ? rho * WD<Q>(a) * (1.0 + 3.0 * eu)
+                                 : rho * WD<Q>(a) * (1.0 + 3.0 * eu + 4.5 * eu * eu - 1.5 * ww);
+            if (p.maxwell) fe += (double)p.mx[a];
+            d[a] = (float)(fe - wr.c[SPEED2<Q>(a)]);
+        }
+    }
     return true;
 }
 
@@ -807,7 +835,7 @@ __device__ __forceinline__ void node_values(const SrcFields& s, const KP<R>& p, 
         if (s.ic != 1.0) W[k] *= s.ic;
     }
     if constexpr (sizeof(R) == 4) {
-        if (!s.xi && fields_values32<Q>(p, rho, W, d)) return;
+        if (!s.xi && fields_values32<Q>(p, wr, rho, W, d)) return;
     }
     fields_values64<Q, R>(s, p, wr, n, rho, W, d);
 }
@@ -873,8 +901,8 @@ __device__ R unbounced(const Src& s, const KP<R>& p, const WRho& wr, const Geo& 
 
 // one padded node per thread.  Before (each node pulling its 18 neighbours'
 // values, with their equilibria in FP64) a 192^3 binary16 box took 12.2 ms
-// from fields and 1.04 ms from FP32 populations; so 0.345 ms and
-// 0.225 ms (0.53 of the copy bandwidth).
+// from fields and 1.04 ms from FP32 populations; so 0.455 ms and
+// 0.22 ms (0.53 of the copy bandwidth).
 template <int Q, class S, class Src, bool CURVED>
 __global__ void __launch_bounds__(NODE_THREADS, CURVED ? 1 : 4)
 k_inverse_stream(typename S::T* __restrict__ P, const uint8_t* __restrict__ cls, const Geo g,
