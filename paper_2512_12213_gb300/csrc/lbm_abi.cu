@@ -492,7 +492,7 @@ void choose_stage(Ctx& x)
     const int R = (int)std::max<size_t>(1, std::min<size_t>((STG_COPY_BYTES + row_bytes - 1) / row_bytes,
                                                             (size_t)x.cfg.ny));
     const size_t stage = stg_stage_bytes((int)Q, R, (int)nxp, (int)x.elem);
-    const size_t budget = (size_t)x.smem_optin - 1024;
+    const size_t budget = stage_budget(x);
     int n = (int)std::min<size_t>(STG_MAX_STAGES, budget / (stage + 2 * sizeof(uint64_t)));
     n -= n % (x.ext ? StgShape<true>::G : StgShape<false>::G);      // every stage belongs to one consumer group
     if (n < 4) return;

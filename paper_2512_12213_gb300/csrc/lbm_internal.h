@@ -173,6 +173,9 @@ struct Ctx {
     long long n_fluid;
 };
 
+// shared memory that a staged step's pipeline may take
+inline size_t stage_budget(const Ctx& c) { return (size_t)c.smem_optin - 1024; }
+
 // blocks of the staged step: one per SM, at most one per tile (each boundary
 // warp writes one partial row of the fused wall force)
 inline int staged_blocks(const Ctx& c) { return (int)(c.stage_tiles < c.sm_count ? c.stage_tiles : c.sm_count); }

@@ -1633,9 +1633,10 @@ cudaError_t launch_step_staged_k(const Ctx& c, const void* src, void* dst, uint3
     using T = typename S::T;
     auto kern = k_step_staged<Q, S, SR, EXT, FACES, LP, INS>;
     // a context always launches the same instantiation: set its shared
-    // memory limit on the first launch
+    // memory limit on the first launch.  The limit is the instantiation's, for
+    // every context of the device, so it is the most that any of them asks for
     if (!c.stage_ready) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c.stage_smem);
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)stage_budget(c));
         if (e != cudaSuccess) return e;
         c.stage_ready = true;
     }

@@ -210,3 +210,31 @@ def test_staged_closed_faces_and_ext_equal_register(orc, name, storage, rounding
     tol = {"f32": 2e-6, "f16s": 1e-4, "bf16s": 1e-3}[storage]
     ref = orc.run(ocfg, mask, f0, 7)
     assert np.abs(fa - ref).max() / np.abs(ref).max() < tol
+
+
+# two contexts of one kernel instantiation with pipelines of different size,
+# both alive, stepped in turn: neither launch may depend on which came before
+@pytest.mark.parametrize("storage,rounding", [("f16s", "stochastic"), ("bf16s", "nearest"), ("f32", "nearest")])
+@pytest.mark.parametrize("name", ["les", "plain"])
+def test_contexts_of_different_pitch_step_in_turn(name, storage, rounding):
+    def states(kernel):
+        sims = []
+        for nx in (192, 256):
+            cfg = dict(lattice=19, nx=nx, ny=24, nz=7, tau=0.56, force_model="e", g=(1e-5, 0, 0), storage=storage,
+                       rounding=rounding, seed=5, step_kernel=kernel, wall_u=((0, 0, 0), (0.1, 0, 0)))
+            if name == "les":
+                cfg.update(periodic=(0, 0, 0), face_wall=(1, 1, 1, 1, 1, 2), les=1, cs=0.1)
+            sim = lbm.Sim(cfg, inputs.empty_mask(nx, 24, 7))
+            rho, u = inputs.smooth_fields(nx, 24, 7, dims=3, u_amplitude=0.03, seed=2)
+            sim.init_equilibrium(rho, u)
+            assert sim.step_kernel == kernel
+            sims.append(sim)
+        for i in (0, 1, 0, 1, 0):
+            sims[i].step(2)
+        out = [s.export_f().cpu().numpy() for s in sims]
+        assert all(s.device_status() == 0 for s in sims)
+        for s in sims:
+            s.close()
+        return out
+    for a, b in zip(states("staged"), states("register")):
+        assert np.array_equal(a, b)
