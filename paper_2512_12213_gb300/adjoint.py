@@ -56,7 +56,7 @@ class DragProblem:
                 lbm.lbm_save_state(s.ctx, self.ckpt[t // self.k], st)
             if t == 0:
                 lbm.lbm_step(s.ctx, 1, st)
-            else:                                # with the force of the step before, beside it
+            else:                                # with the force of the step before
                 lbm.lbm_step_force(s.ctx, self.wall, lbm.ACCUMULATE, 1.0 / self.T, self.Facc, lbm.OUT_DEVICE, st)
         lbm.lbm_wall_force(s.ctx, self.wall, lbm.ACCUMULATE, 1.0 / self.T, self.Facc, lbm.OUT_DEVICE, st)
         F = self.Facc.cpu().numpy()

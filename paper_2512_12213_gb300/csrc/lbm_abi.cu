@@ -756,7 +756,6 @@ lbm_status lbm_create(const lbm_config* cfg, const uint8_t* host_wall_id, void* 
     }
     choose_stage(x);
     x.adj_blocks = 0;
-    x.late_wait = false;
     cudaStream_t st = (cudaStream_t)stream;
     cudaError_t e = cudaMemcpyAsync(x.cls, cls.data(), cls.size(), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess && x.special && x.n_special)
@@ -1122,14 +1121,10 @@ lbm_status lbm_step_force(lbm_ctx* ctx, int wall, unsigned flags, double weight,
     if (x.stage_R <= 0 || !all_periodic(&x.cfg) || x.ext) {
         // the register-tiled step, or a staged step with closed faces (whose
         // face links the boundary warps do not see) or the EXT node code: the
-        // two calls in sequence; with device output nothing lies between the
-        // two kernels, and the register step runs beside the link sum
-        lbm_status s = lbm_wall_force(ctx, wall, flags, weight, out, out_on_host, stream);
+        // two calls in sequence
+        const lbm_status s = lbm_wall_force(ctx, wall, flags, weight, out, out_on_host, stream);
         if (s != LBM_OK) return s;
-        x.late_wait = out_on_host == LBM_OUT_DEVICE;
-        s = lbm_step(ctx, 1, stream);
-        x.late_wait = false;
-        return s;
+        return lbm_step(ctx, 1, stream);
     }
     StgForce fw;
     memset(&fw, 0, sizeof fw);

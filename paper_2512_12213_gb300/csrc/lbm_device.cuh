@@ -29,8 +29,11 @@ namespace lbm {
 // ready, index arithmetic and class bytes done, and pdl_wait releases them
 // when the earlier grid has completed and its stores are visible.  Every
 // thread of such a grid calls pdl_wait before it touches anything an earlier
-// kernel of the stream writes, and before it exits, so the completion of a
-// grid implies that of all before it.  pdl_trigger lets the next grid start;
+// kernel of the stream writes, whichever it is (a trigger makes nothing
+// visible to the grid that it lets start, not even what its own grid waited
+// for: a step that read the populations beside the link kernel, which had
+// waited for them, was taken back), and before it exits, so the completion of
+// a grid implies that of all before it.  pdl_trigger lets the next grid start;
 // a kernel without it holds the next one back to its end, as without all
 // this.  (Steps: 2-D
 // cylinder 512 x 256 FP32 6.2 -> 4.2 us, FP64 channel 64 x 32 6.2 -> 4.0.)

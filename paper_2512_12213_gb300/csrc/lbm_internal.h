@@ -162,7 +162,6 @@ struct Ctx {
     long long stage_tiles;   // tiles per step
     size_t stage_smem;       // dynamic shared memory per block
     mutable bool stage_ready;
-    bool late_wait;          // the step being launched follows the wall force of its own state (lbm_step_force)
     mutable int adj_blocks;  // grid of the adjoint kernel (0: not yet sized)
     unsigned* errflag;
     // curved walls: the wall ids of the geometry (host), to check distances

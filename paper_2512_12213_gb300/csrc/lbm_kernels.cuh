@@ -165,8 +165,7 @@ template <class S, bool EXT, bool FACES = false, bool FULL = false, bool LP = fa
 template <int Q, class S, bool EXT, bool FACES, bool SR, bool FULL = false, bool LP = false>
 __global__ void __launch_bounds__(STEP_THREADS, StepOcc<S, EXT, FACES, FULL, LP>::value)
 k_step(const typename S::T* __restrict__ src, typename S::T* __restrict__ dst,
-       const uint8_t* __restrict__ cls, const Geo g, const KP<typename S::R> p, uint32_t seed, int zero_pad,
-       int late)
+       const uint8_t* __restrict__ cls, const Geo g, const KP<typename S::R> p, uint32_t seed, int zero_pad)
 {
     pdl_trigger();
     using T = typename S::T;
@@ -222,9 +221,7 @@ k_step(const typename S::T* __restrict__ src, typename S::T* __restrict__ dst,
             roff[dy + 1][dz + 1] = ((long long)zs * g.ny + ys) * g.nxp;
         }
     const long long own = row * g.nxp;
-    // (late: the kernel before is the wall force's of the same state, which
-    // this step may run beside)
-    if (!late) pdl_wait(src);
+    pdl_wait(src);
 
     using RawT = typename RawVec<sizeof(T) * V>::type;
     // shifted source values: packed words for 16-bit formats, else elements
@@ -600,7 +597,6 @@ k_step(const typename S::T* __restrict__ src, typename S::T* __restrict__ dst,
             *reinterpret_cast<RawT*>(dst + (long long)a * g.sq + row * g.nxp + x0) = RawT{};
     __syncwarp();
     put_v();
-    if (late) pdl_wait();
 }
 
 // ------------------------------------------------- deviations and populations
@@ -1024,7 +1020,7 @@ k_links(const typename S::T* __restrict__ P, const uint8_t* __restrict__ cls, co
         double* __restrict__ partials, const RedOut ro)
 {
     pdl_wait(P);
-    pdl_trigger();      // after the wait: a step may run beside this kernel
+    pdl_trigger();
     using R = typename S::R;
     __shared__ double sm[3 * 32];
     double acc[3] = {0.0, 0.0, 0.0}, cor[3] = {0.0, 0.0, 0.0};
@@ -1613,7 +1609,7 @@ cudaError_t launch_step_q(const Ctx& c, const void* src, void* dst, uint32_t see
     const bool faces = !c.geo.periodic[0] || !c.geo.periodic[1] || (Q == 19 && !c.geo.periodic[2]);
     auto go = [&](auto fc, auto full, auto lp) {
         return launch_pdl(k_step<Q, S, EXT, fc.value, SR, full.value, lp.value>, blocks, STEP_THREADS, 0, st,
-                          (const T*)src, (T*)dst, c.cls, c.geo, kp_step_of<S>(c), seed, zp, c.late_wait ? 1 : 0);
+                          (const T*)src, (T*)dst, c.cls, c.geo, kp_step_of<S>(c), seed, zp);
     };
     const std::true_type yes{};
     const std::false_type no{};
@@ -1642,7 +1638,7 @@ cudaError_t launch_step_staged_k(const Ctx& c, const void* src, void* dst, uint3
     }
     return launch_pdl(kern, staged_blocks(c), 32 * staged_warps(StgShape<EXT>::CW, c.n_special, c.geo.sq, !c.geo.periodic[0]),
                       c.stage_smem, st, (const T*)src, (T*)dst, c.cls, c.special, c.n_special, c.geo, kp_step_of<S>(c),
-                      seed, c.stage_R, (int)c.stage_tiles, c.stage_n, zero_padding(c, dst), c.late_wait ? 1 : 0, c.errflag, fw);
+                      seed, c.stage_R, (int)c.stage_tiles, c.stage_n, zero_padding(c, dst), c.errflag, fw);
 }
 
 // the staged step (the host chose the tile rows and stage count at create)

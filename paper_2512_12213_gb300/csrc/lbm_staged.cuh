@@ -368,7 +368,7 @@ __global__ void __launch_bounds__(32 * StgShape<EXT>::MAXW, 1)
 k_step_staged(const typename S::T* __restrict__ src, typename S::T* __restrict__ dst,
               const uint8_t* __restrict__ cls, const uint32_t* __restrict__ special, long long nspecial, const Geo g,
               const KP<float> p, uint32_t seed, int R, int ntiles, int nstages, int zero_pad,
-              int late, unsigned* __restrict__ errflag, const StgForce fw)
+              unsigned* __restrict__ errflag, const StgForce fw)
 {
     using T = typename S::T;
     using Rt = typename S::R;
@@ -397,9 +397,7 @@ k_step_staged(const typename S::T* __restrict__ src, typename S::T* __restrict__
         mbar_fence_init();
     }
     __syncthreads();
-    // late: the kernel before is the wall force's of the same state, which
-    // this step may run beside (the producer warp waits at its end)
-    if (!late) pdl_wait(src);
+    pdl_wait(src);
     // insulating walls: the current force coefficient, and this lane's sum of
     // the flow velocity over its nodes (48 bits: a lane takes dozens)
     Rt aeb[3] = {Rt(0), Rt(0), Rt(0)};
@@ -458,7 +456,6 @@ k_step_staged(const typename S::T* __restrict__ src, typename S::T* __restrict__
         }
         __syncwarp();
         if constexpr (INS) put_v();
-        if (late) pdl_wait();
         return;
     }
 

@@ -174,7 +174,7 @@ constexpr int STEP64_THREADS = 128;
 template <int Q, bool EXT, bool FULL>
 __global__ void __launch_bounds__(STEP64_THREADS, 4)
 k_step64(const double* __restrict__ src, double* __restrict__ dst, const uint8_t* __restrict__ cls, const Geo g,
-         const KP<double> p, int zero_pad, int late)
+         const KP<double> p, int zero_pad)
 {
     const unsigned n = blockIdx.x * blockDim.x + threadIdx.x;
     const bool active = n < (unsigned)g.sq;      // the same for 64 threads: the padded node count is a multiple of 64
@@ -183,7 +183,7 @@ k_step64(const double* __restrict__ src, double* __restrict__ dst, const uint8_t
     const int z = (int)(r / (unsigned)g.ny), y = (int)(r - (unsigned)z * (unsigned)g.ny);
     const uint8_t c = active ? cls[n] : (uint8_t)NC_PAD;
     double v[3] = {0.0, 0.0, 0.0};
-    if (!late) pdl_wait(src);          // late: as in k_step
+    pdl_wait(src);
     if (c == NC_PAD || nc_solid(c)) {
         if (active && (c != NC_PAD || zero_pad))
 #pragma unroll
@@ -221,7 +221,6 @@ k_step64(const double* __restrict__ src, double* __restrict__ dst, const uint8_t
                 for (int k = 0; k < 3; ++k) p.ins_rows[(long long)(n >> 6) * 3 + k] = v[k] + half[w >> 1][k];
         }
     }
-    if (late) pdl_wait();
 }
 
 // blocks of one warp (insulating walls: two) until every SM has the 20 warps
@@ -234,7 +233,7 @@ cudaError_t launch_step64(const Ctx& c, const void* src, void* dst, int zero_pad
     const unsigned blocks = (unsigned)((c.geo.sq + threads - 1) / threads);
     auto go = [&](auto ex, auto fu) {
         return launch_pdl(k_step64<Q, ex.value, fu.value>, blocks, threads, 0, st, (const double*)src, (double*)dst,
-                          c.cls, c.geo, c.kpd, zero_pad, c.late_wait ? 1 : 0);
+                          c.cls, c.geo, c.kpd, zero_pad);
     };
     const std::true_type yes{};
     const std::false_type no{};

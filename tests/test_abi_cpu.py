@@ -234,3 +234,26 @@ def test_staged_kernel_refused_where_it_does_not_apply(lib, change):
         lbm.lbm_buffer_sizes(c, mask)
     # the same configuration with the automatic choice is accepted
     lbm.lbm_buffer_sizes(lbm.make_config(**dict(cfg, face_wall=(1, 1, 1, 1, 1, 1), **change)), mask)
+
+
+# A grid of a programmatic launch may start while the one before still runs:
+# only a wait of its own makes earlier kernels' stores visible to it.
+def test_programmatic_kernels_wait_before_they_read():
+    csrc = os.path.join(ROOT, "paper_2512_12213_gb300", "csrc")
+    text = "\n".join(open(os.path.join(csrc, f)).read() for f in sorted(os.listdir(csrc)) if f.endswith((".cu", ".cuh")))
+    kernels = set(re.findall(r"launch_pdl\(\s*(k_\w+)", text))
+    kernels |= set(re.findall(r"auto kern = (k_\w+)", text))
+    kernels |= {k for k in re.findall(r"__global__[^;{]*?\b(k_\w+)\(", text)
+                if "pdl_trigger();" in _body(text, k)}
+    assert {"k_step", "k_step64", "k_step_staged", "k_links", "k_export", "k_adjoint", "k_ins_update"} <= kernels
+    for k in sorted(kernels):
+        body = _body(text, k)
+        assert re.search(r"^    pdl_wait\(", body, re.M), f"{k} does not wait at the top level of its body"
+        assert not re.search(r"\bif \([^\n]*\) pdl_wait", body), f"{k} waits under a condition"
+
+
+def _body(text, kernel):
+    """The body of a kernel: from its opening brace at the margin to the closing one."""
+    at = re.search(r"__global__[^;{]*?\b" + kernel + r"\(", text).end()
+    begin = text.index("\n{\n", at)
+    return text[begin:text.index("\n}\n", begin)]

@@ -202,3 +202,78 @@ def test_steps_in_a_graph(storage, kernel):
     assert torch.equal(fa, fb) and torch.equal(raw(a), raw(b))
     a.close()
     b.close()
+
+
+def _force_box(name):
+    """(configuration, mask, wall distance or None, wall whose force is asked for)"""
+    if name == "cavity":           # every face closed, lid moving, Smagorinsky LES
+        n = 40
+        return dict(nx=n, ny=n, nz=n, periodic=(0, 0, 0), tau=0.55, les=1, cs=0.1, wall_u=((0, 0, 0), (0.1, 0, 0)),
+                    face_wall=(1, 1, 1, 1, 1, 2)), inputs.empty_mask(n, n, n), None, 2
+    if name == "no_links":         # a wall that no node belongs to
+        cfg, mask, _, _ = _force_box("sphere")
+        return dict(cfg, wall_u=((0.01, 0, 0), (0, 0, 0))), mask, None, 2
+    nx, ny, nz = {"insulating_large": (130, 96, 96)}.get(name, (66, 33, 20))
+    centre, r = (20.2, 14.6, 9.8), 4.4
+    mask = inputs.sphere_mask(nx, ny, nz, centre, r)
+    cfg = dict(nx=nx, ny=ny, nz=nz, tau=0.7, g=(1e-5, 0, 0), wall_u=((0.01, 0, 0),))
+    phi = None
+    if name == "closed":           # closed in x and z, body force, no EXT terms
+        cfg.update(periodic=(0, 1, 0))
+    elif name == "les":
+        cfg.update(les=1, cs=0.1, tau=0.56)
+    elif name == "brinkman":
+        cfg.update(stokes=1, darcy=1e-3)
+    elif name.startswith("insulating"):
+        cfg.update(lorentz=1, B=(0.0, 0.05, 0.02), sigma_e=1.0, insulating=1)
+    elif name == "curved":
+        z, y, x = np.mgrid[0:nz, 0:ny, 0:nx].astype(float)
+        phi = (np.sqrt((x - centre[0]) ** 2 + (y - centre[1]) ** 2 + (z - centre[2]) ** 2) - r).astype(np.float32)
+        mask = (phi < 0).astype(np.uint8)
+        cfg.update(curved=1)
+    return cfg, mask, phi, 1
+
+
+# lbm_step_force with device output is the wall force and then the step, in
+# every box whose force is not summed inside the step kernel: the values of the
+# two calls with the device idle in between, step after step
+@pytest.mark.parametrize("name,storage,kernel", [
+    ("cavity", "f16s", "staged"), ("cavity", "f32", "staged"), ("cavity", "bf16s", "register"), ("cavity", "f64", "auto"),
+    ("closed", "f16s", "staged"), ("closed", "f32", "staged"), ("closed", "f64", "auto"),
+    ("les", "f16s", "staged"), ("les", "f32", "staged"), ("les", "f16s", "register"),
+    ("brinkman", "bf16s", "staged"), ("brinkman", "f32", "staged"), ("brinkman", "f64", "auto"),
+    ("insulating", "f32", "register"), ("insulating", "f16s", "auto"), ("insulating", "f64", "auto"),
+    ("insulating_large", "f32", "auto"), ("curved", "f32", "auto"), ("curved", "f16s", "auto"), ("curved", "f64", "auto"),
+    ("sphere", "f16s", "register"), ("sphere", "bf16s", "register"), ("no_links", "f32", "register"),
+    ("no_links", "f16s", "register"), ("no_links", "f64", "auto")])
+def test_step_force_with_device_output(name, storage, kernel):
+    cfg, mask, phi, wall = _force_box(name)
+    cfg = dict(cfg, lattice=19, force_model="e", storage=storage, step_kernel=kernel, seed=3,
+               rounding="stochastic" if storage == "f16s" else "nearest")
+    a, b = lbm.Sim(cfg, mask), lbm.Sim(cfg, mask)
+    if kernel != "auto" or name == "insulating_large":
+        assert a.step_kernel == ("staged" if kernel == "auto" else kernel)
+    nz, ny, nx = mask.shape
+    rho, u = inputs.smooth_fields(nx, ny, nz, dims=3, u_amplitude=0.03, seed=3)
+    n = 60
+    ref, got = (torch.zeros((n, 3), dtype=torch.float64, device="cuda") for _ in range(2))
+    for s in (a, b):
+        if phi is not None:
+            s.set_wall_distance(phi)
+        s.init_equilibrium(rho, u)
+        s.step(1)
+    torch.cuda.synchronize()
+    for i in range(n):
+        lbm.lbm_wall_force(a.ctx, wall, 0, 1.0, ref[i], lbm.OUT_DEVICE, a.stream)
+        torch.cuda.synchronize()
+        a.step(1)
+        torch.cuda.synchronize()
+    for i in range(n):
+        lbm.lbm_step_force(b.ctx, wall, 0, 1.0, got[i], lbm.OUT_DEVICE, b.stream)
+    assert torch.equal(ref, got) and torch.equal(raw(a), raw(b))
+    assert a.device_status() == 0 and b.device_status() == 0
+    assert (name == "no_links") == (not ref.any())
+    if name.startswith("insulating"):
+        assert np.array_equal(a.electric_field(), b.electric_field())
+    a.close()
+    b.close()
