@@ -1080,19 +1080,29 @@ k_links(const typename S::T* __restrict__ P, const uint8_t* __restrict__ cls, co
 // FP64 pipe adds 1.6 lanes per cycle and SM: the plain FP64 sums (95
 // operations and conversions a node) held k_balance at 1.03 ms and k_residual
 // at 1.36 ms on the 256 x 128 x 128 box, 15 times their memory time.  FP32
-// deviations below 1/2 are therefore split without error into three 32-bit
-// integers on the grids 2^-23, 2^-43 and 2^-59 (adding 1.5 times a power of
-// two leaves the rounded multiple in the mantissa), summed in integer
-// arithmetic and joined in one 64-bit integer of units 2^-59: exact for every
-// deviation above 3e-11, and off by 2^-60 below, where an FP64 sum of values
-// near 0.01 rounds by 2^-60 at every addition.  A node with a larger or a
-// non-finite value takes FP64 sums.
+// deviations are therefore scaled by the power of two 2^s that brings the
+// node's largest into 1/4 .. 1/2, split into three 32-bit integers on the
+// grids 2^-23, 2^-43 and 2^-59 (adding 1.5 times a power of two leaves the
+// rounded multiple in the mantissa), summed in integer arithmetic and joined
+// in one 64-bit integer of units 2^-(59 + s).  That is exact for every
+// deviation above 2^-34 of the node's largest, and smaller ones are rounded by
+// 2^-58 of the largest at most, where an FP64 sum rounds by up to 2^-53 of the
+// partial sum at every addition.  A node with a deviation of 1/2 or more or a
+// non-finite one takes FP64 sums.
 constexpr double FIX_UNIT = 1.0 / 576460752303423488.0;      // 2^-59
 
-// V = sum d, sum E d in units of 2^-59; false (V not set) if some |d| >= 1/2
+// V = sum d, sum E d in units of 2^-(59 + s), 0 <= s <= 125; false (V not set)
+// if some |d| >= 1/2
 template <int Q>
-__device__ __forceinline__ bool fixed_moments(const float (&d)[Q], long long (&V)[4])
+__device__ __forceinline__ bool fixed_moments(const float (&d)[Q], long long (&V)[4], int& s)
 {
+    float top = 0.0f;
+#pragma unroll
+    for (int a = 0; a < Q; ++a) top = fmaxf(top, fabsf(d[a]));
+    const unsigned e2 = __float_as_uint(top) >> 23;            // top = 2^(e2 - 127) 1.xx
+    s = top == 0.0f ? 0 : 125 - (int)e2;
+    if (s < 0) return false;
+    const F2 scale = f2s(__uint_as_float((unsigned)(127 + s) << 23));
     constexpr int NP = LatDim<Q>::NP;
     constexpr float M1 = 1.5f, M2 = 1.5f / 1048576.0f, M3 = 1.5f / 68719476736.0f;   // 1.5, 1.5 2^-20, 1.5 2^-36
     unsigned sum[3][4] = {{0, 0, 0, 0}, {0, 0, 0, 0}, {0, 0, 0, 0}};
@@ -1113,7 +1123,7 @@ __device__ __forceinline__ bool fixed_moments(const float (&d)[Q], long long (&V
     for (int k = 0; k < NP; ++k) {
         const int a = PAIR<Q>(k), b = OPP<Q>(a);
         unsigned ua[3], ub[3];
-        split(F2{make_float2(d[a], d[b])}, ua, ub);
+        split(f2mul(F2{make_float2(d[a], d[b])}, scale), ua, ub);
         const int e[3] = {EX<Q>(a), EY<Q>(a), EZ<Q>(a)};
 #pragma unroll
         for (int l = 0; l < 3; ++l) {
@@ -1126,16 +1136,17 @@ __device__ __forceinline__ bool fixed_moments(const float (&d)[Q], long long (&V
     }
     {
         unsigned u0[3], u1[3];
-        split(F2{make_float2(d[0], 0.0f)}, u0, u1);
+        split(f2mul(F2{make_float2(d[0], 0.0f)}, scale), u0, u1);
 #pragma unroll
         for (int l = 0; l < 3; ++l) sum[l][0] += u0[l] - (unsigned)Q * K[l];
     }
-    if (range >> 23) return false;
+    if (range >> 23) return false;               // NaN
 #pragma unroll
     for (int c = 0; c < 4; ++c)
         V[c] = ((long long)(int)sum[0][c] << 36) + ((long long)(int)sum[1][c] << 16) + (long long)(int)sum[2][c];
     return true;
 }
+__device__ __forceinline__ double fixed_unit(int s) { return __hiloint2double((1023 - 59 - s) << 20, 0); }
 // the same in FP64, from the even and odd parts of the opposite pairs
 template <int Q, typename R>
 __device__ __forceinline__ void double_moments(const R (&d)[Q], double (&s)[4])
@@ -1155,8 +1166,10 @@ __device__ __forceinline__ void double_moments(const R (&d)[Q], double (&s)[4])
 }
 
 // ---------------------------------------------------------------- balance
-// A thread's nodes are summed first (FP32 compute: exactly, the 64-bit node
-// sums in two 32-bit halves), then the block in FP64; the uniform body force
+// A thread's nodes are summed first (FP32 compute: the 64-bit node sums in two
+// 32-bit halves, exactly, where they lie on the common grid 2^-59, as they do
+// unless some deviation is below 2^-36; else in FP64), then the block in FP64;
+// the uniform body force
 // multiplies the summed density, a velocity-dependent one each node's.
 template <int Q, class S, bool EXT, bool CURVED>
 __global__ void __launch_bounds__(RED_THREADS)
@@ -1181,14 +1194,23 @@ k_balance(const typename S::T* __restrict__ P, const uint8_t* __restrict__ cls, 
         bool fixed = false;
         if constexpr (sizeof(R) == 4) {
             long long V[4];
-            fixed = fixed_moments<Q>(d, V);
+            int sh;
+            fixed = fixed_moments<Q>(d, V, sh);
             if (fixed) {
+                if (EXT) s[0] = (double)V[0] * fixed_unit(sh);
+                const unsigned long long below = sh < 60 ? (1ull << sh) - 1ull : ~0ull;
+                if (((unsigned long long)(V[0] | V[1] | V[2] | V[3]) & below) == 0ull) {
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    hi[k] += V[k] >> 32;
-                    lo[k] += V[k] & 0xFFFFFFFFll;
+                    for (int k = 0; k < 4; ++k) {
+                        V[k] = sh < 60 ? V[k] >> sh : 0ll;
+                        hi[k] += V[k] >> 32;
+                        lo[k] += V[k] & 0xFFFFFFFFll;
+                    }
+                } else {
+                    const double unit = fixed_unit(sh);
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) tot[k] = fma((double)V[k], unit, tot[k]);
                 }
-                if (EXT) s[0] = (double)V[0] * FIX_UNIT;
             }
         }
         if (!fixed) {
@@ -1262,9 +1284,10 @@ k_residual(const typename S::T* __restrict__ P, const uint8_t* __restrict__ cls,
         bool fixed = false;
         if constexpr (sizeof(R) == 4) {
             long long V[4];
-            fixed = fixed_moments<Q>(d, V);
+            int sh;
+            fixed = fixed_moments<Q>(d, V, sh);
             if (fixed) {
-                unit = FIX_UNIT;
+                unit = fixed_unit(sh);
 #pragma unroll
                 for (int k = 0; k < 4; ++k) s[k] = (double)V[k];
             }

@@ -65,3 +65,53 @@ def test_balance_and_residual_sums(box, scale, storage):
     assert abs(change - math.fsum(np.sqrt(((v - 0.25) ** 2).sum(0))[fluid])) <= 1e-12 * fluid.sum()
     assert np.abs(v_ref.cpu().numpy() - np.where(fluid, v, 0.0)).max() <= 1e-13
     sim.close()
+
+
+# FP32 deviations with full mantissas, of one size and mixed over ten decades
+# in a node, down to the smallest, and beside 1/2, where FP64 sums take over.
+# A node's sums: n - 1 = 18 roundings of 2^-53 of the sum S of magnitudes at
+# most, 2^-48 S with the two roundings that follow
+@pytest.mark.parametrize("box", [(64, 5, 1), (41, 6, 5)])
+@pytest.mark.parametrize("kind", ["mixed", "low", "half", 0.1, 1e-4, 1e-8, 1e-10, 1e-12, 1e-17, 1e-30, 1e-42])
+def test_moments_of_full_mantissas(kind, box):
+    nx, ny, nz = box
+    Q = 9 if nz == 1 else 19
+    g = np.random.default_rng(12)
+    P = g.uniform(0.5, 1.0, (Q, nz, ny, nx)) * g.choice([-1.0, 1.0], (Q, nz, ny, nx))
+    if kind == "mixed":
+        P *= np.exp(g.uniform(math.log(1e-10), math.log(0.49), P.shape))
+    elif kind == "low":
+        P *= np.exp(g.uniform(math.log(1e-17), math.log(1e-7), P.shape))
+    elif kind == "half":
+        P *= 1e-3
+        P[3, 0, 1, 2], P[5, 0, 2, 4] = np.nextafter(np.float32(0.5), np.float32(0)), -np.nextafter(np.float32(0.5), np.float32(0))
+        P[4, 0, 3, 7], P[6, 0, 4, 9] = 0.5, -0.5
+        P[7, 0, 1, 11], P[8, 0, 2, 13] = np.nextafter(np.float32(0.5), np.float32(1)), -0.75
+    else:
+        P *= kind
+    P = P.astype(np.float32)
+    sim = lbm.Sim(dict(lattice=Q, nx=nx, ny=ny, nz=nz, tau=0.8, force_model="e", storage="f32"),
+                  inputs.empty_mask(nx, ny, nz), stage=False)
+    buf = torch.zeros(sim.sizes[lbm.BUF_POP_A], dtype=torch.uint8, device="cuda")
+    nxp = (nx + 63) // 64 * 64
+    buf.view(torch.float32)[:Q * nz * ny * nxp].view(Q, nz, ny, nxp)[..., :nx] = torch.from_numpy(P).cuda()
+    lbm.lbm_load_state(sim.ctx, buf, 1, sim.stream)
+    e = velocities(Q)
+    d = np.stack([np.roll(P[a].astype(np.float64), tuple(e[a][::-1]), axis=(0, 1, 2)) for a in range(Q)])
+    S = np.abs(d).sum(0)
+    node = lambda w: np.array([math.fsum(v) for v in (w[:, None] * d.reshape(Q, -1)).T]).reshape(S.shape)  # noqa: E731
+    rho, j = 1.0 + node(np.ones(Q)), np.stack([node(e[:, k].astype(float)) for k in range(3)])
+    v = j / rho
+    v_ref = torch.zeros((3, nz, ny, nx), dtype=torch.float64, device="cuda")
+    change, total, _ = sim.residual(v_ref)
+    got = v_ref.cpu().numpy()
+    bound = 2.0 ** -48 * (S + np.abs(v) * (S + 1.0)) / np.abs(rho)
+    assert np.all(np.abs(got - v) <= bound)
+    speed = np.sqrt((v * v).sum(0))
+    assert abs(total - math.fsum(speed.ravel())) <= math.fsum(np.sqrt((bound ** 2).sum(0)).ravel()) + 1e-13 * total
+    assert change == total > 0
+    mass, momentum, _ = sim.balance()
+    assert abs(mass - math.fsum(rho.ravel())) <= 1e-13 * (rho.size + S.sum())
+    for k in range(3):
+        assert abs(momentum[k] - math.fsum(j[k].ravel())) <= 1e-13 * S.sum()
+    sim.close()
