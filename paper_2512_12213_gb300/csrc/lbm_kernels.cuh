@@ -601,10 +601,10 @@ k_step(const typename S::T* __restrict__ src, typename S::T* __restrict__ dst,
 
 // ------------------------------------------------- deviations and populations
 // w rho0 of the speed classes (rest, axis, diagonal) in FP64 and as an
-// unevaluated FP32 sum hi + lo (48 bits)
+// unevaluated FP32 sum hi + lo + lo2 of the same value
 struct WRho {
     double c[3];
-    float hi[3], lo[3];
+    float hi[3], lo[3], lo2[3];
 };
 template <int Q> inline WRho wrho_of(double rho0)
 {
@@ -614,18 +614,45 @@ template <int Q> inline WRho wrho_of(double rho0)
         w.c[k] = WD<Q>(a[k]) * rho0;
         w.hi[k] = (float)w.c[k];
         w.lo[k] = (float)(w.c[k] - (double)w.hi[k]);
+        w.lo2[k] = (float)(w.c[k] - (double)w.hi[k] - (double)w.lo[k]);
     }
     return w;
 }
-// d + (hi + lo) rounded once to FP32: the error of d + hi recovered exactly
-// (Knuth's two-sum) and added with lo.  An FP64 addition holds an SM's FP64
-// pipe ~20 cycles a warp, 19 of them a node 0.17 ms of a 256 x 128 x 128 box.
-__device__ __forceinline__ float add_split(float d, float hi, float lo)
+// x + y = s + e without error (Knuth's two-sum), for two values together
+__device__ __forceinline__ F2 two_sum(F2 x, F2 y, F2& e)
 {
-    const float s = __fadd_rn(d, hi), b = __fsub_rn(s, d);
-    const float e = __fadd_rn(__fsub_rn(d, __fsub_rn(s, b)), __fsub_rn(hi, b));
-    const float r = __fadd_rn(s, __fadd_rn(e, lo));
-    return fabsf(s) <= 3.402823466e38f ? r : s;      // an infinite or undefined sum has no error term
+    const F2 s = f2add(x, y), b = f2sub(s, x);
+    e = f2add(f2sub(x, f2sub(s, b)), f2sub(y, b));
+    return s;
+}
+// the node's d_a + sign w_a rho0 rounded once to FP32, two opposite directions
+// together: s + e = d + hi and r + f = s + lo without error, and what is left,
+// e + lo2 + f, is rounded to 2^-24 of itself before it decides the rounding of
+// r.  (With lo2 left out and e + lo rounded first, 7 us less of the 108 of an
+// export of 256 x 128 x 128 FP32 nodes, a value beside rest was off by 0.66
+// units in the last place: s is then a unit of hi, and lo is as large as it.)
+// An FP64 addition holds an SM's FP64 pipe ~20 cycles a warp, 19 of them a
+// node 0.17 ms of that box.
+template <int Q>
+__device__ __forceinline__ void add_wrho(float (&d)[Q], const WRho& wr, float sign)
+{
+    auto add = [&](F2 v, int k) {
+        F2 e, f;
+        const F2 s = two_sum(v, f2s(sign * wr.hi[k]), e), r = two_sum(s, f2s(sign * wr.lo[k]), f);
+        v = f2add(r, f2add(f, f2add(e, f2s(sign * wr.lo2[k]))));
+        // an infinite or undefined sum has no error term
+        if (!(fabsf(s.v.x) <= 3.402823466e38f)) v.v.x = s.v.x;
+        if (!(fabsf(s.v.y) <= 3.402823466e38f)) v.v.y = s.v.y;
+        return v;
+    };
+    d[0] = add(F2{make_float2(d[0], 0.0f)}, 0).v.x;
+#pragma unroll
+    for (int k = 0; k < LatDim<Q>::NP; ++k) {
+        const int a = PAIR<Q>(k), b = OPP<Q>(a);
+        const F2 v = add(F2{make_float2(d[a], d[b])}, SPEED2<Q>(a));
+        d[a] = v.v.x;
+        d[b] = v.v.y;
+    }
 }
 
 // ------------------------------------------ inverse propagation (import/init)
@@ -644,11 +671,13 @@ __device__ __forceinline__ void node_values(const Src& s, const KP<R>&, const WR
     std::remove_cv_t<std::remove_pointer_t<decltype(s.f)>> f[Q];
 #pragma unroll
     for (int a = 0; a < Q; ++a) f[a] = s.f[(long long)a * s.N + n];
+    if constexpr (sizeof(R) == 4 && sizeof(f[0]) == 4) {
 #pragma unroll
-    for (int a = 0; a < Q; ++a) {
-        const int k = SPEED2<Q>(a);
-        if constexpr (sizeof(R) == 4 && sizeof(f[0]) == 4) d[a] = add_split(f[a], -wr.hi[k], -wr.lo[k]);
-        else d[a] = R((double)f[a] - wr.c[k]);
+        for (int a = 0; a < Q; ++a) d[a] = f[a];
+        add_wrho<Q>(d, wr, -1.0f);
+    } else {
+#pragma unroll
+        for (int a = 0; a < Q; ++a) d[a] = R((double)f[a] - wr.c[SPEED2<Q>(a)]);
     }
 }
 // Eq. (1) (+ Eq. 10) in FP64, times 1 + xi.  The FP64 pipe bounds it (1.7
@@ -961,9 +990,9 @@ __device__ __forceinline__ NodeXYZ node_at(const Geo& g, unsigned n)
 
 // f = d + w rho0, one node per thread: bound by its loads and stores (bulk
 // nodes: 19 independent loads, no class lookups; see pull_node), so as many
-// warps as registers allow: five blocks per SM (256 x 128 x 128 FP32 100 us at
-// 48 registers, 107 with four blocks, 119 with three; 0.95 of the copy
-// bandwidth; binary16 94 us, 0.76)
+// warps as registers allow: five blocks per SM (256 x 128 x 128 FP32 108 us at
+// 48 registers, 116 with four blocks; 0.88 of the copy bandwidth; binary16
+// 102 us, 0.70)
 template <int Q, class S, typename OutT, bool CURVED>
 __global__ void __launch_bounds__(NODE_THREADS, 5)
 k_export(const typename S::T* __restrict__ P, const uint8_t* __restrict__ cls, const Geo g,
@@ -982,13 +1011,13 @@ k_export(const typename S::T* __restrict__ P, const uint8_t* __restrict__ cls, c
         }
         R d[Q];
         pull_node<Q, S, false, CURVED>(P, cls, g, p, c, q.x, q.y, q.z, d);
+        if constexpr (sizeof(R) == 4 && sizeof(OutT) == 4) {
+            add_wrho<Q>(d, wr, 1.0f);
 #pragma unroll
-        for (int a = 0; a < Q; ++a) {
-            const int k = SPEED2<Q>(a);
-            if constexpr (sizeof(R) == 4 && sizeof(OutT) == 4)
-                out[(long long)a * N + n] = add_split(d[a], wr.hi[k], wr.lo[k]);
-            else
-                out[(long long)a * N + n] = OutT((double)d[a] + wr.c[k]);
+            for (int a = 0; a < Q; ++a) out[(long long)a * N + n] = d[a];
+        } else {
+#pragma unroll
+            for (int a = 0; a < Q; ++a) out[(long long)a * N + n] = OutT((double)d[a] + wr.c[SPEED2<Q>(a)]);
         }
     }
 }

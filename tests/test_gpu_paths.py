@@ -277,3 +277,41 @@ def test_step_force_with_device_output(name, storage, kernel):
         assert np.array_equal(a.electric_field(), b.electric_field())
     a.close()
     b.close()
+
+
+def load(sim, P, t=0):
+    """Make the FP32 array P (Q, nz, ny, nx) the stored post-collision populations."""
+    buf = torch.zeros(sim.sizes[lbm.BUF_POP_A], dtype=torch.uint8, device="cuda")
+    raw(sim, buf)[..., :sim.shape[2]] = torch.from_numpy(P).cuda()
+    lbm.lbm_load_state(sim.ctx, buf, t, sim.stream)
+    torch.cuda.synchronize()
+
+
+# import and export of FP32 populations within a few FP32 steps of the rest
+# value w rho0 (a deviation of a few units in the last place of f) and of zero:
+# one rounding of the FP64 difference or sum
+@pytest.mark.parametrize("rho0", [1.0, 0.7, 3.1, 1.0 / 3.0])
+@pytest.mark.parametrize("box", [(64, 7, 1), (64, 3, 5)])
+def test_populations_near_rest_are_rounded_once(box, rho0):
+    nx, ny, nz = box
+    Q = 9 if nz == 1 else 19
+    c = W[Q][:, None, None, None] * float(np.float32(rho0))
+    sim = lbm.Sim(dict(lattice=Q, nx=nx, ny=ny, nz=nz, tau=0.8, rho0=rho0, force_model="e", storage="f32"),
+                  inputs.empty_mask(nx, ny, nz), stage=False)
+    steps = np.arange(nx * ny * nz).reshape(nz, ny, nx) - nx * ny * nz // 2
+    f = c.astype(np.float32) + steps * np.spacing(c.astype(np.float32))
+    sim.import_f(torch.from_numpy(f.astype(np.float32)).cuda())
+    P = raw(sim)[..., :nx].cpu().numpy()
+    for a in range(Q):                                       # P_a(x) = f_a(x + E_a) - w_a rho0
+        d = np.roll(f.astype(np.float32).astype(np.float64) - c, tuple(-E[Q][a][::-1]), axis=(1, 2, 3))[a]
+        err = np.abs(P[a].astype(np.float64) - d)
+        assert np.all(err <= 0.5 * np.spacing(np.abs(d).astype(np.float32)) * (1 + 2.0 ** -16)), a
+    # export: a population near zero, f = d + w rho0 with d near -w rho0
+    P = (-c.astype(np.float32) + steps * np.spacing(c.astype(np.float32))).astype(np.float32)
+    load(sim, P)
+    got = sim.export_f(torch.float32).cpu().numpy()
+    for a in range(Q):                                       # f_a(x) = P_a(x - E_a) + w_a rho0
+        want = np.roll(P.astype(np.float64) + c, tuple(E[Q][a][::-1]), axis=(1, 2, 3))[a]
+        err = np.abs(got[a].astype(np.float64) - want)
+        assert np.all(err <= 0.5 * np.spacing(np.abs(want).astype(np.float32)) * (1 + 2.0 ** -16)), a
+    sim.close()
