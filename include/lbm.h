@@ -35,7 +35,8 @@
  *              written by a copy in stream order, valid once the stream has
  *              been synchronised (LBM_ERR_ARG for pageable memory or with
  *              LBM_ACCUMULATE).  Reductions of one context share its scratch,
- *              so they must not be in flight on two streams at once.
+ *              so they must not be in flight on two streams at once (the
+ *              values of those calls are then undefined).
  *   Units    : physical (dx, dt, c = dx/dt); forces are per unit depth in 2-D.
  *   Layout   : canonical arrays exchanged with the caller are dense C arrays,
  *              node index n = (z*ny + y)*nx + x; populations f[a][n] (a the

@@ -583,14 +583,29 @@ size_t pop_bytes(const Ctx& x) { return (size_t)x.cfg.lattice * x.geo.sq * x.ele
     DeviceGuard guard_((x).device);                                              \
     if (!guard_.ok) return cuda_fail((x), cudaErrorInvalidDevice, "set device");
 
+// The ticket of a reduction on a stream.  Each stream has its own, so that
+// reductions in flight on two streams, which share their rows and so spoil
+// their own values, leave no ticket off zero: no later reduction would then
+// find its last block, and nothing would write its output.
+unsigned* ticket_of(Ctx& x, cudaStream_t st)
+{
+    int i = 0;
+    while (i < x.n_tickets && i < N_TICKETS && x.ticket_stream[i] != st) ++i;
+    if (i == x.n_tickets || i == N_TICKETS) {      // a new stream; beyond N_TICKETS of them the oldest gives way
+        i = x.n_tickets % N_TICKETS;
+        x.ticket_stream[i] = st;
+        x.n_tickets = x.n_tickets + 1 < 2 * N_TICKETS ? x.n_tickets + 1 : N_TICKETS;
+    }
+    return reinterpret_cast<unsigned*>(x.scratch + SCRATCH_TICKET_OFF) + i;
+}
+
 // where the last block of a reduction writes: device output directly, host
 // output through the result slot (the mode was checked by out_mode_ok before
 // any launch)
-RedOut red_out(Ctx& x, double* out, int mode, double weight, bool accumulate)
+RedOut red_out(Ctx& x, double* out, int mode, double weight, bool accumulate, cudaStream_t st)
 {
     const bool dev = mode == LBM_OUT_DEVICE;
-    return RedOut{dev ? out : x.scratch + SCRATCH_OUT_OFF, weight, dev && accumulate ? 1 : 0, 0,
-                  reinterpret_cast<unsigned*>(x.scratch + SCRATCH_TICKET_OFF)};
+    return RedOut{dev ? out : x.scratch + SCRATCH_OUT_OFF, weight, dev && accumulate ? 1 : 0, 0, ticket_of(x, st)};
 }
 
 // bring the W sums in the result slot to a host output
@@ -756,6 +771,7 @@ lbm_status lbm_create(const lbm_config* cfg, const uint8_t* host_wall_id, void* 
     }
     choose_stage(x);
     x.adj_blocks = 0;
+    x.n_tickets = 0;
     cudaStream_t st = (cudaStream_t)stream;
     cudaError_t e = cudaMemcpyAsync(x.cls, cls.data(), cls.size(), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess && x.special && x.n_special)
@@ -969,7 +985,7 @@ lbm_status lbm_device_status(lbm_ctx* ctx, uint32_t* flags, int clear, void* str
     if (clear) {
         CK(cudaMemsetAsync(x.errflag, 0, sizeof(uint32_t), st), "clear flags");
         // a step that stopped on a flag may have left the fused force's ticket set
-        CK(cudaMemsetAsync(x.scratch + SCRATCH_TICKET_OFF, 0, sizeof(uint32_t), st), "clear ticket");
+        CK(cudaMemsetAsync(x.scratch + SCRATCH_TICKET_OFF, 0, N_TICKETS * sizeof(unsigned), st), "clear tickets");
     }
     return LBM_OK;
 }
@@ -1096,7 +1112,7 @@ lbm_status lbm_wall_force(lbm_ctx* ctx, int wall, unsigned flags, double weight,
     const long long e = wall < 0 ? x.n_links : x.wall_begin[wall + 1];
     double* part = x.scratch + SCRATCH_RED_OFF;
     const bool acc = (flags & LBM_ACCUMULATE) != 0;
-    const RedOut ro = red_out(x, out, out_on_host, weight, acc);
+    const RedOut ro = red_out(x, out, out_on_host, weight, acc, st);
     int nb = 0;
     if (e > b) CK(x.ops->links(x, x.pop[x.cur], b, e, flags & 3u, part, ro, &nb, st), "link kernel");
     else CK(launch_reduce_rows(part, 0, 3, ro.out, weight, ro.accumulate, st), "reduce");
@@ -1138,7 +1154,7 @@ lbm_status lbm_step_force(lbm_ctx* ctx, int wall, unsigned flags, double weight,
         for (int k = 0; k < 3; ++k) fw.lw[w][k] = x.kpf.LW[w][k];
     // the kernel's last block writes the sum: to out (device output) or to
     // the result slot, copied to the host below
-    fw.ticket = reinterpret_cast<unsigned*>(x.scratch + SCRATCH_TICKET_OFF);
+    fw.ticket = ticket_of(x, st);
     const bool dev = out_on_host == LBM_OUT_DEVICE;
     fw.result = dev ? out : x.scratch + SCRATCH_OUT_OFF;
     fw.weight = weight;
@@ -1175,7 +1191,7 @@ lbm_status lbm_balance(lbm_ctx* ctx, double* out, int out_on_host, void* stream)
     GUARD(x);
     if (!out_mode_ok(out_on_host, false, out, x.err)) return LBM_ERR_ARG;
     cudaStream_t st = (cudaStream_t)stream;
-    const RedOut ro = red_out(x, out, out_on_host, 1.0, false);
+    const RedOut ro = red_out(x, out, out_on_host, 1.0, false, st);
     CK(x.ops->balance(x, x.pop[x.cur], x.scratch + SCRATCH_RED_OFF, ro, st), "balance kernel");
     return finish_reduce(x, 7, out, out_on_host, false, st);
 }
@@ -1190,7 +1206,7 @@ lbm_status lbm_residual(lbm_ctx* ctx, double* v_ref, int update, double* out, in
     if (!out_mode_ok(out_on_host, false, out, x.err)) return LBM_ERR_ARG;
     cudaStream_t st = (cudaStream_t)stream;
     // the two sums and, for device and asynchronous outputs, their ratio
-    RedOut ro = red_out(x, out, out_on_host, 1.0, false);
+    RedOut ro = red_out(x, out, out_on_host, 1.0, false, st);
     ro.ratio = out_on_host != LBM_OUT_HOST;
     CK(x.ops->residual(x, x.pop[x.cur], v_ref, update ? 1 : 0, x.scratch + SCRATCH_RED_OFF, ro, st), "residual kernel");
     if (out_on_host != LBM_OUT_HOST) return finish_reduce(x, 3, out, out_on_host, false, st);
@@ -1279,9 +1295,10 @@ lbm_status lbm_adjoint_gradient(lbm_ctx* ctx, double* out, int out_on_host, void
     if (!out) return arg_fail(x, "out is NULL");
     GUARD(x);
     if (!out_mode_ok(out_on_host, false, out, x.err)) return LBM_ERR_ARG;
-    const RedOut ro = red_out(x, out, out_on_host, 1.0, false);
-    CK(launch_reduce_rows(x.scratch + SCRATCH_ADJ_OFF, ADJ_BLOCKS, 6, ro.out, 1.0, 0, (cudaStream_t)stream), "reduce");
-    return finish_reduce(x, 6, out, out_on_host, false, (cudaStream_t)stream);
+    cudaStream_t st = (cudaStream_t)stream;
+    const RedOut ro = red_out(x, out, out_on_host, 1.0, false, st);
+    CK(launch_reduce_rows(x.scratch + SCRATCH_ADJ_OFF, ADJ_BLOCKS, 6, ro.out, 1.0, 0, st), "reduce");
+    return finish_reduce(x, 6, out, out_on_host, false, st);
 }
 
 }  // extern "C"

@@ -56,7 +56,8 @@ constexpr size_t SCRATCH_RED_OFF = 0;
 constexpr size_t SCRATCH_ADJ_OFF = (size_t)MAX_PARTIAL_ROWS * PARTIAL_WIDTH;
 constexpr size_t SCRATCH_OUT_OFF = SCRATCH_ADJ_OFF + (size_t)ADJ_BLOCKS * 6;
 constexpr size_t SCRATCH_FLAG_OFF = SCRATCH_OUT_OFF + 8;   // device error flags (unsigned)
-constexpr size_t SCRATCH_TICKET_OFF = SCRATCH_FLAG_OFF + 1; // last-block ticket of the reductions (unsigned)
+constexpr size_t SCRATCH_TICKET_OFF = SCRATCH_FLAG_OFF + 1; // last-block tickets of the reductions (unsigned)
+constexpr int N_TICKETS = 14;                               // ... up to the end of the 8 doubles
 constexpr size_t SCRATCH_DOUBLES = SCRATCH_FLAG_OFF + 8;
 // insulating walls only, after the above: the field block (E, the sum of v,
 // the force coefficient in FP64, FP32 and FP32 storage units, the ticket of
@@ -164,6 +165,9 @@ struct Ctx {
     mutable bool stage_ready;
     mutable int adj_blocks;  // grid of the adjoint kernel (0: not yet sized)
     unsigned* errflag;
+    // the streams that reductions have run on, each with a ticket of its own
+    cudaStream_t ticket_stream[N_TICKETS];
+    int n_tickets;
     // curved walls: the wall ids of the geometry (host), to check distances
     std::vector<uint8_t> host_wid;
     // insulating walls: rows of the step's velocity sum and fluid nodes

@@ -315,3 +315,37 @@ def test_populations_near_rest_are_rounded_once(box, rho0):
         err = np.abs(got[a].astype(np.float64) - want)
         assert np.all(err <= 0.5 * np.spacing(np.abs(want).astype(np.float32)) * (1 + 2.0 ** -16)), a
     sim.close()
+
+
+# reductions in flight on several streams, which the header forbids, spoil the
+# values of those calls alone: the ones after them are right, on every stream,
+# also where more streams have been used than have a counter of their own
+def test_reductions_after_overlapping_ones():
+    nx, ny, nz = 64, 24, 20
+    mask = inputs.sphere_mask(nx, ny, nz, (20.2, 11.6, 9.8), 4.4)
+    sim = lbm.Sim(dict(lattice=19, nx=nx, ny=ny, nz=nz, tau=0.7, force_model="e", g=(1e-5, 0, 0), storage="f16s",
+                       wall_u=((0, 0, 0),), step_kernel="staged"), mask)
+    sim.rest()
+    sim.step(20)
+    v_ref = sim.velocity_buffer()
+    scrap = torch.zeros((3, 8), dtype=torch.float64, device="cuda")
+    streams = [torch.cuda.Stream() for _ in range(40)]
+
+    def results(stream):
+        with torch.cuda.stream(stream):
+            force, balance = sim.wall_force(1), sim.balance()
+            return np.hstack([force, *balance, sim.residual(v_ref, update=False)])
+    torch.cuda.synchronize()
+    want = results(streams[0])
+    for k in range(0, 36, 3):
+        for _ in range(20):
+            lbm.lbm_wall_force(sim.ctx, 1, 0, 1.0, scrap[0], lbm.OUT_DEVICE, streams[k].cuda_stream)
+            lbm.lbm_balance(sim.ctx, scrap[1], lbm.OUT_DEVICE, streams[k + 1].cuda_stream)
+            lbm.lbm_residual(sim.ctx, v_ref, False, scrap[2], lbm.OUT_DEVICE, streams[k + 2].cuda_stream)
+        torch.cuda.synchronize()
+        for stream in (streams[k], streams[k + 1], streams[k + 2], streams[39]):
+            assert np.array_equal(results(stream), want)
+    got = np.zeros(3)
+    lbm.lbm_step_force(sim.ctx, 1, 0, 1.0, got, lbm.OUT_HOST, sim.stream)
+    assert np.abs(got - want[:3]).max() <= 1e-12 * np.abs(want[:3]).max()
+    sim.close()
