@@ -88,7 +88,7 @@ k_adjoint(const typename S::T* __restrict__ Pprev, const typename S::R* __restri
                 const int a = OPP<Q>(b);
                 if (!nc_solid(cs[b])) continue;
                 const int wall = nc_wall(cs[b]);
-                d[b] += ladd_of<Q, R>(p, b, wall);
+                d[b] = ladd_on<Q, R>(d[b], p, b, wall);
                 if (wall == target) {
                     // u_w enters f(t+1) and F_t through the Ladd term
                     const R gl = ac.gl[a] * (psi[a] + R(0.5) * ac.seed[a]);

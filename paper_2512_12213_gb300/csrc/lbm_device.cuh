@@ -1023,14 +1023,9 @@ __device__ __forceinline__ void pair_collide_ext(F2 (&d)[Q], const KP<float>& p)
 }
 
 // ---------------------------------------------------- closed box faces
-// Ladd term w_a E_a . LW[wall] of an incoming population
-template <int Q, typename R>
-__device__ __forceinline__ R ladd_of(const KP<R>& p, int a, int wall)
-{
-    return R(WD<Q>(a)) * (R(EX<Q>(a)) * p.LW[wall][0] + R(EY<Q>(a)) * p.LW[wall][1] + R(EZ<Q>(a)) * p.LW[wall][2]);
-}
-// v plus (ladd_on) or minus (ladd_off) that term, rounded once: every kernel
-// forms a bounced population this way, so they agree bit for bit
+// v plus (ladd_on) or minus (ladd_off) the Ladd term w_a E_a . LW[wall] of an
+// incoming population, rounded once: every kernel forms a bounced population
+// this way, so they agree bit for bit
 template <int Q, typename R>
 __device__ __forceinline__ R ladd_on(R v, const KP<R>& p, int a, int wall)
 {

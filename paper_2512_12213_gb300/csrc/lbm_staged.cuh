@@ -340,8 +340,10 @@ __device__ __forceinline__ void gather_periodic(const typename S::T* __restrict_
                 // e_a' (fbar_a' + fbar_b) in lattice units, scaled by the caller
                 const float* lw = fw.lw[wall];
                 const double w = WD<Q>(b);
-                const float Lp = (float)w * ((float)EX<Q>(b) * lw[0] + (float)EY<Q>(b) * lw[1] + (float)EZ<Q>(b) * lw[2]);
-                const double vo = (double)S::to_r(bv[b]), vi = (double)(S::to_r(bv[b]) + Lp);
+                const float Pa = S::to_r(bv[b]);
+                const double vo = (double)Pa;           // rounded as ladd_on, in physical units
+                const double vi = (double)fmaf((float)w, (float)EX<Q>(b) * lw[0] + (float)EY<Q>(b) * lw[1] +
+                                                             (float)EZ<Q>(b) * lw[2], Pa);
                 const double s = vo + vi + 2.0 * w * fw.rho0;
                 const int e[3] = {-EX<Q>(b), -EY<Q>(b), -EZ<Q>(b)};     // e_a', a' = opp(b)
 #pragma unroll

@@ -238,3 +238,26 @@ def test_contexts_of_different_pitch_step_in_turn(name, storage, rounding):
         return out
     for a, b in zip(states("staged"), states("register")):
         assert np.array_equal(a, b)
+
+
+# the force summed in the step takes a moving wall's population as the link
+# kernel does: FP32 values rounded alike, so the two differ by FP64 roundings
+# of 18 additions (4e-15 of the largest term, w rho0) and not by one of FP32
+@pytest.mark.parametrize("storage", ["f32", "f16s", "bf16s"])
+def test_step_force_of_a_moving_wall(storage):
+    nx, ny, nz = 64, 9, 7
+    mask = inputs.empty_mask(nx, ny, nz)
+    mask[3, 4, 20] = 1                                       # one solid node: 18 links
+    cfg = dict(lattice=19, nx=nx, ny=ny, nz=nz, periodic=(1, 1, 1), tau=0.7, force_model="e", g=(2e-5, 0, 0),
+               storage=storage, wall_u=((0.0123, -0.0217, 0.0171),), step_kernel="staged")
+    sim = lbm.Sim(cfg, mask)
+    rho, u = inputs.smooth_fields(nx, ny, nz, dims=3, u_amplitude=0.03, seed=3)
+    sim.init_equilibrium(rho, u)
+    sim.step(1)
+    for flags in (0, lbm.MOVING_CORR):
+        for _ in range(8):
+            ref = sim.wall_force(1, flags)
+            got = np.zeros(3)
+            lbm.lbm_step_force(sim.ctx, 1, flags, 1.0, got, lbm.OUT_HOST, sim.stream)
+            assert np.abs(got - ref).max() <= 1e-14, (flags, got, ref)
+    sim.close()
