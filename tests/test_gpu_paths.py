@@ -349,3 +349,10 @@ def test_reductions_after_overlapping_ones():
     lbm.lbm_step_force(sim.ctx, 1, 0, 1.0, got, lbm.OUT_HOST, sim.stream)
     assert np.abs(got - want[:3]).max() <= 1e-12 * np.abs(want[:3]).max()
     sim.close()
+
+
+# ... with rows that end one node into a pitch, in its last chunk, and of one node
+@pytest.mark.parametrize("storage", ["f32", "f16s"])
+@pytest.mark.parametrize("nx", [1, 61, 63, 65, 124])
+def test_step_from_leaves_no_padding_at_row_ends(nx, storage):
+    test_step_from_leaves_no_padding(nx, storage, "staged")
