@@ -881,17 +881,16 @@ __device__ __forceinline__ long long canon_of(const Geo& g, long long padded)
     return (padded / g.nxp) * g.nx + xs;
 }
 
-// The stored value P_a(x) of a link a that leaves fluid node x (padded own,
-// canonical nd) into a wall, such that the bounced population of opp(a) at x
-// (see bounced) is the given f_opp(a)(x): the inverse of the halfway or
+// The stored value P_a(x) of a link a that leaves fluid node x (padded own)
+// into a wall, such that the bounced population of b = opp(a) at x (see
+// bounced) is the given fb = f_b(x), fa = f_a(x): the inverse of the halfway or
 // interpolated rule.  Every case is explicit except both opposite links of
 // x hitting solids with q >= 1/2, a 2 x 2 solve.
 template <int Q, typename R, class Src>
 __device__ R unbounced(const Src& s, const KP<R>& p, const WRho& wr, const Geo& g, const uint8_t* __restrict__ cls, int x, int y, int z,
-                       long long own, long long nd, int a, int wall)
+                       long long own, R fa, R fb, int a, int wall)
 {
     const int b = OPP<Q>(a);
-    const R fb = src_value<Q, R>(s, p, wr, b, nd);
     const R half = ladd_off<Q, R>(fb, p, b, wall);
     if (!g.phi) return half;
     const long long sa = link_target(g, x, y, z, EX<Q>(a), EY<Q>(a), EZ<Q>(a));
@@ -902,8 +901,7 @@ __device__ R unbounced(const Src& s, const KP<R>& p, const WRho& wr, const Geo& 
     const bool b_fluid = pull_source(g, cls, x, y, z, EX<Q>(a), EY<Q>(a), EZ<Q>(a), nb, wb);   // x + E_b = x - E_a
     if (qa < R(0.5)) {
         if (!b_fluid) return half;
-        const R fa = src_value<Q, R>(s, p, wr, a, nd);                // = P_a(x - E_a)
-        return (half - (R(1) - R(2) * qa) * fa) / (R(2) * qa);
+        return (half - (R(1) - R(2) * qa) * fa) / (R(2) * qa);       // fa = P_a(x - E_a)
     }
     R Pb;
     if (b_fluid) {
@@ -911,7 +909,6 @@ __device__ R unbounced(const Src& s, const KP<R>& p, const WRho& wr, const Geo& 
         return ladd_off<Q, R>(R(2) * qa * fb - (R(2) * qa - R(1)) * Pb, p, b, wall);
     }
     // the link b of x hits a wall too (wall id wb)
-    const R fa = src_value<Q, R>(s, p, wr, a, nd);
     const long long sb = link_target(g, x, y, z, EX<Q>(b), EY<Q>(b), EZ<Q>(b));
     const R qb = (sb >= 0 && nc_solid(cls[sb])) ? R(g.phi[own]) / (R(g.phi[own]) - R(g.phi[sb])) : R(0.5);
     if (qb < R(0.5) || !(sb >= 0 && nc_solid(cls[sb]))) {
@@ -963,7 +960,7 @@ k_inverse_stream(typename S::T* __restrict__ P, const uint8_t* __restrict__ cls,
                     P[(long long)a * g.sq + srcp] = S::from_r(d[a]);
                 else
                     P[(long long)OPP<Q>(a) * g.sq + n] =
-                        S::from_r(unbounced<Q, R>(s, p, wr, g, cls, x, y, z, n, nd, OPP<Q>(a), wall));
+                        S::from_r(unbounced<Q, R>(s, p, wr, g, cls, x, y, z, n, d[OPP<Q>(a)], d[a], OPP<Q>(a), wall));
             }
             return;
         }
