@@ -168,9 +168,9 @@ typedef struct lbm_config {
 /* Kernel of the fused step.  Both compute the same arithmetic and store the
  * same bits; they differ in how the pull sources reach the registers.
  * LBM_STEP_AUTO (0) picks the staged kernel, where it applies and its
- * pipeline fits in shared memory, for 16-bit storage and for FP32 with any of
- * the Lorentz force, Maxwell term, LES, linear equilibrium or Darcy
- * resistance on D3Q19 (large boxes with insulating walls included), unless
+ * pipeline fits in shared memory, for 16-bit storage and for FP32 on D3Q19 with
+ * a closed face or any of the Lorentz force, Maxwell term, LES, linear
+ * equilibrium or Darcy resistance (large boxes with insulating walls included), unless
  * more than 4% (8% with one of those) of the 4-node chunks touch a solid or a
  * ragged row end or the box is one of the few kinds that measured slower; else
  * the register-tiled one.  LBM_STEP_REGISTER

@@ -483,10 +483,15 @@ void choose_stage(Ctx& x)
     // FP32 without the EXT terms: the register-tiled kernel keeps enough bytes
     // in flight (sphere 256 x 128 x 128 97.8 / 111) unless the rows are ragged
     // and short (more than 2%: 130 x 96 x 96 53.5 / 44.7, 67 x 60 x 61 13.5 /
-    // 11.8; below, 250 x 121 x 99 88.7 / 94.5).  With them it holds too few
-    // warps (cavity 256^3 502 / 427, 64^3 12.3 / 10.7, 32^3 7.9 / 5.3; Brinkman
-    // box 256 x 128 x 128 123 / 100).  D2Q9 stays.
-    if (automatic && x.elem != 2 && !(d3 && (x.ext || x.n_special * 50 > x.geo.sq / 4))) return;
+    // 11.8; below, 250 x 121 x 99 88.7 / 94.5).  With closed faces it does not
+    // (box closed in x, y and z 256 x 128 x 128 153 / 103, 256^3 593 / 417,
+    // 96 x 64 x 64 17.2 / 13.8, 64 x 4 x 4 7.0 / 5.1; channel closed in y 134 /
+    // 111, 522 / 423, 13.7 / 12.8, 6.6 / 4.7; with scattered solids in 3.7% of
+    // the chunks 197 / 146), and with the EXT terms it holds too few warps
+    // (cavity 256^3 502 / 427, 64^3 12.3 / 10.7, 32^3 7.9 / 5.3; Brinkman box
+    // 256 x 128 x 128 123 / 100).  D2Q9 stays.
+    const bool closed = !all_periodic(&x.cfg);
+    if (automatic && x.elem != 2 && !(d3 && (x.ext || closed || x.n_special * 50 > x.geo.sq / 4))) return;
     const size_t Q = x.cfg.lattice, nxp = x.geo.nxp;
     const size_t row_bytes = nxp * x.elem;
     const int R = (int)std::max<size_t>(1, std::min<size_t>((STG_COPY_BYTES + row_bytes - 1) / row_bytes,
@@ -503,7 +508,7 @@ void choose_stage(Ctx& x)
     // per block; LES and plain node codes do not (cavity binary16 128^3 80.5 /
     // 49.5, 64^3 10.8 / 10.6, 32^3 10.2 / 7.5)
     const bool scalar = x.ext && !x.les_pair && x.n_special * 200 <= x.geo.sq / 4;
-    const bool long_tiles = d3 ? scalar : (!all_periodic(&x.cfg) || x.ext);
+    const bool long_tiles = d3 ? scalar : (closed || x.ext);
     if (automatic && x.elem == 2 && long_tiles && tiles < 16ll * x.sm_count) return;
     if (x.insulating) {
         // from 16 tiles per block (256 x 128 x 128 139 / 121, 130 x 96 x 96 86 / 77,

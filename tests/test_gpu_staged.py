@@ -261,3 +261,23 @@ def test_step_force_of_a_moving_wall(storage):
             lbm.lbm_step_force(sim.ctx, 1, flags, 1.0, got, lbm.OUT_HOST, sim.stream)
             assert np.abs(got - ref).max() <= 1e-14, (flags, got, ref)
     sim.close()
+
+
+# FP32 boxes with a closed face run the staged kernel unless asked otherwise
+# (periodic ones the register kernel): same bits
+@pytest.mark.parametrize("periodic", [(0, 0, 0), (0, 1, 1), (1, 0, 1), (1, 1, 0), (1, 1, 1)])
+@pytest.mark.parametrize("box", [(64, 5, 3), (72, 33, 10)])
+def test_automatic_kernel_of_closed_fp32_boxes(box, periodic):
+    nx, ny, nz = box
+    out = []
+    for kernel in ("auto", "register"):
+        sim = lbm.Sim(dict(lattice=19, nx=nx, ny=ny, nz=nz, periodic=periodic, tau=0.6, force_model="d", g=(1e-4, 0, 0),
+                           storage="f32", wall_u=((0, 0, 0), (0.03, 0.01, 0)), face_wall=(1, 2, 1, 2, 1, 2),
+                           step_kernel=kernel), inputs.empty_mask(nx, ny, nz))
+        assert sim.step_kernel == ("register" if kernel == "register" or all(periodic) else "staged")
+        sim.init_equilibrium(*inputs.smooth_fields(nx, ny, nz, dims=3, u_amplitude=0.04, seed=4))
+        sim.step(9)
+        assert sim.device_status() == 0
+        out.append(sim.export_f())
+        sim.close()
+    assert torch.equal(out[0], out[1])
