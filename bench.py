@@ -10,7 +10,9 @@ with their drag error against FP64; the FP32 D3Q19 lid-driven LES cavity;
 adjoint throughput on the 2-D cylinder; an end-to-end run through host
 buffers; the roofline of the fused step kernel; the CPU oracle.
 
-    python bench.py [--steps K] [--warmup W] [--gpus N] [--impl ours|reference]
+    python bench.py [--steps K] [--warmup W] [--gpus N] [--impl ours|reference] [--details FILE]
+
+prints one short JSON line on stdout and every measurement in full on stderr.
 
 N > 1 runs N independent replicas (one per rank, launched by torchrun) and
 reports their summed throughput.
@@ -51,6 +53,7 @@ def parse():
     p.add_argument("--impl", default="ours", choices=["ours", "reference"])
     p.add_argument("--drag-steps", type=int, default=2000)
     p.add_argument("--no-extras", action="store_true", help="headline only")
+    p.add_argument("--details", default=None, help="also write every measurement in full to this file (JSON)")
     p.add_argument("--storage", default="f16s", choices=["f64", "f32", "f16s", "bf16s"],
                    help="storage of the headline run (profiling)")
     p.add_argument("--rounding", default="stochastic", choices=["nearest", "stochastic"],
@@ -87,6 +90,38 @@ def whole_job_mlups(ws, nodes, steps, total_ms):
     """Node updates of all replicas per second (weak scaling: every rank
     advances its own box of `nodes` nodes `steps` times), in millions."""
     return ws * nodes * steps / (total_ms * 1e-3) / 1e6
+
+
+def emit(line, details, path=None):
+    """Print the result line, alone on stdout and short enough to be kept
+    whole by whoever records the output's end (it was 15 kB with everything in
+    it): the headline, its end-to-end and baseline rates, roofline and clocks,
+    and the main figure of each further measurement.  Those in full, and the
+    line's own notes, go to stderr as one line of JSON and to `path`."""
+    short = {k: v for k, v in line.items() if k not in ("e2e", "cpu_baseline", "repeats")}
+    for key, keep in (("e2e", ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step")),
+                      ("cpu_baseline", ("value", "unit", "cores", "kind", "sample", "cpu_model")),
+                      ("repeats", ("blocks", "block_ms"))):
+        if key in line:
+            short[key] = {k: line[key][k] for k in keep if k in line[key]}
+    figure = {"storage_variants": ("mlups",), "drag_error_vs_f64": ("rel_err_mean",), "cavity_les_f32": ("mlups", "frac"),
+              "extensions_f32": ("mlups",), "adjoint": ("adjoint_kernel_mlups", "adjoint_kernel_frac")}
+    for key, keep in figure.items():
+        if key not in details:
+            continue
+        v = details[key]
+        if any(k in v for k in keep):
+            short[key] = {k: v[k] for k in keep if k in v}
+        else:
+            short[key] = {name: {k: d[k] for k in keep if k in d} for name, d in v.items()
+                          if isinstance(d, dict) and any(k in d for k in keep)}
+    full = json.dumps(dict(line, **details))
+    if details:
+        print("details: " + full, file=sys.stderr, flush=True)
+    if path:
+        with open(path, "w") as fh:
+            fh.write(full + "\n")
+    print(json.dumps(short), flush=True)
 
 
 def peaks():
@@ -209,6 +244,16 @@ def make_workload(workloads, name, storage, size=256):
     return out if len(out) == 3 else (out[0], out[1], None)
 
 
+def force_in_step(sim):
+    """Whether lbm_step_force sums the drag inside the step kernel: the staged
+    step of boxes periodic on every axis with the plain node code; elsewhere
+    it is two calls."""
+    c = sim.cfg
+    ext = c.lorentz or c.maxwell or c.les or c.stokes or c.darcy > 0
+    periodic = c.periodic[0] and c.periodic[1] and (c.lattice == 9 or c.periodic[2])
+    return sim.step_kernel == "staged" and periodic and not ext
+
+
 def timed_run(torch, lbm, sim, steps, warmup, wall=1, events=True, repeats=1):
     """Warm up, then time `repeats` blocks of exactly `steps` steps with CUDA
     events on the launching stream.  A step is the fused collide-stream
@@ -224,12 +269,7 @@ def timed_run(torch, lbm, sim, steps, warmup, wall=1, events=True, repeats=1):
     cs = torch.cuda.current_stream()
     side = torch.cuda.Stream(device=cs.device)
     hist = torch.zeros((max(steps, warmup, 1), 3), dtype=torch.float64, device=sim.device)
-    # lbm_step_force sums the drag inside the staged step in boxes periodic
-    # on every axis with the plain node code; elsewhere it is two calls
-    c = sim.cfg
-    ext = c.lorentz or c.maxwell or c.les or c.stokes or c.darcy > 0
-    periodic = c.periodic[0] and c.periodic[1] and (c.lattice == 9 or c.periodic[2])
-    fused = sim.step_kernel == "staged" and periodic and not ext
+    fused = force_in_step(sim)
 
     def one(i, a=None, b=None):
         if fused:
@@ -312,7 +352,7 @@ def run_ours(args):
     if phi is not None:
         sim.set_wall_distance(phi)
     sim.rest()
-    step_kernel = sim.step_kernel
+    step_kernel, fused = sim.step_kernel, force_in_step(sim)
     N = cfg["nx"] * cfg["ny"] * cfg["nz"]
     fluid = int((mask == 0).sum())
     bpn = bytes_per_node(19, args.storage, induced=bool(cfg.get("induced")))
@@ -333,7 +373,7 @@ def run_ours(args):
     elif args.workload in EXTENSIONS:
         kernel = EXTENSIONS[args.workload][1].replace(",S", "," + kname)
     elif step_kernel == "staged":
-        kernel = f"k_step_staged<19,{kname},SR={int(sr)}>"
+        kernel = f"k_step_staged<19,{kname},EXT={int(bool(cfg.get('les')))},SR={int(sr)}>"
     else:
         kernel = f"k_step<19,{kname},EXT={int(bool(cfg.get('les')))},SR={int(sr)}>"
     roof = {"kernel": kernel, "bound": "hbm", "achieved": round(achieved, 1),
@@ -396,12 +436,12 @@ def run_ours(args):
                                                   else (" (stochastic rounding)" if sr else "")),
                        "compute": "f32",
                        "step": ("collide-stream with the FP64 drag summed in the step kernel + its fixed-order "
-                                "reduction" if step_kernel == "staged" else
+                                "reduction" if fused else
                                 "fused collide-stream + FP64 drag reduction (on a second stream beside the step)"),
                        "l2": f"inputs larger than L2: {N * (bpn - 1) / 2 / 1e6:.0f} MB of populations read and the same "
                   "written per step",
                        "parallelism": f"{ws} independent replica(s)"},
-            "roofline": roof, "gpu_launches": (1 if step_kernel == "staged" else 2) * args.steps,
+            "roofline": roof, "gpu_launches": (1 if fused else 2) * args.steps,
             "clocks": clocks.summary(),
             "repeats": {"blocks": args.repeats, "block_ms": [round(b, 4) for b in blocks_ms],
                         "value_from": "median block (no per-step events); the roofline's kernel time is the "
@@ -414,8 +454,7 @@ def run_ours(args):
             line["e2e"] = e2e
         if cpu:
             line["cpu_baseline"] = cpu
-        line.update(out)
-        print(json.dumps(line), flush=True)
+        emit(line, out, args.details)
     if ws > 1:
         dist.barrier()
         dist.destroy_process_group()

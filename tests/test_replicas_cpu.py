@@ -63,3 +63,31 @@ def test_reference_arm_prints_on_rank_zero_only():
     lines = [json.loads(x) for x in r.stdout.splitlines() if x.startswith("{")]
     assert len(lines) == 1
     assert lines[0]["impl"] == "reference" and lines[0]["n_gpus"] == 2 and lines[0]["value"] > 0
+
+
+def test_result_line_is_short_and_complete(capsys, tmp_path):
+    """The line that a recorder keeps the end of: the agreed keys, the main
+    figures, under 4,000 characters however much was measured; all of it in
+    the details."""
+    sys.path.insert(0, ROOT)
+    import bench
+    keys = {"metric": bench.METRIC, "value": 72000.5, "unit": "MLUPS", "n_gpus": 1, "steps": 20, "warmup": 5,
+            "ms_per_step": 0.0545, "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f32",
+            "data": "synthetic", "config": {"workload": bench.WORKLOAD, "l2": "x" * 100}, "gpu_launches": 20,
+            "clocks": {"sm_mhz": 2070.0, "sm_max_mhz": 2070.0, "reasons": []}, "roofline": {"frac": 0.85}}
+    e2e = {"value": 58000.0, "unit": "MLUPS", "h2d_bytes_per_step": 1.0, "d2h_bytes_per_step": 2.0}
+    line = dict(keys, e2e=dict(e2e, note="n" * 3000), cpu_baseline={"value": 26.1, "unit": "MLUPS", "single": {"x": "y" * 2000}},
+                repeats={"blocks": 5, "block_ms": [1.0] * 5, "value_from": "z" * 500})
+    case = {"mlups": 1.0, "frac": 0.5, "adjoint_kernel_mlups": 3.0, "grad": [0.123456789] * 600, "rel_err_mean": 1e-4}
+    out = {k: {n: dict(case) for n in ("a", "b", "c", "d")} for k in
+           ("storage_variants", "adjoint", "cavity_les_f32", "cavity_sweep", "extensions_f32", "drag_error_vs_f64")}
+    path = tmp_path / "details.json"
+    bench.emit(line, out, str(path))
+    cap = capsys.readouterr()
+    assert cap.out.count("\n") == 1 and len(cap.out) < 4000
+    got = json.loads(cap.out)
+    assert all(got[k] == v for k, v in keys.items()) and got["e2e"] == e2e and got["cpu_baseline"]["value"] == 26.1
+    assert got["adjoint"]["b"] == {"adjoint_kernel_mlups": 3.0} and got["cavity_les_f32"]["a"] == {"mlups": 1.0, "frac": 0.5}
+    full = json.loads(path.read_text())
+    assert full == json.loads(cap.err.split("details: ", 1)[1]) and full["cavity_sweep"] == out["cavity_sweep"]
+    assert full["e2e"]["note"] == "n" * 3000
