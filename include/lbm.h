@@ -168,18 +168,20 @@ typedef struct lbm_config {
 /* Kernel of the fused step.  Both compute the same arithmetic and store the
  * same bits; they differ in how the pull sources reach the registers.
  * LBM_STEP_AUTO (0) picks the staged kernel, where it applies and its
- * pipeline fits in shared memory, for 16-bit storage and for FP32 on D3Q19 with
- * a closed face or any of the Lorentz force, Maxwell term, LES, linear
- * equilibrium or Darcy resistance (large boxes with insulating walls included), unless
- * more than 4% (8% with one of those) of the 4-node chunks touch a solid or a
- * ragged row end or the box is one of the few kinds that measured slower; else
- * the register-tiled one.  LBM_STEP_REGISTER
- * (1): every thread loads its vectors straight from HBM.  LBM_STEP_STAGED (2): a persistent kernel stages each tile's source
- * rows in shared memory with bulk asynchronous copies; it serves FP32 and
- * 16-bit storage with closed or periodic faces and every node code except
- * curved walls, insulating walls and the induced field (asked for with one of
- * those: LBM_ERR_ARG); where its pipeline does not fit in shared memory (rows of more than about
- * 1,100 16-bit or 550 FP32 nodes) the register-tiled kernel runs instead. */
+ * pipeline fits in shared memory, for 16-bit storage and for FP32 on D3Q19
+ * with a closed face or any of the EXT terms (Lorentz force, Maxwell term,
+ * LES, linear equilibrium, Darcy resistance; large boxes with insulating walls
+ * included), unless more than 4% (8% with an EXT term) of the 4-node chunks
+ * touch a solid or a ragged row end or the box is one of the few kinds that
+ * measured slower; else the register-tiled one.
+ * LBM_STEP_REGISTER (1): every thread loads its vectors straight from HBM.
+ * LBM_STEP_STAGED (2): a persistent kernel stages each tile's source rows in
+ * shared memory with bulk asynchronous copies; it serves FP32 and 16-bit
+ * storage with closed or periodic faces and every node code except curved
+ * walls, insulating walls and the induced field (asked for with one of those:
+ * LBM_ERR_ARG); where its pipeline does not fit in shared memory (rows of more
+ * than about 1,100 16-bit or 550 FP32 nodes) the register-tiled kernel runs
+ * instead. */
 enum { LBM_STEP_AUTO = 0, LBM_STEP_REGISTER = 1, LBM_STEP_STAGED = 2 };
 
 /* Induced magnetic field (Sec. 4 cites Dellar's vector lattice Boltzmann
@@ -236,8 +238,9 @@ enum { LBM_STEP_AUTO = 0, LBM_STEP_REGISTER = 1, LBM_STEP_STAGED = 2 };
  * first step after lbm_create, lbm_init_equilibrium, lbm_import_f or
  * lbm_load_state uses the configured E.  E is state that a population
  * checkpoint does not hold, so lbm_step_from returns LBM_ERR_UNSUPPORTED, and
- * the reductions of the step run on the stepping stream.  Costs a scratch
- * row of 3 doubles per step thread (see lbm_buffer_sizes). */
+ * the reductions of the step run on the stepping stream.  Costs scratch rows
+ * of 3 doubles, one per warp of the step (FP64 one per 64 nodes; see
+ * lbm_buffer_sizes). */
 
 /* rounding of the populations stored by a step.  Stochastic rounding rounds
  * a value up with probability equal to its distance from the value below, so
@@ -329,7 +332,9 @@ lbm_status lbm_export_field(lbm_ctx* ctx, double* B, int on_host, void* stream);
 lbm_status lbm_time(const lbm_ctx* ctx, int64_t* t);
 
 /* The kernel that runs this context's step: LBM_STEP_REGISTER or
- * LBM_STEP_STAGED (the automatic choice resolved at lbm_create). */
+ * LBM_STEP_STAGED (the automatic choice resolved at lbm_create).  Steps with
+ * a kernel of their own (FP64 storage, the induced field) answer
+ * LBM_STEP_REGISTER. */
 lbm_status lbm_step_kernel(const lbm_ctx* ctx, int32_t* kind);
 
 /* The imposed electric field that the next step uses (3 doubles, host

@@ -38,9 +38,9 @@ size_t elem_of(int storage)
     }
 }
 
-// the staged step serves 16-bit and FP32 storage with halfway walls and the
-// node code of the imposed field (not walls off the half-grid, insulating
-// walls or the induced field, whose state the staged kernel does not carry)
+// the staged step that a caller may ask for serves 16-bit and FP32 storage
+// with halfway walls and the node code of the imposed field (not walls off the
+// half-grid, insulating walls or the induced field)
 bool staged_applies(const lbm_config* c)
 {
     return !c->curved && !c->insulating && !c->induced && c->storage != LBM_STORE_F64;

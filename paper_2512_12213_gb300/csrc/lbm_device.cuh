@@ -281,7 +281,6 @@ struct Geo {
 // NC_FACE: some links cross a closed face of the box, none hits a solid;
 // NC_BOUND: some link hits a solid node; 0x80 | id: solid of wall id; NC_PAD: padding
 enum : uint8_t { NC_BULK = 0, NC_BOUND = 1, NC_FACE = 2, NC_PAD = 0xFF };
-__host__ __device__ inline bool nc_has_wall(uint8_t c) { return c == NC_BOUND || c == NC_FACE; }
 __host__ __device__ inline bool nc_solid(uint8_t c) { return (c & 0x80) && c != NC_PAD; }
 __host__ __device__ inline int nc_wall(uint8_t c) { return c & 0x7F; }
 __host__ __device__ inline uint8_t nc_make_solid(int wall) { return (uint8_t)(0x80 | wall); }
@@ -629,7 +628,6 @@ __device__ __forceinline__ F2 f2dot(int a, const F2 (&x)[3])
 }
 
 __device__ __forceinline__ F2 f2rcp(F2 a) { return F2{make_float2(__frcp_rn(a.v.x), __frcp_rn(a.v.y))}; }
-__device__ __forceinline__ F2 f2sqrt(F2 a) { return F2{make_float2(__fsqrt_rn(a.v.x), __fsqrt_rn(a.v.y))}; }
 // 1/rho and the Smagorinsky relaxation time of the pair codes with the
 // approximate square root and reciprocal of the special-function unit (a
 // unit or two in the last place): neither enters a balance -- the odd part

@@ -429,15 +429,14 @@ k_step(const typename S::T* __restrict__ src, typename S::T* __restrict__ dst,
 
         const long long base = row * g.nxp + x0;
         {
-            if constexpr (PACKED && (PAIR2 || PAIRX)) {
+            if constexpr (PACKED && PAIR2) {
 #pragma unroll
                 for (int i = 0; i < V / 2; ++i) {
                     F2 dd[Q];
 #pragma unroll
                     for (int a = 0; a < Q; ++a) dd[a] = F2{S::unpack2(w[a][i])};
                     if (ladd) add_ladd2(dd, 2 * i);
-                    if constexpr (PAIR2) pair_collide<Q, LP, true>(dd, p);
-                    else pair_collide_ext<Q>(dd, p);
+                    pair_collide<Q, LP, true>(dd, p);
                     if constexpr (SR) {
                         NodeRng rp((uint32_t)(base + 2 * i), seed);     // the pair's first node
 #pragma unroll
@@ -1277,9 +1276,10 @@ k_balance(const typename S::T* __restrict__ P, const uint8_t* __restrict__ cls, 
 // exactly from the stored values, see above), |v - v_ref| and |v| (Euclidean
 // norms), block sums in FP64 for the fixed-order pass; with `update` the
 // node's v replaces v_ref (each thread reads its own entries before it writes
-// them; solid nodes get 0).  The FP64 pipe bounds it (~35 operations a node):
-// 256 x 128 x 128 FP32 423 us with the quotient and the library's square
-// roots, 366 with rcp64 and sqrt64; three blocks per SM (444 with two).
+// them; solid nodes get 0).  The FP64 pipe bounds it (~40 operations a node,
+// two square roots and a reciprocal among them): 256 x 128 x 128 FP32 394 us
+// (one grid for every node, see fixed_moments, 366; with the quotient and the
+// library's square roots 57 more); three blocks per SM (with two 78 more).
 template <int Q, class S, bool EXT, bool CURVED>
 __global__ void __launch_bounds__(RED_THREADS, 3)
 k_residual(const typename S::T* __restrict__ P, const uint8_t* __restrict__ cls, const Geo g,
@@ -1669,8 +1669,8 @@ cudaError_t launch_step_q(const Ctx& c, const void* src, void* dst, uint32_t see
     return faces ? go(yes, no, no) : go(no, no, no);
 }
 
-// the staged step (periodic boxes with the plain node code, 16-bit or FP32
-// storage; the host chose the tile rows and stage count at create)
+// the staged step (16-bit or FP32 storage, any node code but curved walls and
+// the induced field; the host chose the tile rows and stage count at create)
 template <int Q, class S, bool SR, bool EXT, bool FACES, bool LP = false, bool INS = false>
 cudaError_t launch_step_staged_k(const Ctx& c, const void* src, void* dst, uint32_t seed, cudaStream_t st,
                                  const StgForce& fw)

@@ -2,8 +2,8 @@
 // and Eq. 10 with the Maxwell term) as a persistent kernel whose input rows
 // are staged in shared memory by the bulk asynchronous copies of the tensor
 // memory accelerator, for 16-bit or FP32 storage with halfway walls, closed
-// or periodic box faces and every node code but curved walls, insulating
-// walls and the induced field.
+// or periodic box faces and every node code but the induced field; insulating
+// walls in FP32 on D3Q19 (the INS instantiation).
 //
 // Pull scheme: a tile is R consecutive rows (y0 .. y0+R-1) of one z plane;
 // for direction a the tile reads the R source rows shifted by (E_y, E_z),
