@@ -761,7 +761,7 @@ __device__ __forceinline__ FF ff_split(double x, bool& ok)
 // and  w2 Z + 9/2 w2 (K_i + K_j +- 2 X) +- 3 w2 (J_i +- J_j); 9/2 w is a power
 // of two.  Rounded to FP32 at the end, as the FP64 values were: the stored values'
 // error against 64 bits is the rounding's, 2.7e-8, at deviations of 1e-2 to
-// 1e-8 alike.  256 x 128 x 128: 1,335 us in FP64 -> 185 us.  A value that lies within the two evaluations' errors of the
+// 1e-8 alike.  256 x 128 x 128: 1,335 us in FP64 -> 168 us.  A value that lies within the two evaluations' errors of the
 // middle of two FP32 numbers (about one of 1e5) takes the FP64 formula, so
 // that the rounding is that of the FP64 evaluation; not in a flow whose
 // deviations are below 1e-8, where the sums here are the more exact.  false (d
@@ -922,8 +922,8 @@ __device__ R unbounced(const Src& s, const KP<R>& p, const WRho& wr, const Geo& 
 
 // one padded node per thread.  Before (each node pulling its 18 neighbours'
 // values, with their equilibria in FP64) a 192^3 binary16 box took 12.2 ms
-// from fields and 1.04 ms from FP32 populations; so 0.455 ms and
-// 0.22 ms (0.53 of the copy bandwidth).
+// from fields and 1.04 ms from FP32 populations; so 0.44 ms and
+// 0.23 ms (0.53 of the copy bandwidth).
 template <int Q, class S, class Src, bool CURVED>
 __global__ void __launch_bounds__(NODE_THREADS, CURVED ? 1 : 4)
 k_inverse_stream(typename S::T* __restrict__ P, const uint8_t* __restrict__ cls, const Geo g,
