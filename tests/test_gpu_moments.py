@@ -115,3 +115,40 @@ def test_moments_of_full_mantissas(kind, box):
     for k in range(3):
         assert abs(momentum[k] - math.fsum(j[k].ravel())) <= 1e-13 * S.sum()
     sim.close()
+
+
+# the residual's FP64 reciprocal (third-order iteration from FP32: 2^-13 of a
+# unit in the last place before its rounding) and square root, one value at a
+# time: v = j / rho with j a power of two is the reciprocal itself, and the sum
+# over one node of |v| the root of v v; densities beyond FP32's range take the
+# plain quotient and root
+@pytest.mark.parametrize("exponent", [0, 60, -60, 125, -125, 300, -300])
+def test_reciprocal_and_root_are_rounded(exponent):
+    from fractions import Fraction
+    unit = 2.0 ** exponent
+    g = np.random.default_rng(7)
+    nx, ny = 64, 8
+    cfg = dict(lattice=9, ny=ny, nz=1, tau=0.8, rho0=unit, force_model="e", storage="f64")
+    sim = lbm.Sim(dict(cfg, nx=nx), inputs.empty_mask(nx, ny, 1), stage=False)
+    P = np.zeros((9, ny, nx))
+    P[0] = (np.exp2(g.uniform(-5, 5, (ny, nx))) * g.uniform(1, 2, (ny, nx)) - 1.0) * unit
+    P[1], P[3] = unit / 16, -unit / 16                       # j = (unit / 8, 0), no density
+    lbm.lbm_load_state(sim.ctx, torch.from_numpy(P).cuda().view(torch.uint8), 1, sim.stream)
+    v_ref = torch.zeros((3, 1, ny, nx), dtype=torch.float64, device="cuda")
+    sim.residual(v_ref)
+    v, rho = v_ref[0, 0].cpu().numpy(), P[0] + unit
+    ulp = Fraction(1, 2) + Fraction(1, 2 ** 12)
+    for got, r in zip(v.ravel(), rho.ravel()):
+        assert abs(Fraction(got) - Fraction(unit) / 8 / Fraction(r)) <= ulp * Fraction(np.spacing(got))
+    sim.close()
+    sim = lbm.Sim(dict(cfg, nx=1, ny=1), inputs.empty_mask(1, 1, 1), stage=False)
+    one = torch.zeros(sim.sizes[lbm.BUF_POP_A], dtype=torch.uint8, device="cuda")
+    row = one.view(torch.float64)[:9 * 64].view(9, 64)
+    v_ref = torch.zeros((3, 1, 1, 1), dtype=torch.float64, device="cuda")
+    for d0, speed in list(zip(P[0].ravel(), v.ravel()))[:60]:
+        row[0, 0], row[1, 0], row[3, 0] = d0, unit / 16, -unit / 16
+        lbm.lbm_load_state(sim.ctx, one, 1, sim.stream)
+        _, total, _ = sim.residual(v_ref, update=False)
+        vv, err = speed * speed, ulp * Fraction(np.spacing(total))
+        assert (Fraction(total) - err) ** 2 <= Fraction(vv) <= (Fraction(total) + err) ** 2
+    sim.close()
